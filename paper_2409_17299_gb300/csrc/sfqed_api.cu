@@ -12,7 +12,7 @@ static void free_ctx(qed_ctx *c) {
     sfq_batch_free(c);
     sfq_level_graphs_free(c);
     sfq_step_graph_free(c);
-    void *dev[] = {c->coef64, c->coef32, c->icdf_em64, c->icdf_pair64, c->icdf_em32, c->icdf_pair32, c->gl,
+    void *dev[] = {c->coef64, c->coef32, c->icdf_em64, c->icdf_pair64, c->icdf_em32, c->icdf_pair32,
                    c->ctl, c->tau[0], c->tau[1], c->tau[2], c->blk, c->slots, c->snap, c->lev,
                    c->mlp_p, c->mlp_w16, c->mlp_loss};
     for (void *p : dev)
@@ -52,7 +52,6 @@ extern "C" qed_status qed_init_tables(qed_ctx **out, const qed_config *cfg, void
               cudaMalloc(&c->icdf_pair64, sizeof(double) * PAIR_NCHI * PAIR_NS) == cudaSuccess &&
               cudaMalloc(&c->icdf_em32, sizeof(float) * EM_NCHI * EM_NS) == cudaSuccess &&
               cudaMalloc(&c->icdf_pair32, sizeof(float) * PAIR_NCHI * PAIR_NS) == cudaSuccess &&
-              cudaMalloc(&c->gl, sizeof(double) * 64) == cudaSuccess &&
               cudaMalloc(&c->ctl, sizeof(DevCtl)) == cudaSuccess &&
               cudaMalloc(&c->lev, sizeof(LevelWork)) == cudaSuccess &&
               cudaHostAlloc(&c->ctl_host, sizeof(DevCtl), cudaHostAllocDefault) == cudaSuccess &&

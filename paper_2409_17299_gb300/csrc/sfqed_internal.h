@@ -169,7 +169,6 @@ struct qed_ctx {
     float *coef32;
     double *icdf_em64, *icdf_pair64;
     float *icdf_em32, *icdf_pair32;
-    double *gl;              // Gauss-Legendre nodes and weights (work)
     // control
     sfq::DevCtl *ctl;
     sfq::DevCtl *ctl_host;   // pinned mirror (read back at the end of a batch of steps)
