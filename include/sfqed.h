@@ -92,9 +92,10 @@ typedef struct {
                                  choice, else 4 */
     int event_method;         /* QED_METHOD_SUBSTEP (Algorithm 1, default) or
                                  QED_METHOD_OPTICAL_DEPTH (see below) */
-    int pass_limit;           /* newborn passes (Algorithm 2 sweeps) a step may run; a
-                                 step that needs more stops there and the call returns
-                                 QED_ERR_TIMEOUT; 0 = 100000 */
+    int pass_limit;           /* generations of newborns (Algorithm 2: a particle born in a
+                                 step, one born of it in the same step, ...) a step may
+                                 run; a step that needs more stops there and the call
+                                 returns QED_ERR_TIMEOUT; 0 = 100000 */
     int wait_polls;           /* polls of each grid barrier inside qed_train_surrogate
                                  before the launch gives up (QED_ERR_TIMEOUT); 0 = 2^24 */
     int reserved[1];
@@ -141,7 +142,7 @@ typedef struct {
     int64_t needed_capacity[3];
     int64_t max_subevents;    /* largest number of events of one particle in one step */
     int64_t overflow;         /* 1 if a species ran out of capacity */
-    int64_t passes;           /* newborn passes run (Algorithm 2 sweeps) */
+    int64_t passes;           /* generations of newborns, summed over the steps (Algorithm 2) */
     int64_t thinned;          /* particles removed by leveling */
     int64_t lepton_steps;     /* particle-steps done by the lepton kernel */
     int64_t photon_steps;     /* particle-steps done by the photon kernel */
@@ -197,8 +198,8 @@ qed_status qed_push_and_generate(qed_ctx *ctx, qed_particles *p, const qed_field
  * (the steps run in call order with the indices given).
  *
  * Each step runs as one CUDA graph launch (Sec. 3, Algorithms 1-2): the
- * step-start passes, a device-side loop over newborn passes (bounded by
- * 100000 passes per step, QED_ERR_TIMEOUT beyond), and per species the merge
+ * photon and the lepton pass with everything born in the step (bounded by
+ * 100000 generations, QED_ERR_TIMEOUT beyond), and per species the merge
  * step -- leveling when the count exceeds thin_cap, converted photons removed
  * -- decided by the device.  The host never waits inside a batch.  With
  * cfg.profile (per-kernel events) or without conditional graph nodes, the

@@ -321,6 +321,24 @@ __device__ __forceinline__ double chi_fp64(double e0, double px, double py, doub
 // S + 2 e0 sum|E_i (p x B)_i|, exceeds four times S + T the cancellation is
 // real and the direct form is evaluated in FP64 instead.  Returns chi.
 // ---------------------------------------------------------------------------
+// a^2 + b^2 + c^2.  FIXED: every operation rounded explicitly, the middle
+// product on its own.  Without it the compiler decides which product it
+// fuses, and that depends on the code around the inlined copy.
+template <bool FIXED> __device__ __forceinline__ float sum_sq(float a, float b, float c) {
+    if constexpr (FIXED) return __fmaf_rn(c, c, __fmaf_rn(a, a, __fmul_rn(b, b)));
+    else return a * a + b * b + c * c;
+}
+template <bool FIXED> __device__ __forceinline__ double sum_sq(double a, double b, double c) {
+    if constexpr (FIXED) return __fma_rn(c, c, __fma_rn(a, a, __dmul_rn(b, b)));
+    else return a * a + b * b + c * c;
+}
+
+template <bool FIXED>
+__device__ __forceinline__ float sum_sq6(float a, float b, float c, float d, float e, float f) {
+    if constexpr (FIXED) return __fmaf_rn(f, f, __fmaf_rn(e, e, __fmaf_rn(d, d, sum_sq<true>(a, b, c))));
+    else return a * a + b * b + c * c + d * d + e * e + f * f;
+}
+
 __device__ __forceinline__ float diff_of_products(float a, float b, float c, float d) {
     // a*b - c*d
     const float w = c * d;
@@ -333,7 +351,7 @@ __device__ __forceinline__ float diff_of_products(float a, float b, float c, flo
 // squares), 2 if E = 0 everywhere (chi^2 R^2 = |p x B|^2), 3 if E and B are
 // parallel everywhere (T = 2 e0 E.(p x B) = 2 e0 p.(B x E) = 0, so
 // chi^2 R^2 = S, again a sum of squares), else 0.
-template <bool LEPTON>
+template <bool LEPTON, bool FIXED = false>
 __device__ __forceinline__ float chi_guarded(float e0, const float p[3], const float E[3], const float B[3],
                                              unsigned *fp64_used, int zero = 0) {
     if (zero == 3) {
@@ -343,23 +361,23 @@ __device__ __forceinline__ float chi_guarded(float e0, const float p[3], const f
         const float bx = diff_of_products(p[1], B[2], p[2], B[1]);
         const float by = diff_of_products(p[2], B[0], p[0], B[2]);
         const float bz = diff_of_products(p[0], B[1], p[1], B[0]);
-        float S = ax * ax + ay * ay + az * az + bx * bx + by * by + bz * bz;
-        if (LEPTON) S += E[0] * E[0] + E[1] * E[1] + E[2] * E[2];
+        float S = sum_sq6<FIXED>(ax, ay, az, bx, by, bz);
+        if (LEPTON) S += sum_sq<FIXED>(E[0], E[1], E[2]);
         return f_sqrt(S) * (float)(1.0 / RS);
     }
     if (zero == 1) {
         const float ax = diff_of_products(p[1], E[2], p[2], E[1]);
         const float ay = diff_of_products(p[2], E[0], p[0], E[2]);
         const float az = diff_of_products(p[0], E[1], p[1], E[0]);
-        float S = ax * ax + ay * ay + az * az;
-        if (LEPTON) S += E[0] * E[0] + E[1] * E[1] + E[2] * E[2];
+        float S = sum_sq<FIXED>(ax, ay, az);
+        if (LEPTON) S += sum_sq<FIXED>(E[0], E[1], E[2]);
         return f_sqrt(S) * (float)(1.0 / RS);
     }
     if (zero == 2) {
         const float bx = diff_of_products(p[1], B[2], p[2], B[1]);
         const float by = diff_of_products(p[2], B[0], p[0], B[2]);
         const float bz = diff_of_products(p[0], B[1], p[1], B[0]);
-        return f_sqrt(bx * bx + by * by + bz * bz) * (float)(1.0 / RS);
+        return f_sqrt(sum_sq<FIXED>(bx, by, bz)) * (float)(1.0 / RS);
     }
     const float ax = diff_of_products(p[1], E[2], p[2], E[1]);
     const float ay = diff_of_products(p[2], E[0], p[0], E[2]);
@@ -367,8 +385,8 @@ __device__ __forceinline__ float chi_guarded(float e0, const float p[3], const f
     const float bx = diff_of_products(p[1], B[2], p[2], B[1]);
     const float by = diff_of_products(p[2], B[0], p[0], B[2]);
     const float bz = diff_of_products(p[0], B[1], p[1], B[0]);
-    float S = ax * ax + ay * ay + az * az + bx * bx + by * by + bz * bz;
-    if (LEPTON) S += E[0] * E[0] + E[1] * E[1] + E[2] * E[2];
+    float S = sum_sq6<FIXED>(ax, ay, az, bx, by, bz);
+    if (LEPTON) S += sum_sq<FIXED>(E[0], E[1], E[2]);
     const float te = 2.0f * e0;
     const float T = te * (E[0] * bx + E[1] * by + E[2] * bz);
     const float M = S + te * (fabsf(E[0] * bx) + fabsf(E[1] * by) + fabsf(E[2] * bz));
@@ -381,24 +399,24 @@ __device__ __forceinline__ float chi_guarded(float e0, const float p[3], const f
 }
 
 // chi of a lepton (also gamma and p^2) or a photon in the mode's precision
-template <class T>
+template <class T, bool FIXED = false>
 __device__ __forceinline__ void lepton_chi(const T p[3], const T E[3], const T B[3], T &gam, T &chi, T &p2,
                                            unsigned &n64, int zero = 0) {
     if constexpr (sizeof(T) == 8) {
-        p2 = p[0] * p[0] + p[1] * p[1] + p[2] * p[2];
+        p2 = sum_sq<FIXED>(p[0], p[1], p[2]);
         gam = sqrt(1.0 + p2);
         chi = chi_fp64(gam, p[0], p[1], p[2], E[0], E[1], E[2], B[0], B[1], B[2]);
     } else {
-        p2 = p[0] * p[0] + p[1] * p[1] + p[2] * p[2];
+        p2 = sum_sq<FIXED>(p[0], p[1], p[2]);
         gam = f_sqrt(1.0f + p2);
-        chi = chi_guarded<true>(gam, p, E, B, &n64, zero);
+        chi = chi_guarded<true, FIXED>(gam, p, E, B, &n64, zero);
     }
 }
 
-template <class T>
+template <class T, bool FIXED = false>
 __device__ __forceinline__ T photon_chi(T k0, const T k[3], const T E[3], const T B[3], unsigned &n64, int zero = 0) {
     if constexpr (sizeof(T) == 8) return chi_fp64(k0, k[0], k[1], k[2], E[0], E[1], E[2], B[0], B[1], B[2]);
-    else return chi_guarded<false>(k0, k, E, B, &n64, zero);
+    else return chi_guarded<false, FIXED>(k0, k, E, B, &n64, zero);
 }
 
 // ---------------------------------------------------------------------------

@@ -46,8 +46,8 @@ struct DevCtl {
     unsigned long long max_subevents;
     unsigned long long overflow;
     unsigned long long needed[3];
-    unsigned long long more;            // the last pass setup found work
-    unsigned long long passes;
+    unsigned long long more;            // the last lepton pass left newborns behind
+    unsigned long long passes;          // generations of newborns, summed over the steps
     unsigned long long thinned;
     unsigned long long alive[3];        // compaction: alive entries per species
     unsigned long long holes[3];        // compaction: dead entries below alive[s]
@@ -55,15 +55,17 @@ struct DevCtl {
     unsigned long long chi_fp64;        // FP32 mode: chi evaluations that fell back to FP64
     unsigned long long graph_kernels;   // kernels run inside graphs (their launches are on the device)
     unsigned long long step_next;       // index of the step the next step-begin kernel opens
-    unsigned long long step_passes;     // newborn passes of the current step
+    unsigned long long step_passes;     // generations of newborns in the current step
     unsigned long long timeout;         // a bounded device-side loop gave up (QED_ERR_TIMEOUT)
     double sv_t_n;                      // current step: t_n = step * dt
     float sv_t_red_f;                   // current step: (t_n mod 2 pi) rounded to float
     unsigned sv_step;                   // current step index (Philox counter word 2)
     unsigned long long deferred[3];     // dead entries left in place by the last merge step
     unsigned long long moved;           // compaction: entries moved into holes
-    unsigned long long pass_limit;      // newborn passes a step may run (then timeout)
-    unsigned long long pad[4];
+    unsigned long long pass_limit;      // generations of newborns a step may run (then timeout)
+    unsigned long long born[2];         // leptons after the photon pass (its pairs lie behind the step-start range)
+    unsigned long long arrive;          // blocks of the running pass kernel that have finished
+    unsigned long long spilled;         // newborn leptons left behind by the lepton pass
 };
 static_assert(sizeof(DevCtl) == 384, "control block layout");
 
@@ -126,7 +128,7 @@ struct SpeciesDev {
     void *x, *y, *z, *px, *py, *pz, *w;
     unsigned long long *id;
     unsigned *nev;
-    double *tau;            // birth clock of newborns (context work buffer)
+    double *tau;            // birth clock of newborn leptons (context work buffer)
     void *od;               // remaining optical depth (QED_METHOD_OPTICAL_DEPTH, T), or null
 };
 
@@ -154,7 +156,7 @@ struct PassArgs {
     PhiloxKeys keys;        // round keys of seed (event draws)
     int pass;               // 0: particles present at the step start (tau = 0)
     int soft_filter;
-    int record_newborn_tau; // newborns get their birth clock stored (cascades)
+    int fly_newborns;       // newborns are pushed to the end of their birth step (cascades)
 };
 
 }  // namespace sfq
@@ -174,8 +176,8 @@ struct qed_ctx {
     sfq::DevCtl *ctl_host;   // pinned mirror (read back at the end of a batch of steps)
     sfq::DevCtl *ctl_up;     // pinned staging of the upload when a batch of steps opens
     // newborn birth clocks
-    double *tau[3];
-    int64_t tau_cap[3];
+    double *tau[2];
+    int64_t tau_cap[2];
     // compaction / leveling work buffers
     unsigned long long *blk;      // per-block counts
     int64_t blk_cap;
@@ -205,7 +207,6 @@ struct qed_ctx {
     size_t grid_il_bytes;
     int tuned_threads;           // block shape picked by the autotuner (0: none yet)
     int tuned_budget;            // step budget picked by the autotuner (0: none yet)
-    int spec_passes;             // newborn passes enqueued per host check (from the last step)
     int lev_chunk[3];            // leveling passes enqueued per host check (from the last leveling)
     // steps enqueued without waiting (qed_push_async) until qed_push_wait:
     // the device control block holds the counts meanwhile
@@ -318,11 +319,13 @@ qed_status sfq_drain_events(qed_ctx *ctx);
 // pass launchers, one per field variant (sfqed_pass_analytic.cu, sfqed_pass_grid.cu)
 namespace sfq {
 namespace pass_analytic {
-template <class T> qed_status launch_pass(qed_ctx *ctx, PassArgs &a, bool photons);
+template <class T>
+qed_status launch_pass(qed_ctx *ctx, PassArgs &a, bool photons, cudaGraphConditionalHandle h, int loop);
 template <class T> qed_status launch_od(qed_ctx *ctx, PassArgs &a, bool photons);
 }
 namespace pass_grid {
-template <class T> qed_status launch_pass(qed_ctx *ctx, PassArgs &a, bool photons);
+template <class T>
+qed_status launch_pass(qed_ctx *ctx, PassArgs &a, bool photons, cudaGraphConditionalHandle h, int loop);
 template <class T> qed_status launch_od(qed_ctx *ctx, PassArgs &a, bool photons);
 }
 }  // namespace sfq

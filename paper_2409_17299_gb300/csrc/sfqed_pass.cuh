@@ -7,9 +7,24 @@
 // One pass kernel per particle kind.  Each thread takes one particle of the
 // pass range (grid-stride), runs Algorithm 1 for it to the end of the step
 // (rate -> waiting time -> Boris push -> event), and appends every particle
-// it creates with a warp-aggregated atomic.  Newborns carry their birth
-// clock and are pushed by the next pass (Algorithm 2): leptons and photons
-// are swept alternately until a pass creates nothing.
+// it creates with a warp-aggregated atomic.
+//
+// Algorithm 2 (newborns are pushed to the end of their birth step) takes no
+// sweeps of its own: draws are keyed by id, so the order in which newborns
+// are pushed does not matter.  The photon pass runs first; the pairs it
+// creates carry their birth clock and are taken up by the lepton pass behind
+// the step-start leptons.  In the lepton pass a new photon flies to the step
+// end at once, in the thread that emitted it (the field at the emission point
+// is at hand, and the photon's record is written once, at its final place),
+// and the leptons of a pair it creates go to the block's queue.  Sweeping the
+// newborns in passes of their own took 3 to 5 further passes over each
+// species per step, each two or three launches and a read and a write of
+// every newborn (standing-wave cascade, 1e7 particles per species: 0.26 of
+// 1.9 ms per step; at 5e5 photons 44 of 145 us).  20 steps at the start of a
+// cascade (1e5 leptons) 3.36 -> 2.86 ms, 40 steps with the network sampler at
+// 1e7 photons 34.3 -> 30.0 ms, with the table at 5e7 88.8 -> 87.0 ms, of the
+// standing wave at 1e7 per species 89.6 -> 88.2 ms.  Only when a block's queue
+// is full do newborn leptons wait for a further launch of the lepton pass.
 #pragma once
 
 #include <math.h>
@@ -73,24 +88,54 @@ template <class T> __device__ __forceinline__ T t_inf();
 template <> __device__ __forceinline__ double t_inf<double>() { return __longlong_as_double(0x7ff0000000000000ll); }
 template <> __device__ __forceinline__ float t_inf<float>() { return __int_as_float(0x7f800000); }
 
-__device__ __forceinline__ void flush_stats(DevCtl *ctl, unsigned long long steps, unsigned long long ev,
-                                            unsigned mx, bool pair, unsigned n64) {
+// Statistics of one thread: particles pushed and events of each kind.
+struct PassStats {
+    unsigned long long lep = 0, ph = 0, em = 0, pr = 0;
+    unsigned mx = 0, n64 = 0, gen = 0;
+};
+
+__device__ __forceinline__ void flush_stats(DevCtl *ctl, PassStats s) {
     // called by every lane of the warp after the grid-stride loop
     for (int o = 16; o > 0; o >>= 1) {
-        steps += __shfl_down_sync(0xffffffffu, steps, o);
-        ev += __shfl_down_sync(0xffffffffu, ev, o);
-        mx = max(mx, __shfl_down_sync(0xffffffffu, mx, o));
-        n64 += __shfl_down_sync(0xffffffffu, n64, o);
+        s.lep += __shfl_down_sync(0xffffffffu, s.lep, o);
+        s.ph += __shfl_down_sync(0xffffffffu, s.ph, o);
+        s.em += __shfl_down_sync(0xffffffffu, s.em, o);
+        s.pr += __shfl_down_sync(0xffffffffu, s.pr, o);
+        s.mx = max(s.mx, __shfl_down_sync(0xffffffffu, s.mx, o));
+        s.n64 += __shfl_down_sync(0xffffffffu, s.n64, o);
+        s.gen = max(s.gen, __shfl_down_sync(0xffffffffu, s.gen, o));
     }
     if ((threadIdx.x & 31) == 0) {
-        if (n64) atomicAdd(&ctl->chi_fp64, (unsigned long long)n64);
-        if (steps) {
-            atomicAdd(&ctl->particle_steps, steps);
-            atomicAdd(pair ? &ctl->photon_steps : &ctl->lepton_steps, steps);
-        }
-        if (ev) atomicAdd(pair ? &ctl->pair_events : &ctl->emit_events, ev);
-        if (mx) atomicMax(&ctl->max_subevents, (unsigned long long)mx);
+        if (s.n64) atomicAdd(&ctl->chi_fp64, (unsigned long long)s.n64);
+        if (s.lep + s.ph) atomicAdd(&ctl->particle_steps, s.lep + s.ph);
+        if (s.lep) atomicAdd(&ctl->lepton_steps, s.lep);
+        if (s.ph) atomicAdd(&ctl->photon_steps, s.ph);
+        if (s.em) atomicAdd(&ctl->emit_events, s.em);
+        if (s.pr) atomicAdd(&ctl->pair_events, s.pr);
+        if (s.mx) atomicMax(&ctl->max_subevents, (unsigned long long)s.mx);
+        if (s.gen) atomicMax(&ctl->step_passes, (unsigned long long)s.gen);
     }
+}
+
+// True in every thread of the block that finishes last in its launch; what
+// the other blocks wrote is then visible.  Called once per block, by all its
+// threads.
+__device__ __forceinline__ bool last_block(DevCtl *ctl) {
+    __shared__ int s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_last = atomicAdd(&ctl->arrive, 1ull) == gridDim.x - 1;
+        if (s_last) ctl->arrive = 0;
+        __threadfence();
+    }
+    __syncthreads();
+    return s_last != 0;
+}
+
+__device__ __forceinline__ unsigned long long count_now(DevCtl *ctl, int s) {
+    const unsigned long long c = __ldcg(&ctl->count[s]);
+    return c < ctl->capacity[s] ? c : ctl->capacity[s];
 }
 
 // chi and energy of a lepton / photon in the mode's precision: FP64 mode uses
@@ -103,25 +148,48 @@ __device__ __forceinline__ void note_overflow(DevCtl *ctl, int s, unsigned long 
 // Algorithm 1 for electrons and positrons (both species of one pass).
 //
 // Divergence control (the GPU form of Algorithm 3's "sort handled particles
-// to the front"): phase 1 pushes every particle of a 256-particle tile to its
-// first event or to the end of the step; particles at an event go to a
-// per-block stack in shared memory.  Whenever the stack holds a full round,
+// to the front"): phase 1 pushes every particle of a tile (one per thread) to
+// its first event or to the end of the step; particles at an event go to
+// a per-block stack in shared memory.  Whenever the stack holds a full round,
 // the block pops one item per thread and processes it densely: the event
-// (chi at the point, energy draw, recoil, photon append), then the next
+// (chi at the point, energy draw, recoil, the photon's flight), then the next
 // waiting time, ending either at the step end (state stored) or at the next
-// event (pushed back).  The stack is drained after the last tile.
-constexpr int LB = 256;            // threads per block of the lepton pass
-constexpr int LQ = 2 * LB;         // stack capacity: < LB left + LB pushed
+// event (pushed back).  The stack is drained after the last tile.  Newborn
+// leptons enter the stack at their birth clock, without an event pending.
+//
+// Threads per block of the lepton pass: 256 in FP32, three blocks per SM (four
+// would spill the photon's flight: 2.5% slower at 5e7 photons).  In FP64 128:
+// the pass is bound by the FP64 pipe, which a few warps keep busy, and
+// smaller blocks spread a small ensemble over more SMs (16384 electrons, one
+// step: 87 us at 256 threads, 79 us at 128).
+template <class T> constexpr int LB = sizeof(T) == 4 ? 256 : 128;
+constexpr unsigned RESUME = 0x80000000u;   // stack item flag: no event pending (a newborn at its birth clock)
 
 template <class T> struct LeptonStack {
-    T x[3][LQ], p[3][LQ];
-    double tau[LQ];
-    unsigned long long id[LQ];
-    T w[LQ];
-    unsigned idx[LQ];              // index | species << 31
-    unsigned k[LQ];                // events so far in this step (the pending one not counted)
-    uint2 r[LQ];                   // the pending event's energy draw words
-    int n;
+    static constexpr int Q = 2 * LB<T>;    // items: < LB left + LB pushed
+    T x[3][Q], p[3][Q];
+    double tau[Q];
+    unsigned long long id[Q];
+    T w[Q];
+    unsigned idx[Q];               // index | species << 31
+    unsigned k[Q];                 // events so far in this step (the pending one not counted)
+    unsigned gen[Q];               // generation within the step (0: present at its start) | RESUME
+    uint2 r[Q];                    // the pending event's energy draw words
+    // newborn leptons of this block's photons, not on the stack yet (their
+    // state is in the species arrays)
+    unsigned nb_idx[LB<T>], nb_gen[LB<T>];
+    // items pushed in iteration i of the block's loop are counted in
+    // pushed[i mod 3]: the stack's size is then a uniform register value, no
+    // thread reads a counter that another may already be adding to, and the
+    // counter of iteration i + 1 is cleared in iteration i
+    int pushed[3], nb_pushed[3];
+};
+
+// the block's view of its stack in one iteration
+struct StackPos {
+    int n;        // stack items below this iteration's pushes
+    int nb;       // waiting newborns
+    int it;       // iteration mod 3
 };
 
 template <class T> struct LeptonCtx {
@@ -130,6 +198,7 @@ template <class T> struct LeptonCtx {
     const T *coef;
     const T *icdf;
     unsigned long long cap_ph;
+    unsigned gen_limit;     // generations a step may run (then it is marked as timed out)
     T alpha_r;
     const StepTime &tm;     // the step's time and index (block's shared copy)
     Phase<T> ph0;           // time phase at the step start (tau = 0)
@@ -158,7 +227,9 @@ __device__ __forceinline__ bool advance(const LeptonCtx<T> &c, T x[3], T p[3], T
     if constexpr (FRESH) field_at<T>(a, x, c.ph0, E, B);
     else field_tau<T>(a, c.tm, x, tau, E, B);
     T gam, chi, p2;
-    lepton_chi<T>(p, E, B, gam, chi, p2, n64, a.field_zero);
+    // after an event the copy of this code depends on what surrounds it: its
+    // sums are rounded explicitly
+    lepton_chi<T, !FRESH>(p, E, B, gam, chi, p2, n64, a.field_zero);
     const T lam = p2 > (T)0 ? f_div(c.alpha_r, gam) * rate_em<T>(c.coef, chi) : (T)0;
     T dth = t_inf<T>();
     if (lam > lam_skip<T>(a)) {
@@ -197,268 +268,46 @@ __device__ __forceinline__ bool advance(const LeptonCtx<T> &c, T x[3], T p[3], T
 }
 
 // Kinematics of an emission with photon fraction delta (and 1 - delta) from a
-// lepton of energy gam and momentum p at x: collinear, energy-conserving
-// recoil; the photon is appended.
+// lepton of energy gam and momentum p: collinear, energy-conserving recoil.
+// Returns whether the photon is kept, its momentum in kv.
 template <class T>
-__device__ __forceinline__ void emit_with(const LeptonCtx<T> &c, const T x[3], T p[3], double tau, T w,
-                                          unsigned long long id, unsigned k, T gam, T p2, T delta, T om) {
-    const PassArgs &a = c.a;
+__device__ __forceinline__ bool recoil(const PassArgs &a, T p[3], T gam, T p2, T delta, T om, T kv[3]) {
     T g_after = om * gam, k0 = delta * gam;
     if (g_after < (T)1) { g_after = (T)1; k0 = gam - (T)1; }
     const T inv = f_rsqrt(p2);
     const T nx = p[0] * inv, ny = p[1] * inv, nz = p[2] * inv;
     const T pa = f_sqrt((g_after - (T)1) * (g_after + (T)1));
-    if (!(a.soft_filter && k0 < (T)2)) {
-        const uint4 rid = event_draw(a.seed ^ CHILD_KEY_XOR, id, c.tm.step, k);
-        const unsigned long long slot = warp_append(&c.ctl->count[2], 1);
-        if (slot < c.cap_ph) {
-            const SpeciesDev &P = a.sp[2];
-            st<T>(P.x, slot, x[0]); st<T>(P.y, slot, x[1]); st<T>(P.z, slot, x[2]);
-            st<T>(P.px, slot, k0 * nx); st<T>(P.py, slot, k0 * ny); st<T>(P.pz, slot, k0 * nz);
-            st<T>(P.w, slot, w);
-            P.id[slot] = (unsigned long long)rid.x | ((unsigned long long)rid.y << 32);
-            P.nev[slot] = 0u;
-            if (a.record_newborn_tau) P.tau[slot] = tau;
-            if (P.od) st<T>(P.od, slot, (T)0);       // optical depth not drawn yet
-        } else {
-            note_overflow(c.ctl, 2, slot);
-        }
-    }
+    kv[0] = k0 * nx; kv[1] = k0 * ny; kv[2] = k0 * nz;
     p[0] = pa * nx; p[1] = pa * ny; p[2] = pa * nz;
-}
-
-// The event at the particle's current point with the table sampler: chi
-// there, energy fraction from the inverse CDF, then the kinematics.
-template <class T>
-__device__ __forceinline__ void emit(const LeptonCtx<T> &c, const T x[3], T p[3], double tau, T w,
-                                     unsigned long long id, unsigned k, uint2 rz, unsigned &n64) {
-    T E[3], B[3];
-    field_tau<T>(c.a, c.tm, x, tau, E, B);
-    T gam, chi, p2;
-    lepton_chi<T>(p, E, B, gam, chi, p2, n64, c.a.field_zero);
-    T om, ue, ve;
-    Uniform<T>::draw(rz.x, rz.y, ue, ve);
-    const T delta = sample_emission<T>(c.icdf, chi, ue, ve, &om);
-    emit_with<T>(c, x, p, tau, w, id, k, gam, p2, delta, om);
-}
-
-// Network sampler of a block: the staged network (dynamic shared memory)
-constexpr int MLP_SMEM_BYTES = MLP_INF_BYTES;
-
-template <class T>
-__device__ __forceinline__ void finish(const PassArgs &a, unsigned idx, const T x[3], const T p[3], unsigned k) {
-    const SpeciesDev &S = a.sp[idx >> 31];
-    const unsigned i = idx & 0x7FFFFFFFu;
-    st<T>(S.x, i, x[0]); st<T>(S.y, i, x[1]); st<T>(S.z, i, x[2]);
-    st<T>(S.px, i, p[0]); st<T>(S.py, i, p[1]); st<T>(S.pz, i, p[2]);
-    if (k) S.nev[i] += k;
+    return !(a.soft_filter && k0 < (T)2);
 }
 
 template <class T>
-__device__ __forceinline__ void stack_push(LeptonStack<T> &q, const T x[3], const T p[3], double tau,
-                                           unsigned long long id, T w, unsigned idx, unsigned k, uint2 rz) {
-    const int slot = atomicAdd(&q.n, 1);
-    q.x[0][slot] = x[0]; q.x[1][slot] = x[1]; q.x[2][slot] = x[2];
-    q.p[0][slot] = p[0]; q.p[1][slot] = p[1]; q.p[2][slot] = p[2];
-    q.tau[slot] = tau; q.id[slot] = id; q.w[slot] = w; q.idx[slot] = idx; q.k[slot] = k; q.r[slot] = rz;
-}
-
-// Pop min(n, LB) items, one per thread, and process each to its next event
-// or the step end.  Every thread of the block calls this.
-template <class T, bool MLP>
-__device__ __forceinline__ void stack_round(const LeptonCtx<T> &c, LeptonStack<T> &q, unsigned long long &ev,
-                                            unsigned &mx, unsigned &n64, const MlpInf &ms) {
-    const int n = q.n;
-    const int take = n < LB ? n : LB;
-    const int t = threadIdx.x;
-    T x[3], p[3], w = 0;
-    double tau = 0.0;
-    unsigned long long id = 0;
-    unsigned idx = 0, k = 0;
-    uint2 rz = make_uint2(0, 0);
-    const bool mine = t < take;
-    if (mine) {
-        const int s = n - take + t;
-        x[0] = q.x[0][s]; x[1] = q.x[1][s]; x[2] = q.x[2][s];
-        p[0] = q.p[0][s]; p[1] = q.p[1][s]; p[2] = q.p[2][s];
-        tau = q.tau[s]; id = q.id[s]; w = q.w[s]; idx = q.idx[s]; k = q.k[s]; rz = q.r[s];
-    }
-    __syncthreads();
-    if (t == 0) q.n = n - take;
-    __syncthreads();
-    if constexpr (MLP) {
-        // event-point state per item, then the whole warp evaluates the
-        // network for its 32 items on the tensor cores
-        T gam = (T)1, chi = (T)0, p2 = (T)0, ue = (T)0.5, ve = (T)0.5;
-        float f0 = 0.f, f1 = 0.f;
-        bool use_net = false;
-        if (mine) {
-            T E[3], B[3];
-            field_tau<T>(c.a, c.tm, x, tau, E, B);
-            lepton_chi<T>(p, E, B, gam, chi, p2, n64, c.a.field_zero);
-            Uniform<T>::draw(rz.x, rz.y, ue, ve);
-            const float sl = (float)logit(ue, ve);
-            const float cf = (float)chi;
-            use_net = cf >= 1e-3f && cf <= 1e3f && fabsf(sl) < 16.0f;
-            if (use_net) { f0 = log10f(cf) / 3.0f; f1 = sl / 16.0f; }
-        }
-        const float y = mlp_forward_warp(f0, f1, ms);
-        if (mine) {
-            T delta, om;
-            if (use_net) {
-                const T aa = (T)3 * chi * (T)__expf(16.0f * (y - 0.5f));
-                om = (T)2 / ((T)2 + aa);
-                delta = aa / ((T)2 + aa);
-            } else {
-                delta = sample_emission<T>(c.icdf, chi, ue, ve, &om);
-            }
-            emit_with<T>(c, x, p, tau, w, id, k, gam, p2, delta, om);
-        }
+__device__ __forceinline__ void append_photon(const PassArgs &a, DevCtl *ctl, unsigned long long cap, const T x[3],
+                                              const T kv[3], T w, uint4 rid) {
+    const unsigned long long slot = warp_append(&ctl->count[2], 1);
+    if (slot < cap) {
+        const SpeciesDev &P = a.sp[2];
+        st<T>(P.x, slot, x[0]); st<T>(P.y, slot, x[1]); st<T>(P.z, slot, x[2]);
+        st<T>(P.px, slot, kv[0]); st<T>(P.py, slot, kv[1]); st<T>(P.pz, slot, kv[2]);
+        st<T>(P.w, slot, w);
+        P.id[slot] = (unsigned long long)rid.x | ((unsigned long long)rid.y << 32);
+        P.nev[slot] = 0u;
+        if (P.od) st<T>(P.od, slot, (T)0);       // optical depth not drawn yet
     } else {
-        if (mine) emit<T>(c, x, p, tau, w, id, k, rz, n64);
+        note_overflow(ctl, 2, slot);
     }
-    if (mine) {
-        ++k;
-        ++ev;
-        const T qch = (idx >> 31) ? (T)1 : (T)-1;
-        if (before_step_end(tau, c.a.dt) && advance<T, false>(c, x, p, qch, tau, id, k, rz, n64)) {
-            stack_push<T>(q, x, p, tau, id, w, idx, k, rz);
-        } else {
-            finish<T>(c.a, idx, x, p, k);
-            mx = max(mx, k);
-        }
-    }
-    __syncthreads();
-}
-
-template <class T, bool FRESH, bool MLP>
-__global__ void __launch_bounds__(LB, (sizeof(T) == 4 ? (MLP ? 2 : 4) : 1)) k_lepton_pass(PassArgs a) {
-    // blocks past the pass's range leave before staging anything (a newborn
-    // pass is often far smaller than the resident grid)
-    if ((unsigned long long)blockIdx.x * LB >= (a.ctl->end[0] - a.ctl->begin[0]) + (a.ctl->end[1] - a.ctl->begin[1]))
-        return;
-    __shared__ __align__(16) T s_coef[RateWords<T>::N];
-    __shared__ LeptonStack<T> q;
-    __shared__ StepTime s_tm;
-    extern __shared__ __align__(16) unsigned char dyn[];
-    MlpInf ms{nullptr, nullptr, nullptr};
-    if constexpr (MLP) ms = mlp_stage(dyn, a.mlp_w16);
-    for (int i = threadIdx.x; i < RateWords<T>::N; i += blockDim.x) s_coef[i] = reinterpret_cast<const T *>(a.coef)[i];
-    if (threadIdx.x == 0) {
-        q.n = 0;
-        s_tm = load_step_time(a);
-    }
-    __syncthreads();
-    DevCtl *ctl = a.ctl;
-    // 32-bit indices (a species holds fewer than 2^31 entries: bit 31 of idx names the species)
-    const unsigned b0 = (unsigned)ctl->begin[0], n0 = (unsigned)(ctl->end[0] - ctl->begin[0]);
-    const unsigned b1 = (unsigned)ctl->begin[1], n1 = (unsigned)(ctl->end[1] - ctl->begin[1]);
-    const unsigned n = n0 + n1;
-    const LeptonCtx<T> c{a, ctl, s_coef, reinterpret_cast<const T *>(a.icdf_em), ctl->capacity[2], (T)(ALPHA * RS),
-                         s_tm, time_phase<T, StepTime>(s_tm, 0.0)};
-    unsigned long long my_steps = 0, my_ev = 0;
-    unsigned my_max = 0, n64 = 0;
-
-    // FP32 step-start pass: each thread stages its particle of the block's
-    // next tile in shared memory while the block works on the current tile
-    constexpr bool STAGE = FRESH && sizeof(T) == 4;
-    constexpr int NF = STAGE ? 9 : 1, NT = STAGE ? LB : 1;
-    __shared__ __align__(16) float stg[NF][NT];            // w x y z px py pz id(2 words)
-    const unsigned stride = gridDim.x * LB;
-    auto stage = [&](unsigned jj) {
-        if constexpr (STAGE) {
-            const int sp = jj < n0 ? 0 : 1;
-            const unsigned ii = sp == 0 ? b0 + jj : b1 + (jj - n0);
-            const SpeciesDev &P = a.sp[sp];
-            const int t = threadIdx.x;
-            cp_async4(&stg[0][t], reinterpret_cast<const float *>(P.w) + ii);
-            cp_async4(&stg[1][t], reinterpret_cast<const float *>(P.x) + ii);
-            cp_async4(&stg[2][t], reinterpret_cast<const float *>(P.y) + ii);
-            cp_async4(&stg[3][t], reinterpret_cast<const float *>(P.z) + ii);
-            cp_async4(&stg[4][t], reinterpret_cast<const float *>(P.px) + ii);
-            cp_async4(&stg[5][t], reinterpret_cast<const float *>(P.py) + ii);
-            cp_async4(&stg[6][t], reinterpret_cast<const float *>(P.pz) + ii);
-            cp_async4(&stg[7][t], P.id + ii);
-            cp_async4(&stg[8][t], reinterpret_cast<const unsigned *>(P.id + ii) + 1);
-        }
-    };
-    if constexpr (STAGE) {
-        const unsigned j0 = blockIdx.x * LB + threadIdx.x;
-        if (j0 < n) stage(j0);
-        cp_async_commit();
-    }
-
-    // One loop with one call of stack_round: the next tile is taken while the
-    // stack holds less than a round, the stack is drained at the end.  The
-    // round (and the event arithmetic in it) then has a single inlined copy,
-    // so which round processes a particle, which depends on the order of the
-    // arrays, cannot change how its results are rounded.
-    unsigned base = blockIdx.x * LB;
-    for (;;) {
-        if (base < n && q.n < LB) {
-            const unsigned j = base + threadIdx.x;
-            T w = (T)0, x[3], p[3];
-            unsigned long long id = 0;
-            if constexpr (STAGE) {
-                // this thread's staged particle, then the next tile's copies in
-                // flight (the slots are free once read)
-                cp_async_wait_all();
-                if (j < n) {
-                    const int t = threadIdx.x;
-                    w = stg[0][t];
-                    x[0] = stg[1][t]; x[1] = stg[2][t]; x[2] = stg[3][t];
-                    p[0] = stg[4][t]; p[1] = stg[5][t]; p[2] = stg[6][t];
-                    id = (unsigned long long)__float_as_uint(stg[7][t]) |
-                         ((unsigned long long)__float_as_uint(stg[8][t]) << 32);
-                }
-                if (j + stride < n) stage(j + stride);
-                cp_async_commit();
-            }
-            if (j < n) {
-                const int s = j < n0 ? 0 : 1;
-                const unsigned i = s == 0 ? b0 + j : b1 + (j - n0);
-                const SpeciesDev &S = a.sp[s];
-                if constexpr (!STAGE) {
-                    w = ld<T>(S.w, i);
-                    x[0] = ld<T>(S.x, i); x[1] = ld<T>(S.y, i); x[2] = ld<T>(S.z, i);
-                    p[0] = ld<T>(S.px, i); p[1] = ld<T>(S.py, i); p[2] = ld<T>(S.pz, i);
-                    id = __ldg(S.id + i);
-                }
-                if (w > (T)0) {
-                    double tau = FRESH ? 0.0 : S.tau[i];
-                    const unsigned idx = i | ((unsigned)s << 31);
-                    ++my_steps;
-                    uint2 rz = make_uint2(0, 0);
-                    const T qch = s == 0 ? (T)-1 : (T)1;
-                    bool event;
-                    if constexpr (FRESH) event = advance<T, true>(c, x, p, qch, tau, id, 0u, rz, n64);
-                    else event = before_step_end(tau, a.dt) && advance<T, false>(c, x, p, qch, tau, id, 0u, rz, n64);
-                    if (event) {
-                        stack_push<T>(q, x, p, tau, id, w, idx, 0u, rz);
-                    } else {
-                        finish<T>(a, idx, x, p, 0u);
-                    }
-                }
-            }
-            base += stride;
-            __syncthreads();
-            continue;
-        }
-        if (q.n == 0) break;
-        stack_round<T, MLP>(c, q, my_ev, my_max, n64, ms);
-    }
-    __syncwarp();
-    flush_stats(ctl, my_steps, my_ev, my_max, false, n64);
 }
 
 // Pair creation at a photon's event point x at clock tau (Sec. 3): chi there,
 // electron fraction from the inverse CDF with the draw words rz, both leptons
 // along the photon's direction with energy-conserving momenta, appended with
-// their ids and birth clock.  The caller removes the photon.
-template <class T>
+// their ids.  born(species, slot) is called for each lepton that got a place.
+// The caller removes the photon.
+template <class T, class F>
 __device__ __forceinline__ void pair_create(const PassArgs &a, const StepTime &tm, const T *icdf, const T x[3],
                                             const T kv[3], T k0, T nx, T ny, T nz, double tau, T w,
-                                            unsigned long long id, unsigned k, uint2 rz, unsigned &n64) {
+                                            unsigned long long id, unsigned k, uint2 rz, unsigned &n64, F born) {
     DevCtl *ctl = a.ctl;
     T E[3], B[3];
     field_tau<T>(a, tm, x, tau, E, B);
@@ -482,6 +331,7 @@ __device__ __forceinline__ void pair_create(const PassArgs &a, const StepTime &t
         P.nev[se] = 0u;
         P.tau[se] = tau;
         if (P.od) st<T>(P.od, se, (T)0);
+        born(0, (unsigned)se);
     } else {
         note_overflow(ctl, 0, se);
     }
@@ -494,152 +344,484 @@ __device__ __forceinline__ void pair_create(const PassArgs &a, const StepTime &t
         P.nev[sp] = 0u;
         P.tau[sp] = tau;
         if (P.od) st<T>(P.od, sp, (T)0);
+        born(1, (unsigned)sp);
     } else {
         note_overflow(ctl, 1, sp);
     }
 }
 
-// One photon of a pass from its loaded state (index i, weight w, position x,
-// momentum k, id): straight flight, pair creation at the event (the photon
-// is removed: weight 0 and its event count stored here).  Returns false for
-// a dead photon (weight 0: nothing to do and nothing to store); otherwise x
-// holds the new position, which the caller stores, and k the events.
+// A copy of v that the compiler does not see through.  Sub-expressions shared
+// with other code may be fused into multiply-adds differently than alone; a
+// photon's flight from such copies is rounded as in a kernel of its own, and
+// does not change how the surrounding lepton arithmetic is rounded.
+__device__ __forceinline__ float own(float v) { asm volatile("" : "+f"(v)); return v; }
+__device__ __forceinline__ double own(double v) { asm volatile("" : "+d"(v)); return v; }
+
+// One waiting time of a photon of energy k0 and direction n at x, where the
+// field is (E, B), at clock tau (FRESH: the step start, tau = 0): the photon
+// flies to the step end (returns false) or to the point where it converts
+// (returns true: tau there, the pair's draw words in rz).
 template <class T, bool FRESH>
-__device__ __forceinline__ bool photon_step(const PassArgs &a, const StepTime &tm, const T *s_coef, const T *icdf,
-                                            const Phase<T> &ph0, const SpeciesDev &S, unsigned i, T w, T x[3],
-                                            T kx, T ky, T kz, unsigned long long id, unsigned &k, unsigned &n64) {
-    k = 0;
-    if (!(w > (T)0)) return false;
+__device__ __forceinline__ bool photon_flight(const PassArgs &a, const StepTime &tm, const T *s_coef, const T E[3],
+                                              const T B[3], T x[3], const T kv[3], T k0, T inv, T nx, T ny, T nz,
+                                              double &tau, unsigned long long id, uint2 &rz, unsigned &n64) {
     const T alpha_r = (T)(ALPHA * RS);
-    double tau = FRESH ? 0.0 : S.tau[i];
-    const T kv[3] = {kx, ky, kz};
-    const T k0 = f_sqrt(kx * kx + ky * ky + kz * kz);
-    if (k0 > (T)0) {
-        const T inv = f_div((T)1, k0);
-        const T nx = kx * inv, ny = ky * inv, nz = kz * inv;
-        // one waiting time: the photon either reaches the step end or converts
-        if (FRESH || before_step_end(tau, a.dt)) {
-            T E[3], B[3];
-            if constexpr (FRESH) field_at<T>(a, x, ph0, E, B);
-            else field_tau<T>(a, tm, x, tau, E, B);
-            T chi = photon_chi<T>(k0, kv, E, B, n64, a.field_zero);
-            T lam;
-            if constexpr (sizeof(T) == 4) lam = alpha_r * inv * rate_pair<T>(s_coef, chi);
-            else lam = alpha_r / k0 * rate_pair<T>(s_coef, chi);     // the oracle's rounding
-            uint4 r = make_uint4(0, 0, 0, 0);
-            T dth = t_inf<T>();
-            if (lam > lam_skip<T>(a)) {
-                r = event_draw(a.keys, id, tm.step, k);
-                T uw, vw;
-                Uniform<T>::draw(r.x, r.y, uw, vw);
-                dth = f_div(Uniform<T>::neglog(uw, vw), lam);
-            }
-            bool no_event;
-            T h;
-            if constexpr (FRESH && sizeof(T) == 4) { no_event = dth >= a.dt_f_gt; h = a.dt_f; }
-            else if constexpr (FRESH) { no_event = dth > a.dt; h = a.dt; }
-            else if constexpr (sizeof(T) == 4) {
-                // as in the lepton pass: the FP64 test decided in FP32 outside a margin
-                const float rf = __double2float_rn(a.dt - tau);
-                const float marg = fmaf(rf, 0x1p-20f, a.dt_f * 0x1p-40f);
-                if (dth > rf + marg) no_event = true;
-                else if (dth < rf - marg) no_event = false;
-                else no_event = tau + (double)dth > a.dt;
-                h = rf;
-            } else { no_event = tau + (double)dth > a.dt; h = (T)(a.dt - tau); }
-            if (no_event) {
-                x[0] += nx * h; x[1] += ny * h; x[2] += nz * h;
-            } else {
-                x[0] += nx * dth; x[1] += ny * dth; x[2] += nz * dth;
-                if constexpr (FRESH) tau = (double)dth;
-                else tau += (double)dth;
-                pair_create<T>(a, tm, icdf, x, kv, k0, nx, ny, nz, tau, w, id, k, make_uint2(r.z, r.w), n64);
-                k = 1;
-                st<T>(S.w, i, (T)0);       // the photon is eliminated
-                S.nev[i] += k;
-            }
-        }
+    T chi = photon_chi<T, !FRESH>(k0, kv, E, B, n64, a.field_zero);
+    T lam;
+    if constexpr (sizeof(T) == 4) lam = alpha_r * inv * rate_pair<T>(s_coef, chi);
+    else lam = alpha_r / k0 * rate_pair<T>(s_coef, chi);     // the oracle's rounding
+    uint4 r = make_uint4(0, 0, 0, 0);
+    T dth = t_inf<T>();
+    if (lam > lam_skip<T>(a)) {
+        r = event_draw(a.keys, id, tm.step, 0u);
+        T uw, vw;
+        Uniform<T>::draw(r.x, r.y, uw, vw);
+        dth = f_div(Uniform<T>::neglog(uw, vw), lam);
     }
+    bool no_event;
+    T h;
+    if constexpr (FRESH && sizeof(T) == 4) { no_event = dth >= a.dt_f_gt; h = a.dt_f; }
+    else if constexpr (FRESH) { no_event = dth > a.dt; h = a.dt; }
+    else if constexpr (sizeof(T) == 4) {
+        // as in the lepton pass: the FP64 test decided in FP32 outside a margin
+        const float rf = __double2float_rn(a.dt - tau);
+        const float marg = fmaf(rf, 0x1p-20f, a.dt_f * 0x1p-40f);
+        if (dth > rf + marg) no_event = true;
+        else if (dth < rf - marg) no_event = false;
+        else no_event = tau + (double)dth > a.dt;
+        h = rf;
+    } else { no_event = tau + (double)dth > a.dt; h = (T)(a.dt - tau); }
+    if (no_event) {
+        x[0] += nx * h; x[1] += ny * h; x[2] += nz * h;
+        return false;
+    }
+    x[0] += nx * dth; x[1] += ny * dth; x[2] += nz * dth;
+    if constexpr (FRESH) tau = (double)dth;
+    else tau += (double)dth;
+    rz = make_uint2(r.z, r.w);
     return true;
 }
 
+// A photon emitted in this step (momentum kv, field (E, B) at its birth point
+// x, generation gen): its flight to the step end, then its record; or the
+// pair it creates, whose leptons wait in the block's newborn list, or, when
+// that is full, in the species arrays for a further launch.
+template <class T>
+__device__ __forceinline__ void fly_newborn(const LeptonCtx<T> &c, LeptonStack<T> &q, const StackPos &pos,
+                                            const T Ee[3], const T Be[3], const T xe[3], const T ke[3], double tau,
+                                            T w, uint4 rid, unsigned gen, PassStats &ps) {
+    const PassArgs &a = c.a;
+    const unsigned long long id = (unsigned long long)rid.x | ((unsigned long long)rid.y << 32);
+    T x[3] = {own(xe[0]), own(xe[1]), own(xe[2])};
+    const T E[3] = {own(Ee[0]), own(Ee[1]), own(Ee[2])}, B[3] = {own(Be[0]), own(Be[1]), own(Be[2])};
+    const T kv[3] = {own(ke[0]), own(ke[1]), own(ke[2])};
+    const T k0 = f_sqrt(kv[0] * kv[0] + kv[1] * kv[1] + kv[2] * kv[2]);
+    bool alive = true;
+    ++ps.ph;
+    ps.gen = max(ps.gen, gen);
+    if (gen > c.gen_limit) atomicExch(&c.ctl->timeout, 1ull);
+    else if (k0 > (T)0 && before_step_end(tau, a.dt)) {
+        const T inv = f_div((T)1, k0);
+        const T nx = kv[0] * inv, ny = kv[1] * inv, nz = kv[2] * inv;
+        uint2 rz = make_uint2(0, 0);
+        if (photon_flight<T, false>(a, c.tm, c.coef, E, B, x, kv, k0, inv, nx, ny, nz, tau, id, rz, ps.n64)) {
+            alive = false;
+            ++ps.pr;
+            ps.mx = max(ps.mx, 1u);
+            pair_create<T>(a, c.tm, reinterpret_cast<const T *>(a.icdf_pair), x, kv, k0, nx, ny, nz, tau, w, id, 0u, rz,
+                           ps.n64, [&](int s, unsigned i) {
+                const int at = pos.nb + atomicAdd(&q.nb_pushed[pos.it], 1);
+                if (at < LB<T>) {
+                    q.nb_idx[at] = i | ((unsigned)s << 31);
+                    q.nb_gen[at] = gen + 1u;
+                } else {
+                    // left at its birth clock for a further launch; the sign
+                    // bit marks it (those taken up here stay unmarked)
+                    a.sp[s].tau[i] = -tau;
+                    atomicAdd(&c.ctl->spilled, 1ull);
+                }
+            });
+        }
+    }
+    if (alive) append_photon<T>(a, c.ctl, c.cap_ph, x, kv, w, rid);
+}
+
+// Network sampler of a block: the staged network (dynamic shared memory)
+constexpr int MLP_SMEM_BYTES = MLP_INF_BYTES;
+
+template <class T>
+__device__ __forceinline__ void finish(const PassArgs &a, unsigned idx, const T x[3], const T p[3], unsigned k) {
+    const SpeciesDev &S = a.sp[idx >> 31];
+    const unsigned i = idx & 0x7FFFFFFFu;
+    st<T>(S.x, i, x[0]); st<T>(S.y, i, x[1]); st<T>(S.z, i, x[2]);
+    st<T>(S.px, i, p[0]); st<T>(S.py, i, p[1]); st<T>(S.pz, i, p[2]);
+    if (k) S.nev[i] += k;
+}
+
+template <class T>
+__device__ __forceinline__ void stack_push(LeptonStack<T> &q, const StackPos &pos, const T x[3], const T p[3],
+                                           double tau, unsigned long long id, T w, unsigned idx, unsigned k,
+                                           unsigned gen, uint2 rz) {
+    const int slot = pos.n + atomicAdd(&q.pushed[pos.it], 1);
+    q.x[0][slot] = x[0]; q.x[1][slot] = x[1]; q.x[2][slot] = x[2];
+    q.p[0][slot] = p[0]; q.p[1][slot] = p[1]; q.p[2][slot] = p[2];
+    q.tau[slot] = tau; q.id[slot] = id; q.w[slot] = w; q.idx[slot] = idx; q.k[slot] = k; q.gen[slot] = gen;
+    q.r[slot] = rz;
+}
+
+// Pop min(n, LB) items, one per thread, and process each to its next event
+// or the step end.  Every thread of the block calls this; pos.n is the
+// stack's size and becomes the size below the round's pushes.
+template <class T, bool MLP>
+__device__ __forceinline__ void stack_round(const LeptonCtx<T> &c, LeptonStack<T> &q, StackPos &pos, PassStats &ps,
+                                            const MlpInf &ms) {
+    const int take = pos.n < LB<T> ? pos.n : LB<T>;
+    const int t = threadIdx.x;
+    T x[3], p[3], w = 0;
+    double tau = 0.0;
+    unsigned long long id = 0;
+    unsigned idx = 0, k = 0, gen = RESUME;
+    uint2 rz = make_uint2(0, 0);
+    const bool mine = t < take;
+    pos.n -= take;
+    if (mine) {
+        const int s = pos.n + t;
+        x[0] = q.x[0][s]; x[1] = q.x[1][s]; x[2] = q.x[2][s];
+        p[0] = q.p[0][s]; p[1] = q.p[1][s]; p[2] = q.p[2][s];
+        tau = q.tau[s]; id = q.id[s]; w = q.w[s]; idx = q.idx[s]; k = q.k[s]; gen = q.gen[s]; rz = q.r[s];
+    }
+    __syncthreads();                                // the popped places may now be pushed to
+    const bool event = !(gen & RESUME);
+    gen &= ~RESUME;
+    // the event at the particle's current point: chi there, energy fraction
+    // from the inverse CDF (or the network: the whole warp evaluates it for
+    // its 32 items on the tensor cores), then the kinematics
+    T E[3], B[3], gam = (T)1, chi = (T)0, p2 = (T)0, ue = (T)0.5, ve = (T)0.5, delta = (T)0, om = (T)1;
+    if (event) {
+        field_tau<T>(c.a, c.tm, x, tau, E, B);
+        lepton_chi<T>(p, E, B, gam, chi, p2, ps.n64, c.a.field_zero);
+        Uniform<T>::draw(rz.x, rz.y, ue, ve);
+    }
+    if constexpr (MLP) {
+        float f0 = 0.f, f1 = 0.f;
+        bool use_net = false;
+        if (event) {
+            const float sl = (float)logit(ue, ve);
+            const float cf = (float)chi;
+            use_net = cf >= 1e-3f && cf <= 1e3f && fabsf(sl) < 16.0f;
+            if (use_net) { f0 = log10f(cf) / 3.0f; f1 = sl / 16.0f; }
+        }
+        const float y = mlp_forward_warp(f0, f1, ms);
+        if (event) {
+            if (use_net) {
+                const T aa = (T)3 * chi * (T)__expf(16.0f * (y - 0.5f));
+                om = (T)2 / ((T)2 + aa);
+                delta = aa / ((T)2 + aa);
+            } else {
+                delta = sample_emission<T>(c.icdf, chi, ue, ve, &om);
+            }
+        }
+    } else {
+        if (event) delta = sample_emission<T>(c.icdf, chi, ue, ve, &om);
+    }
+    if (event) {
+        T kv[3];
+        if (recoil<T>(c.a, p, gam, p2, delta, om, kv)) {
+            const uint4 rid = event_draw(c.a.seed ^ CHILD_KEY_XOR, id, c.tm.step, k);
+            if (c.a.fly_newborns) fly_newborn<T>(c, q, pos, E, B, x, kv, tau, w, rid, gen + 1u, ps);
+            else append_photon<T>(c.a, c.ctl, c.cap_ph, x, kv, w, rid);
+        }
+        ++k;
+        ++ps.em;
+    }
+    if (mine) {
+        const T qch = (idx >> 31) ? (T)1 : (T)-1;
+        if (before_step_end(tau, c.a.dt) && advance<T, false>(c, x, p, qch, tau, id, k, rz, ps.n64)) {
+            stack_push<T>(q, pos, x, p, tau, id, w, idx, k, gen, rz);
+        } else {
+            finish<T>(c.a, idx, x, p, k);
+            ps.mx = max(ps.mx, k);
+        }
+    }
+}
+
+// One step's leptons.  FRESH: those present at the step start, then the
+// newborns of the photon pass; else the newborns that a full block list left
+// behind in the previous launch.  The last block to finish opens the next
+// such launch (`loop`: through the step graph's while node `h`).
+template <class T, bool FRESH, bool MLP>
+__global__ void __launch_bounds__(LB<T>, (sizeof(T) == 4 && !MLP ? 3 : 2))
+    k_lepton_pass(const __grid_constant__ PassArgs a, cudaGraphConditionalHandle h, int loop) {
+    DevCtl *ctl = a.ctl;
+    // 32-bit indices (a species holds fewer than 2^31 entries: bit 31 of idx names the species)
+    const unsigned n0 = FRESH ? (unsigned)ctl->end[0] : 0u, n1 = FRESH ? (unsigned)ctl->end[1] : 0u;
+    const unsigned n = n0 + n1;
+    const unsigned nb0 = (unsigned)(FRESH ? ctl->end[0] : ctl->begin[0]);
+    const unsigned nb1 = (unsigned)(FRESH ? ctl->end[1] : ctl->begin[1]);
+    const unsigned m0 = (unsigned)(FRESH ? ctl->born[0] : ctl->end[0]) - nb0;
+    const unsigned m = m0 + (unsigned)(FRESH ? ctl->born[1] : ctl->end[1]) - nb1;
+    const unsigned nb_blk = gridDim.x - 1 - blockIdx.x;      // newborn tiles from the far end: few steps have many
+    constexpr int NT = LB<T>;
+    __shared__ __align__(16) T s_coef[RateWords<T>::N];
+    __shared__ LeptonStack<T> q;
+    __shared__ StepTime s_tm;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    PassStats ps;
+    // blocks past the pass's ranges stage nothing
+    if (blockIdx.x * NT < n || nb_blk * NT < m) {
+        MlpInf ms{nullptr, nullptr, nullptr};
+        if constexpr (MLP) ms = mlp_stage(dyn, a.mlp_w16);
+        for (int i = threadIdx.x; i < RateWords<T>::N; i += NT) s_coef[i] = reinterpret_cast<const T *>(a.coef)[i];
+        if (threadIdx.x < 3) q.pushed[threadIdx.x] = q.nb_pushed[threadIdx.x] = 0;
+        if (threadIdx.x == 0) s_tm = load_step_time(a);
+        __syncthreads();
+        const unsigned gen_limit = (unsigned)ctl->pass_limit;
+        const unsigned gen0 = FRESH ? 1u : (unsigned)ctl->step_passes + 1u;   // generation of the newborns waiting
+        const LeptonCtx<T> c{a, ctl, s_coef, reinterpret_cast<const T *>(a.icdf_em), ctl->capacity[2], gen_limit,
+                             (T)(ALPHA * RS), s_tm, time_phase<T, StepTime>(s_tm, 0.0)};
+        // FP32 step-start pass: each thread stages its particle of the block's
+        // next tile in shared memory while the block works on the current tile
+        constexpr bool STAGE = FRESH && sizeof(T) == 4;
+        constexpr int NF = STAGE ? 9 : 1, NS = STAGE ? NT : 1;
+        __shared__ __align__(16) float stg[NF][NS];            // w x y z px py pz id(2 words)
+        const unsigned stride = gridDim.x * NT;
+        auto stage = [&](unsigned jj) {
+            if constexpr (STAGE) {
+                const int sp = jj < n0 ? 0 : 1;
+                const unsigned ii = sp == 0 ? jj : jj - n0;
+                const SpeciesDev &P = a.sp[sp];
+                const int t = threadIdx.x;
+                cp_async4(&stg[0][t], reinterpret_cast<const float *>(P.w) + ii);
+                cp_async4(&stg[1][t], reinterpret_cast<const float *>(P.x) + ii);
+                cp_async4(&stg[2][t], reinterpret_cast<const float *>(P.y) + ii);
+                cp_async4(&stg[3][t], reinterpret_cast<const float *>(P.z) + ii);
+                cp_async4(&stg[4][t], reinterpret_cast<const float *>(P.px) + ii);
+                cp_async4(&stg[5][t], reinterpret_cast<const float *>(P.py) + ii);
+                cp_async4(&stg[6][t], reinterpret_cast<const float *>(P.pz) + ii);
+                cp_async4(&stg[7][t], P.id + ii);
+                cp_async4(&stg[8][t], reinterpret_cast<const unsigned *>(P.id + ii) + 1);
+            }
+        };
+        unsigned base = blockIdx.x * NT, nb_base = nb_blk * NT;
+        if constexpr (STAGE) {
+            if (base + threadIdx.x < n) stage(base + threadIdx.x);
+            cp_async_commit();
+        }
+
+        // One loop with one call of stack_round: the next tile is taken while the
+        // stack holds less than a round, the stack is drained at the end.  The
+        // round (and the event arithmetic in it) then has a single inlined copy,
+        // so which round processes a particle, which depends on the order of the
+        // arrays, cannot change how its results are rounded.
+        StackPos pos{0, 0, 0};
+        for (;;) {
+            const bool fresh = base < n && pos.nb < NT / 2;
+            if (pos.n < NT && fresh) {
+                const unsigned j = base + threadIdx.x;
+                T w = (T)0, x[3], p[3];
+                unsigned long long id = 0;
+                if constexpr (STAGE) {
+                    // this thread's staged particle, then the next tile's copies in
+                    // flight (the slots are free once read)
+                    cp_async_wait_all();
+                    if (j < n) {
+                        const int t = threadIdx.x;
+                        w = stg[0][t];
+                        x[0] = stg[1][t]; x[1] = stg[2][t]; x[2] = stg[3][t];
+                        p[0] = stg[4][t]; p[1] = stg[5][t]; p[2] = stg[6][t];
+                        id = (unsigned long long)__float_as_uint(stg[7][t]) |
+                             ((unsigned long long)__float_as_uint(stg[8][t]) << 32);
+                    }
+                    if (j + stride < n) stage(j + stride);
+                    cp_async_commit();
+                }
+                if (j < n) {
+                    const int s = j < n0 ? 0 : 1;
+                    const unsigned i = s == 0 ? j : j - n0;
+                    const SpeciesDev &S = a.sp[s];
+                    if constexpr (!STAGE) {
+                        w = ld<T>(S.w, i);
+                        x[0] = ld<T>(S.x, i); x[1] = ld<T>(S.y, i); x[2] = ld<T>(S.z, i);
+                        p[0] = ld<T>(S.px, i); p[1] = ld<T>(S.py, i); p[2] = ld<T>(S.pz, i);
+                        id = __ldg(S.id + i);
+                    }
+                    if (w > (T)0) {
+                        double tau = 0.0;
+                        const unsigned idx = i | ((unsigned)s << 31);
+                        ++ps.lep;
+                        uint2 rz = make_uint2(0, 0);
+                        const T qch = s == 0 ? (T)-1 : (T)1;
+                        if (advance<T, true>(c, x, p, qch, tau, id, 0u, rz, ps.n64)) {
+                            stack_push<T>(q, pos, x, p, tau, id, w, idx, 0u, 0u, rz);
+                        } else {
+                            finish<T>(a, idx, x, p, 0u);
+                        }
+                    }
+                }
+                base += stride;
+            } else if (pos.n < NT && (pos.nb > 0 || nb_base < m)) {
+                // newborn leptons onto the stack: this block's own first, else a
+                // tile of those waiting in the species arrays
+                const bool own = pos.nb > 0;
+                const unsigned t = threadIdx.x;
+                unsigned idx = 0, gen = gen0;
+                bool have = false;
+                if (own) {
+                    have = t < (unsigned)pos.nb;
+                    if (have) { idx = q.nb_idx[t]; gen = q.nb_gen[t]; }
+                } else {
+                    const unsigned j = nb_base + t;
+                    have = j < m;
+                    if (have) idx = j < m0 ? nb0 + j : (nb1 + (j - m0)) | 0x80000000u;
+                    nb_base += stride;
+                }
+                if (have) {
+                    const SpeciesDev &S = a.sp[idx >> 31];
+                    const unsigned i = idx & 0x7FFFFFFFu;
+                    double tau = S.tau[i];
+                    const T w = ld<T>(S.w, i);
+                    if constexpr (!FRESH) {
+                        // among those appended since, only the ones left behind carry the mark
+                        if (!own) {
+                            have = __double_as_longlong(tau) < 0;
+                            tau = -tau;
+                        }
+                    }
+                    if (have && gen > gen_limit) {
+                        atomicExch(&ctl->timeout, 1ull);
+                        have = false;
+                    }
+                    if (have && w > (T)0) {
+                        ++ps.lep;
+                        ps.gen = max(ps.gen, gen);
+                        const T x[3] = {ld<T>(S.x, i), ld<T>(S.y, i), ld<T>(S.z, i)};
+                        const T p[3] = {ld<T>(S.px, i), ld<T>(S.py, i), ld<T>(S.pz, i)};
+                        stack_push<T>(q, pos, x, p, tau, S.id[i], w, idx, 0u, gen | RESUME, make_uint2(0, 0));
+                    }
+                }
+                if (own) pos.nb = 0;
+            } else {
+                if (pos.n == 0) break;
+                stack_round<T, MLP>(c, q, pos, ps, ms);
+            }
+            // the sizes after this iteration's pushes; the next iteration's
+            // counters were last read an iteration ago
+            const int nx = pos.it == 2 ? 0 : pos.it + 1;
+            if (threadIdx.x == 0) q.pushed[nx] = q.nb_pushed[nx] = 0;
+            __syncthreads();
+            pos.n += q.pushed[pos.it];
+            pos.nb = min(pos.nb + q.nb_pushed[pos.it], NT);
+            pos.it = nx;
+        }
+        __syncwarp();
+        flush_stats(ctl, ps);
+    }
+    if (!a.fly_newborns) return;
+    if (last_block(ctl) && threadIdx.x == 0) {
+        const bool more = __ldcg(&ctl->spilled) != 0 && !__ldcg(&ctl->overflow) && !__ldcg(&ctl->timeout);
+        for (int s = 0; s < 2; ++s) {
+            ctl->begin[s] = FRESH ? ctl->born[s] : ctl->end[s];
+            ctl->end[s] = count_now(ctl, s);
+        }
+        ctl->more = more;
+        if (!more) ctl->passes += __ldcg(&ctl->step_passes);
+        ctl->spilled = 0;
+        if (!FRESH && loop) ctl->graph_kernels += 1;
+        if (loop) cudaGraphSetConditional(h, more ? 1u : 0u);
+    }
+}
+
 // Photon push: straight flight, pair creation at the event, the photon is
-// removed (weight 0) and the pair appended.
-template <class T, bool FRESH>
+// removed (weight 0) and the pair appended, its leptons left to the lepton
+// pass of the same step (the last block to finish closes their range).
+template <class T>
 __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_photon_pass(PassArgs a) {
-    if ((unsigned long long)blockIdx.x * blockDim.x >= a.ctl->end[2] - a.ctl->begin[2]) return;   // no photon here
+    DevCtl *ctl = a.ctl;
+    constexpr int NT = 256;
+    // 32-bit indices (a species holds fewer than 2^31 entries)
+    const unsigned n = (unsigned)ctl->end[2];
     __shared__ __align__(16) T s_coef[RateWords<T>::N];
     __shared__ StepTime s_tm;
-    for (int i = threadIdx.x; i < RateWords<T>::N; i += blockDim.x) s_coef[i] = reinterpret_cast<const T *>(a.coef)[i];
-    if (threadIdx.x == 0) s_tm = load_step_time(a);
-    __syncthreads();
-    const StepTime &tm = s_tm;
-    DevCtl *ctl = a.ctl;
-    // 32-bit indices (a species holds fewer than 2^31 entries)
-    const unsigned b = (unsigned)ctl->begin[2], n = (unsigned)(ctl->end[2] - ctl->begin[2]);
-    const T *icdf = reinterpret_cast<const T *>(a.icdf_pair);
-    const SpeciesDev &S = a.sp[2];
-    unsigned long long my_steps = 0, my_ev = 0;
-    unsigned my_max = 0, n64 = 0;
-    const Phase<T> ph0 = time_phase<T, StepTime>(tm, 0.0);
-    // FP32 step-start pass: each thread stages its next photon in shared
-    // memory (two buffers) while it works on the current one
-    constexpr bool STAGE = FRESH && sizeof(T) == 4;
-    constexpr int NB = STAGE ? 2 : 1, NF = STAGE ? 9 : 1, NT = STAGE ? LB : 1;
-    __shared__ __align__(16) float stg[NB][NF][NT];       // w x y z kx ky kz id(2 words)
-    const unsigned stride = gridDim.x * blockDim.x;
-    auto stage = [&](unsigned jj, int buf) {
+    if (blockIdx.x * NT < n) {
+        for (int i = threadIdx.x; i < RateWords<T>::N; i += NT) s_coef[i] = reinterpret_cast<const T *>(a.coef)[i];
+        if (threadIdx.x == 0) s_tm = load_step_time(a);
+        __syncthreads();
+        const StepTime &tm = s_tm;
+        const T *icdf = reinterpret_cast<const T *>(a.icdf_pair);
+        const SpeciesDev &S = a.sp[2];
+        PassStats ps;
+        const Phase<T> ph0 = time_phase<T, StepTime>(tm, 0.0);
+        // FP32: each thread stages its next photon in shared memory (two
+        // buffers) while it works on the current one
+        constexpr bool STAGE = sizeof(T) == 4;
+        constexpr int NB = STAGE ? 2 : 1, NF = STAGE ? 9 : 1, NS = STAGE ? NT : 1;
+        __shared__ __align__(16) float stg[NB][NF][NS];       // w x y z kx ky kz id(2 words)
+        const unsigned stride = gridDim.x * NT;
+        auto stage = [&](unsigned i, int buf) {
+            if constexpr (STAGE) {
+                const int t = threadIdx.x;
+                cp_async4(&stg[buf][0][t], reinterpret_cast<const float *>(S.w) + i);
+                cp_async4(&stg[buf][1][t], reinterpret_cast<const float *>(S.x) + i);
+                cp_async4(&stg[buf][2][t], reinterpret_cast<const float *>(S.y) + i);
+                cp_async4(&stg[buf][3][t], reinterpret_cast<const float *>(S.z) + i);
+                cp_async4(&stg[buf][4][t], reinterpret_cast<const float *>(S.px) + i);
+                cp_async4(&stg[buf][5][t], reinterpret_cast<const float *>(S.py) + i);
+                cp_async4(&stg[buf][6][t], reinterpret_cast<const float *>(S.pz) + i);
+                cp_async4(&stg[buf][7][t], S.id + i);          // id: two 4-byte halves
+                cp_async4(&stg[buf][8][t], reinterpret_cast<const unsigned *>(S.id + i) + 1);
+            }
+        };
+        const unsigned j0 = blockIdx.x * NT + threadIdx.x;
         if constexpr (STAGE) {
-            const unsigned ii = b + jj;
-            const int t = threadIdx.x;
-            cp_async4(&stg[buf][0][t], reinterpret_cast<const float *>(S.w) + ii);
-            cp_async4(&stg[buf][1][t], reinterpret_cast<const float *>(S.x) + ii);
-            cp_async4(&stg[buf][2][t], reinterpret_cast<const float *>(S.y) + ii);
-            cp_async4(&stg[buf][3][t], reinterpret_cast<const float *>(S.z) + ii);
-            cp_async4(&stg[buf][4][t], reinterpret_cast<const float *>(S.px) + ii);
-            cp_async4(&stg[buf][5][t], reinterpret_cast<const float *>(S.py) + ii);
-            cp_async4(&stg[buf][6][t], reinterpret_cast<const float *>(S.pz) + ii);
-            cp_async4(&stg[buf][7][t], S.id + ii);          // id: two 4-byte halves
-            cp_async4(&stg[buf][8][t], reinterpret_cast<const unsigned *>(S.id + ii) + 1);
-        }
-    };
-    const unsigned j0 = blockIdx.x * blockDim.x + threadIdx.x;
-    if constexpr (STAGE) {
-        if (j0 < n) stage(j0, 0);
-        cp_async_commit();
-    }
-    int buf = 0;
-    for (unsigned j = j0; j < n; j += stride, buf ^= 1) {
-        const unsigned i = b + j;
-        T w, x[3], kx, ky, kz;
-        unsigned long long id;
-        if constexpr (STAGE) {
-            if (j + stride < n) stage(j + stride, buf ^ 1);
+            if (j0 < n) stage(j0, 0);
             cp_async_commit();
-            cp_async_wait_prev();                // this thread's copies of photon j have landed
-            const int t = threadIdx.x;
-            w = stg[buf][0][t];
-            x[0] = stg[buf][1][t]; x[1] = stg[buf][2][t]; x[2] = stg[buf][3][t];
-            kx = stg[buf][4][t]; ky = stg[buf][5][t]; kz = stg[buf][6][t];
-            id = (unsigned long long)__float_as_uint(stg[buf][7][t]) |
-                 ((unsigned long long)__float_as_uint(stg[buf][8][t]) << 32);
-        } else {
-            // all loads issued together (live photons are the rule: the photons
-            // that converted were removed at the end of the previous step)
-            w = ld<T>(S.w, i);
-            x[0] = ld<T>(S.x, i); x[1] = ld<T>(S.y, i); x[2] = ld<T>(S.z, i);
-            kx = ld<T>(S.px, i); ky = ld<T>(S.py, i); kz = ld<T>(S.pz, i);
-            id = __ldg(S.id + i);
         }
-        unsigned k;
-        if (!photon_step<T, FRESH>(a, tm, s_coef, icdf, ph0, S, i, w, x, kx, ky, kz, id, k, n64)) continue;
-        st<T>(S.x, i, x[0]); st<T>(S.y, i, x[1]); st<T>(S.z, i, x[2]);
-        ++my_steps;
-        my_ev += k;
-        my_max = max(my_max, k);
+        int buf = 0;
+        for (unsigned i = j0; i < n; i += stride, buf ^= 1) {
+            T w, x[3], kv[3];
+            unsigned long long id;
+            if constexpr (STAGE) {
+                if (i + stride < n) stage(i + stride, buf ^ 1);
+                cp_async_commit();
+                cp_async_wait_prev();                // this thread's copies of photon i have landed
+                const int t = threadIdx.x;
+                w = stg[buf][0][t];
+                x[0] = stg[buf][1][t]; x[1] = stg[buf][2][t]; x[2] = stg[buf][3][t];
+                kv[0] = stg[buf][4][t]; kv[1] = stg[buf][5][t]; kv[2] = stg[buf][6][t];
+                id = (unsigned long long)__float_as_uint(stg[buf][7][t]) |
+                     ((unsigned long long)__float_as_uint(stg[buf][8][t]) << 32);
+            } else {
+                // all loads issued together (live photons are the rule)
+                w = ld<T>(S.w, i);
+                x[0] = ld<T>(S.x, i); x[1] = ld<T>(S.y, i); x[2] = ld<T>(S.z, i);
+                kv[0] = ld<T>(S.px, i); kv[1] = ld<T>(S.py, i); kv[2] = ld<T>(S.pz, i);
+                id = __ldg(S.id + i);
+            }
+            if (!(w > (T)0)) continue;
+            ++ps.ph;
+            const T k0 = f_sqrt(kv[0] * kv[0] + kv[1] * kv[1] + kv[2] * kv[2]);
+            if (k0 > (T)0) {
+                const T inv = f_div((T)1, k0);
+                const T nx = kv[0] * inv, ny = kv[1] * inv, nz = kv[2] * inv;
+                T E[3], B[3];
+                field_at<T>(a, x, ph0, E, B);
+                double tau = 0.0;
+                uint2 rz = make_uint2(0, 0);
+                if (photon_flight<T, true>(a, tm, s_coef, E, B, x, kv, k0, inv, nx, ny, nz, tau, id, rz, ps.n64)) {
+                    pair_create<T>(a, tm, icdf, x, kv, k0, nx, ny, nz, tau, w, id, 0u, rz, ps.n64,
+                                   [](int, unsigned) {});
+                    st<T>(S.w, i, (T)0);       // the photon is eliminated
+                    S.nev[i] += 1u;
+                    ++ps.pr;
+                    ps.mx = 1u;
+                }
+            }
+            st<T>(S.x, i, x[0]); st<T>(S.y, i, x[1]); st<T>(S.z, i, x[2]);
+        }
+        __syncwarp();
+        flush_stats(ctl, ps);
     }
-    __syncwarp();
-    flush_stats(ctl, my_steps, my_ev, my_max, true, n64);
+    if (last_block(ctl) && threadIdx.x < 2) ctl->born[threadIdx.x] = count_now(ctl, threadIdx.x);
 }
 
 
@@ -687,10 +869,9 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_lepton_od(Pas
     const unsigned long long b0 = ctl->begin[0], n0 = ctl->end[0] - b0;
     const unsigned long long b1 = ctl->begin[1], n1 = ctl->end[1] - b1;
     const unsigned long long n = n0 + n1;
-    const LeptonCtx<T> c{a, ctl, s_coef, reinterpret_cast<const T *>(a.icdf_em), ctl->capacity[2], (T)(ALPHA * RS),
+    const LeptonCtx<T> c{a, ctl, s_coef, reinterpret_cast<const T *>(a.icdf_em), ctl->capacity[2], 0u, (T)(ALPHA * RS),
                          tm, time_phase<T, StepTime>(tm, 0.0)};
-    unsigned long long my_steps = 0, my_ev = 0;
-    unsigned my_max = 0, n64 = 0;
+    PassStats ps;
     for (unsigned long long j = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; j < n;
          j += (unsigned long long)gridDim.x * blockDim.x) {
         const int s = j < n0 ? 0 : 1;
@@ -702,11 +883,11 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_lepton_od(Pas
         T p[3] = {ld<T>(S.px, i), ld<T>(S.py, i), ld<T>(S.pz, i)};
         const unsigned long long id = __ldg(S.id + i);
         T od = ld<T>(S.od, i);
-        ++my_steps;
+        ++ps.lep;
         T E[3], B[3];
         field_at<T>(a, x, c.ph0, E, B);
         T gam, chi, p2;
-        lepton_chi<T>(p, E, B, gam, chi, p2, n64, a.field_zero);
+        lepton_chi<T>(p, E, B, gam, chi, p2, ps.n64, a.field_zero);
         const T lam = p2 > (T)0 ? c.alpha_r / gam * rate_em<T>(c.coef, chi) : (T)0;
         od = od_advance<T>(a, tm.step, id, od, lam);
         const T qch = s == 0 ? (T)-1 : (T)1;
@@ -715,12 +896,14 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_lepton_od(Pas
         if (od <= (T)0) {
             // the event at the end of the step
             field_tau<T>(a, tm, x, a.dt, E, B);
-            lepton_chi<T>(p, E, B, gam, chi, p2, n64, a.field_zero);
+            lepton_chi<T>(p, E, B, gam, chi, p2, ps.n64, a.field_zero);
             const uint4 r = event_draw(a.keys, id, tm.step, 0u);
             T om, ue, ve;
             Uniform<T>::draw(r.z, r.w, ue, ve);
             const T delta = sample_emission<T>(c.icdf, chi, ue, ve, &om);
-            emit_with<T>(c, x, p, a.dt, w, id, 0u, gam, p2, delta, om);
+            T kv[3];
+            if (recoil<T>(a, p, gam, p2, delta, om, kv))
+                append_photon<T>(a, ctl, c.cap_ph, x, kv, w, event_draw(a.seed ^ CHILD_KEY_XOR, id, tm.step, 0u));
             od = od_exp1<T>(r);
             k = 1;
         }
@@ -728,11 +911,11 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_lepton_od(Pas
         st<T>(S.px, i, p[0]); st<T>(S.py, i, p[1]); st<T>(S.pz, i, p[2]);
         st<T>(S.od, i, od);
         if (k) S.nev[i] += 1u;
-        my_ev += k;
-        my_max = max(my_max, k);
+        ps.em += k;
+        ps.mx = max(ps.mx, k);
     }
     __syncwarp();
-    flush_stats(ctl, my_steps, my_ev, my_max, false, n64);
+    flush_stats(ctl, ps);
 }
 
 template <class T>
@@ -749,8 +932,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_photon_od(Pas
     const T *icdf = reinterpret_cast<const T *>(a.icdf_pair);
     const T alpha_r = (T)(ALPHA * RS);
     const SpeciesDev &S = a.sp[2];
-    unsigned long long my_steps = 0, my_ev = 0;
-    unsigned my_max = 0, n64 = 0;
+    PassStats ps;
     const Phase<T> ph0 = time_phase<T, StepTime>(tm, 0.0);
     // FP32: each thread stages its next photon in shared memory (two
     // buffers) while it works on the current one, as in the step-start pass
@@ -803,7 +985,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_photon_od(Pas
             od = ld<T>(S.od, i);
         }
         if (!(w > (T)0)) continue;
-        ++my_steps;
+        ++ps.ph;
         const T k0 = f_sqrt(kv[0] * kv[0] + kv[1] * kv[1] + kv[2] * kv[2]);
         unsigned k = 0;
         if (k0 > (T)0) {
@@ -811,7 +993,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_photon_od(Pas
             const T nx = kv[0] * inv, ny = kv[1] * inv, nz = kv[2] * inv;
             T E[3], B[3];
             field_at<T>(a, x, ph0, E, B);
-            T chi = photon_chi<T>(k0, kv, E, B, n64, a.field_zero);
+            T chi = photon_chi<T>(k0, kv, E, B, ps.n64, a.field_zero);
             const T lam = alpha_r / k0 * rate_pair<T>(s_coef, chi);
             od = od_advance<T>(a, tm.step, id, od, lam);
             const T h = dt_of<T>(a);
@@ -819,7 +1001,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_photon_od(Pas
             if (od <= (T)0) {
                 // pair creation at the end of the step
                 field_tau<T>(a, tm, x, a.dt, E, B);
-                chi = photon_chi<T>(k0, kv, E, B, n64, a.field_zero);
+                chi = photon_chi<T>(k0, kv, E, B, ps.n64, a.field_zero);
                 const uint4 r = event_draw(a.keys, id, tm.step, 0u);
                 T om, ue, ve;
                 Uniform<T>::draw(r.z, r.w, ue, ve);
@@ -860,11 +1042,11 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_photon_od(Pas
         st<T>(S.x, i, x[0]); st<T>(S.y, i, x[1]); st<T>(S.z, i, x[2]);
         st<T>(S.od, i, od);
         if (k) { st<T>(S.w, i, w); S.nev[i] += 1u; }
-        my_ev += k;
-        my_max = max(my_max, k);
+        ps.pr += k;
+        ps.mx = max(ps.mx, k);
     }
     __syncwarp();
-    flush_stats(ctl, my_steps, my_ev, my_max, true, n64);
+    flush_stats(ctl, ps);
 }
 
 // ---- host side ----
@@ -917,32 +1099,41 @@ template <class K> inline int resident_blocks_smem(const qed_ctx *ctx, K kernel,
     return ctx->sm_count * per_sm;
 }
 
-template <class T, bool FRESH>
-qed_status launch_pass_t(qed_ctx *ctx, PassArgs &a, bool photons) {
-    const int threads = LB;
-    const int bp = resident_blocks(ctx, k_photon_pass<T, FRESH>, threads);
-    cudaStream_t st = ctx->stream;
-    qed_status e;
-    if (a.mlp_w16) {
+template <class T, bool FRESH, bool MLP>
+qed_status launch_leptons(qed_ctx *ctx, PassArgs &a, cudaGraphConditionalHandle h, int loop) {
+    const int threads = LB<T>, smem = MLP ? MLP_SMEM_BYTES : 0;
+    if constexpr (MLP) {
         static bool attr_set = false;   // the attribute is per function, set once
         if (!attr_set) {
-            SFQ_CUDA(cudaFuncSetAttribute(k_lepton_pass<T, FRESH, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          MLP_SMEM_BYTES));
+            SFQ_CUDA(cudaFuncSetAttribute(k_lepton_pass<T, FRESH, MLP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
             attr_set = true;
         }
-        const int bl = resident_blocks_smem(ctx, k_lepton_pass<T, FRESH, true>, threads, MLP_SMEM_BYTES);
-        e = timed_launch(ctx, 0, [&] { k_lepton_pass<T, FRESH, true><<<bl, threads, MLP_SMEM_BYTES, st>>>(a); });
-    } else {
-        const int bl = resident_blocks(ctx, k_lepton_pass<T, FRESH, false>, threads);
-        e = timed_launch(ctx, 0, [&] { k_lepton_pass<T, FRESH, false><<<bl, threads, 0, st>>>(a); });
     }
-    if (e != QED_OK) return e;
+    const int bl = MLP ? resident_blocks_smem(ctx, k_lepton_pass<T, FRESH, MLP>, threads, smem)
+                       : resident_blocks(ctx, k_lepton_pass<T, FRESH, MLP>, threads);
+    qed_status e =
+        timed_launch(ctx, 0, [&] { k_lepton_pass<T, FRESH, MLP><<<bl, threads, smem, ctx->stream>>>(a, h, loop); });
     SFQ_LAUNCHED(ctx, 1);
-    if (photons) {
-        e = timed_launch(ctx, 1, [&] { k_photon_pass<T, FRESH><<<bp, threads, 0, st>>>(a); });
+    return e;
+}
+
+// One step (a.pass == 0): the photons, then the leptons with the newborns;
+// or a further launch for newborns left behind (a.pass > 0).  loop: the
+// lepton pass sets the condition of the step graph's while node h.
+template <class T>
+qed_status launch_pass(qed_ctx *ctx, PassArgs &a, bool photons, cudaGraphConditionalHandle h, int loop) {
+    qed_status e = QED_OK;
+    if (a.pass == 0 && photons) {
+        const int bp = resident_blocks(ctx, k_photon_pass<T>, 256);
+        e = timed_launch(ctx, 1, [&] { k_photon_pass<T><<<bp, 256, 0, ctx->stream>>>(a); });
         if (e != QED_OK) return e;
         SFQ_LAUNCHED(ctx, 1);
     }
+    if (a.mlp_w16)
+        e = a.pass == 0 ? launch_leptons<T, true, true>(ctx, a, h, loop) : launch_leptons<T, false, true>(ctx, a, h, loop);
+    else
+        e = a.pass == 0 ? launch_leptons<T, true, false>(ctx, a, h, loop) : launch_leptons<T, false, false>(ctx, a, h, loop);
+    if (e != QED_OK) return e;
     SFQ_CUDA(cudaGetLastError());
     return QED_OK;
 }
@@ -964,12 +1155,6 @@ qed_status launch_od(qed_ctx *ctx, PassArgs &a, bool photons) {
     SFQ_CUDA(cudaGetLastError());
     return QED_OK;
 }
-
-template <class T>
-qed_status launch_pass(qed_ctx *ctx, PassArgs &a, bool photons) {
-    return a.pass == 0 ? launch_pass_t<T, true>(ctx, a, photons) : launch_pass_t<T, false>(ctx, a, photons);
-}
-
 
 }  // namespace SFQ_PASS_NS
 }  // namespace sfq

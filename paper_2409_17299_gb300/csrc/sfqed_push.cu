@@ -1,11 +1,7 @@
 // K2 / K3: the per-particle QED step (arXiv:2409.17299 Sec. 3, Algorithms 1-2).
 //
-// One pass kernel per particle kind.  Each thread takes one particle of the
-// pass range (grid-stride), runs Algorithm 1 for it to the end of the step
-// (rate -> waiting time -> Boris push -> event), and appends every particle
-// it creates with a warp-aggregated atomic.  Newborns carry their birth
-// clock and are pushed by the next pass (Algorithm 2): leptons and photons
-// are swept alternately until a pass creates nothing.
+// One pass kernel per particle kind (sfqed_pass.cuh): the photons, then the
+// leptons with everything born in the step (Algorithm 2).
 #include <math.h>
 #include <string.h>
 
@@ -28,8 +24,8 @@ __global__ void k_grid_interleave(const T *src, T *dst, long long nodes) {
     dst[8 * n + 7] = (T)0;
 }
 
-// Newborn passes of one step after which the step gives up (QED_ERR_TIMEOUT),
-// unless the configuration sets another limit.
+// Generations of newborns in one step after which the step gives up
+// (QED_ERR_TIMEOUT), unless the configuration sets another limit.
 constexpr unsigned long long PASS_LIMIT = 100000;
 static unsigned long long pass_limit_of(const qed_ctx *ctx) {
     return ctx->cfg.pass_limit > 0 ? (unsigned long long)ctx->cfg.pass_limit : PASS_LIMIT;
@@ -56,48 +52,13 @@ __global__ void k_step_begin(DevCtl *ctl, double dt) {
     for (int s = 0; s < 3; ++s) {
         ctl->begin[s] = 0;
         ctl->end[s] = stop ? 0 : min(ctl->count[s], ctl->capacity[s]);
+        if (s < 2) ctl->born[s] = ctl->end[s];
     }
+    ctl->arrive = 0;
+    ctl->spilled = 0;
 }
 
 __global__ void k_set_step(DevCtl *ctl, unsigned long long step) { ctl->step_next = step; }
-
-__global__ void k_set_timeout(DevCtl *ctl) { ctl->timeout = 1; }
-
-// Pass ranges of the next newborn pass: the particles appended since the
-// previous pass.  In a step graph it also sets the condition of the loop
-// over passes (the only setter): another pass while one found work, at most
-// ctl->pass_limit per step (then the step is marked as timed out).
-__device__ __forceinline__ unsigned long long pass_setup(DevCtl *ctl) {
-    unsigned long long more = 0;
-    for (int s = 0; s < 3; ++s) {
-        const unsigned long long e = min(ctl->count[s], ctl->capacity[s]);
-        ctl->begin[s] = ctl->end[s];
-        ctl->end[s] = e;
-        if (e > ctl->begin[s]) more = 1;
-    }
-    if (ctl_stopped(ctl)) {
-        more = 0;
-        for (int s = 0; s < 3; ++s) ctl->begin[s] = ctl->end[s];
-    }
-    ctl->more = more;
-    ctl->passes += more;
-    ctl->step_passes += more;
-    return more;
-}
-
-__global__ void k_pass_setup(DevCtl *ctl) { pass_setup(ctl); }
-
-__global__ void k_pass_setup_cond(DevCtl *ctl, cudaGraphConditionalHandle h, int in_body) {
-    unsigned long long more = pass_setup(ctl);
-    const unsigned long long limit = ctl->pass_limit ? ctl->pass_limit : PASS_LIMIT;
-    if (more && ctl->step_passes > limit) {
-        ctl->timeout = 1;
-        more = 0;
-        for (int s = 0; s < 3; ++s) ctl->begin[s] = ctl->end[s];
-    }
-    if (in_body) ctl->graph_kernels += 3;       // the loop body: two passes and this kernel
-    cudaGraphSetConditional(h, more ? 1u : 0u);
-}
 
 // ---- component kernels for the parity tests ----
 __global__ void k_philox(const uint4 *ctr, long long n, uint2 key, uint4 *out) {
@@ -262,9 +223,9 @@ template <class F> static qed_status timed_block(qed_ctx *ctx, int which, F body
 
 // the pass kernels of the field's variant (analytic descriptors or grid)
 template <class T>
-static qed_status launch_pass(qed_ctx *ctx, PassArgs &a, bool photons) {
-    if (a.field_kind == QED_FIELD_GRID) return pass_grid::launch_pass<T>(ctx, a, photons);
-    return pass_analytic::launch_pass<T>(ctx, a, photons);
+static qed_status launch_pass(qed_ctx *ctx, PassArgs &a, bool photons, cudaGraphConditionalHandle h = 0, int loop = 0) {
+    if (a.field_kind == QED_FIELD_GRID) return pass_grid::launch_pass<T>(ctx, a, photons, h, loop);
+    return pass_analytic::launch_pass<T>(ctx, a, photons, h, loop);
 }
 
 template <class T>
@@ -274,10 +235,10 @@ static qed_status launch_od(qed_ctx *ctx, PassArgs &a, bool photons) {
 }
 
 // ---- the captured PIC step ----
-// One step as a CUDA graph: the step-begin kernel, the step-start passes,
-// then (a cascade) a while node sweeping the newborns until a pass creates
-// nothing (Algorithm 2), then each species' merge step (leveling and removal
-// of dead entries) decided on the device.  Every kernel reads its ranges and
+// One step as a CUDA graph: the step-begin kernel, the photon pass and the
+// lepton pass (a cascade: with a while node for newborns that a full block
+// list left behind, Algorithm 2), then each species' merge step (leveling and
+// removal of dead entries) decided on the device.  Every kernel reads its ranges and
 // the step's time from the control block, so one graph serves every step and
 // no step needs the host: a batch of steps is a run of graph launches.  The
 // graph is rebuilt when the bound arrays, capacities, field or step change.
@@ -321,16 +282,16 @@ static qed_status build_step_graph(qed_ctx *ctx, const PassArgs &args, qed_parti
         cudaError_t e = gb.capture(gb.g, [&] {
             k_step_begin<<<1, 1, 0, ctx->stream>>>(ctx->ctl, dt);
             a.pass = 0;
-            const qed_status q = od_method ? launch_od<T>(ctx, a, cascade) : launch_pass<T>(ctx, a, cascade);
+            const qed_status q = od_method ? launch_od<T>(ctx, a, cascade)
+                                           : launch_pass<T>(ctx, a, cascade, h_pass, loop ? 1 : 0);
             if (q != QED_OK) return q;
-            if (loop) k_pass_setup_cond<<<1, 1, 0, ctx->stream>>>(ctx->ctl, h_pass, 0);
             return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
         });
         if (e != cudaSuccess) {
             rc = QED_ERR_CUDA;
             break;
         }
-        gb.top_kernels = 2 + (cascade ? 1 : 0) + (loop ? 1 : 0);
+        gb.top_kernels = 2 + (cascade ? 1 : 0);
         if (loop) {
             cudaGraph_t body;
             if (gb.conditional(h_pass, cudaGraphCondTypeWhile, &body) != cudaSuccess) {
@@ -339,9 +300,8 @@ static qed_status build_step_graph(qed_ctx *ctx, const PassArgs &args, qed_parti
             }
             e = gb.capture(body, [&] {
                 a.pass = 1;
-                const qed_status q = launch_pass<T>(ctx, a, true);
+                const qed_status q = launch_pass<T>(ctx, a, true, h_pass, 1);
                 if (q != QED_OK) return q;
-                k_pass_setup_cond<<<1, 1, 0, ctx->stream>>>(ctx->ctl, h_pass, 1);
                 return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
             });
             if (e != cudaSuccess) {
@@ -391,7 +351,7 @@ static StepGraph *step_graph_for(qed_ctx *ctx, const PassArgs &a, qed_particles 
 }
 
 // Host-driven steps: the same kernels launched one by one, the host reading
-// the control block between newborn-pass groups and before the merge step.
+// the control block after the passes, before the merge step.
 // Used to time the kernels individually (cfg.profile: CUDA events around
 // each launch) and where graphs with conditional nodes are unavailable.
 template <class T>
@@ -399,7 +359,6 @@ static qed_status host_steps(qed_ctx *ctx, qed_particles *pw, PassArgs &a, doubl
     const bool cascade = ctx->cfg.push_photons != 0;
     const bool od_method = ctx->cfg.event_method == QED_METHOD_OPTICAL_DEPTH;
     qed_particles P = *pw;                         // counts below: bounds read back from the device
-    int spec_passes = ctx->spec_passes > 0 ? ctx->spec_passes : 2;
     for (int it = 0; it < nsteps; ++it) {
         a.pass = 0;
         k_step_begin<<<1, 1, 0, ctx->stream>>>(ctx->ctl, dt);
@@ -407,34 +366,14 @@ static qed_status host_steps(qed_ctx *ctx, qed_particles *pw, PassArgs &a, doubl
         qed_status e = od_method ? launch_od<T>(ctx, a, cascade) : launch_pass<T>(ctx, a, cascade);
         if (e != QED_OK) return e;
         if (cascade && !od_method) {
-            // Algorithm 2: sweep the newborns until a pass creates nothing.
-            // Passes are enqueued in groups (a pass over an empty range
-            // returns at once), so the host reads the control block once per
-            // group; the group size follows the previous step's pass count.
-            int pass = 1;
-            k_pass_setup<<<1, 1, 0, ctx->stream>>>(ctx->ctl);
-            SFQ_LAUNCHED(ctx, 1);
-            for (;;) {
-                for (int g = 0; g < spec_passes; ++g, ++pass) {
-                    a.pass = pass;
-                    e = launch_pass<T>(ctx, a, true);
-                    if (e != QED_OK) return e;
-                    k_pass_setup<<<1, 1, 0, ctx->stream>>>(ctx->ctl);
-                    SFQ_LAUNCHED(ctx, 1);
-                }
+            // newborns left behind by a full block list take further launches
+            for (a.pass = 1;; ++a.pass) {
                 e = read_ctl(ctx);
                 if (e != QED_OK) return e;
-                if (ctx->ctl_host->overflow || !ctx->ctl_host->more) break;
-                if ((unsigned long long)pass >= pass_limit_of(ctx)) {
-                    // give up like the graph's loop does (the wait reports it)
-                    k_set_timeout<<<1, 1, 0, ctx->stream>>>(ctx->ctl);
-                    SFQ_LAUNCHED(ctx, 1);
-                    break;
-                }
+                if (!ctx->ctl_host->more) break;
+                e = launch_pass<T>(ctx, a, true);
+                if (e != QED_OK) return e;
             }
-            // passes with work in this step (the control block counts them)
-            const long long used = (long long)ctx->ctl_host->step_passes;
-            spec_passes = used < 1 ? 1 : (used > 8 ? 8 : (int)used);
         }
         if (cascade || ctx->cfg.thin_cap > 0) {
             // merge step (Sec. 4.2): drop dead photons, then level
@@ -459,7 +398,6 @@ static qed_status host_steps(qed_ctx *ctx, qed_particles *pw, PassArgs &a, doubl
             }
         }
     }
-    ctx->spec_passes = spec_passes;
     return QED_OK;
 }
 
@@ -488,7 +426,7 @@ static qed_status open_batch(qed_ctx *ctx, qed_particles *p, int64_t step0) {
     SFQ_CUDA(cudaMemcpyAsync(ctx->ctl, &h, sizeof(DevCtl), cudaMemcpyHostToDevice, ctx->stream));
     int64_t cap_max = 0;
     for (int s = 0; s < 3; ++s) {
-        qed_status e = ensure_tau(ctx, s, p->s[s].capacity);
+        qed_status e = s < 2 ? ensure_tau(ctx, s, p->s[s].capacity) : QED_OK;
         if (e != QED_OK) return e;
         cap_max = p->s[s].capacity > cap_max ? p->s[s].capacity : cap_max;
     }
@@ -533,7 +471,8 @@ static qed_status enqueue_steps(qed_ctx *ctx, const qed_field_desc *field, doubl
     for (int s = 0; s < 3; ++s) {
         const qed_species &S = p->s[s];
         a.sp[s] = SpeciesDev{S.x, S.y, S.z, S.px, S.py, S.pz, S.w,
-                             reinterpret_cast<unsigned long long *>(S.id), S.nevents, ctx->tau[s], ctx->od[s]};
+                             reinterpret_cast<unsigned long long *>(S.id), S.nevents, s < 2 ? ctx->tau[s] : nullptr,
+                             ctx->od[s]};
     }
     a.ctl = ctx->ctl;
     const bool f32 = sizeof(T) == 4;
@@ -579,7 +518,7 @@ static qed_status enqueue_steps(qed_ctx *ctx, const qed_field_desc *field, doubl
     a.seed = ctx->cfg.seed;
     a.keys = philox_keys(ctx->cfg.seed);
     a.soft_filter = ctx->cfg.soft_photon_filter;
-    a.record_newborn_tau = cascade ? 1 : 0;
+    a.fly_newborns = cascade && ctx->cfg.event_method == QED_METHOD_SUBSTEP ? 1 : 0;
 
     ctx->async_deferred = 1;
     StepGraph *G = ctx->cfg.profile ? nullptr : step_graph_for<T>(ctx, a, p, dt);
