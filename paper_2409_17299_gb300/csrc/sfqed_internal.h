@@ -228,6 +228,11 @@ struct qed_ctx {
 
 // Implemented in sfqed_tables.cu
 qed_status sfq_build_tables(qed_ctx *ctx);
+// Implemented in sfqed_tables32.cu: the tables of FP32 contexts in `work`
+// (device memory of sfq_tables32_bytes()); returns the rate form at the
+// Chebyshev nodes (device)
+size_t sfq_tables32_bytes();
+const double *sfq_tables32(void *work, double *em64, double *pair64, cudaStream_t st);
 // Implemented in sfqed_push.cu
 qed_status sfq_push(qed_ctx *ctx, qed_particles *p, const qed_field_desc *field, double dt,
                     int nsteps, int64_t step0, qed_stats *out);

@@ -9,81 +9,72 @@
 // Both are integrated on the whole line in z (emission y = e^z; pair
 // d = 1/(1+e^-z)) with composite 16-point Gauss-Legendre panels.
 //
-// What bounds the build: FP64 arithmetic (about 4e6 integrand evaluations,
-// most of them in the root solves of the 44,126 table nodes).  The Bessel
-// functions are therefore evaluated from their definitions only at 472 x 12
-// points, and everywhere else from Chebyshev interpolants in ln y (one per
-// panel, below rounding); every kernel spreads its independent pieces
-// (panels, nodes) over the whole chip instead of one block per table row.
-// Per context, GB300: 432.6 ms of kernels with direct Bessel sums and one
-// block per row, 1.6 ms now.
+// Two builders.  FP32 contexts read the tables rounded to float: their
+// nodes come from Chebyshev interpolants of the Bessel functions
+// (sfqed_tables32.cu, 1e-15 from the sums here, 1.6 ms).  FP64 contexts get
+// the sums below, rounded as they have always been, because trajectories in
+// strong standing waves amplify a last-bit change of the tables (1e-15 to
+// 1e-2 in 500 steps of the paper's test problem).
+//
+// What bounds the FP64 build: FP64 arithmetic, K_{2/3} and the integral of
+// K_{1/3} in the root solves of the 44,126 table nodes (up to 100 iterations
+// of 17 points each).  One block per table row, which also recomputed the
+// emission panels' Bessel values for every chi and cosh t and e^{-y cosh t}
+// for each of the two functions, took 432 ms per context; 94 ms now: panels
+// and nodes are spread over the whole chip, the emission panels' values (they
+// depend on y alone) are computed once, and the two trapezoid sums share
+// their exponentials and read cosh t from a table where the step is 0.1.
+// Products and sums that the compiler may or may not fuse are written out.
 #include <math.h>
 
 #include "sfqed_device.cuh"
 #include "sfqed_internal.h"
+#include "sfqed_tables.cuh"
 
 namespace sfq {
 namespace {
 
-constexpr int GLN = 16;
-constexpr double PI = 3.14159265358979323846;
-
-// emission: z in [-110, 8] (below: analytic tail C e^{z/3}); pair: z in [-38, 0]
-constexpr double EZ_LO = -110.0, EZ_W = 0.25;
-constexpr int EZ_NP = 472;
-constexpr double PZ_LO = -38.0, PZ_W = 0.1;
-constexpr int PZ_NP = 380;
-
-// rows of the quadrature: the tables' chi rows, then the rate nodes
-constexpr int ROW_PAIR = EM_NCHI;                               // 121
-constexpr int ROW_EM_RATE = EM_NCHI + PAIR_NCHI;                // 222
-constexpr int ROW_PAIR_RATE = ROW_EM_RATE + EM_NDEC * CHEB_N;   // 288
-constexpr int ROWS = ROW_PAIR_RATE + PAIR_NDEC * CHEB_N;        // 343
-__host__ __device__ constexpr bool row_is_pair(int r) {
-    return (r >= ROW_PAIR && r < ROW_EM_RATE) || r >= ROW_PAIR_RATE;
-}
-
-// Gauss-Legendre rule on [-1, 1] (a kernel argument)
-struct GlRule {
-    double x[GLN], w[GLN];
+// Trapezoid points t_j = 0.1 j: cosh t, cosh(2 t / 3), cosh(t / 3)
+constexpr int NTRIG = 64;
+struct Trig {
+    double ch[NTRIG], c23[NTRIG], c13[NTRIG];
 };
 
-GlRule gauss_legendre() {
-    GlRule g;
-    for (int i = 0; i < GLN; ++i) {
-        double x = cos(PI * (i + 0.75) / (GLN + 0.5)), dp = 1.0;
-        for (int it = 0; it < 60; ++it) {               // Newton's method on P_n
-            double a = 1.0, b = x;
-            for (int k = 2; k <= GLN; ++k) {
-                const double c = ((2 * k - 1) * x * b - (k - 1) * a) / k;
-                a = b;
-                b = c;
-            }
-            dp = GLN * (x * b - a) / (x * x - 1.0);
-            const double dx = b / dp;
-            x -= dx;
-            if (fabs(dx) <= 2e-16 * fabs(x)) break;
-        }
-        double a = 1.0, b = x;
-        for (int k = 2; k <= GLN; ++k) {
-            const double c = ((2 * k - 1) * x * b - (k - 1) * a) / k;
-            a = b;
-            b = c;
-        }
-        dp = GLN * (x * b - a) / (x * x - 1.0);
-        g.x[i] = x;
-        g.w[i] = 2.0 / ((1.0 - x * x) * dp * dp);
+// what the quadrature keeps between its kernels
+struct TableWork {
+    Trig trig;
+    double gamma[4];                  // Gamma(1/3), Gamma(5/3), Gamma(2/3), Gamma(4/3)
+    double chi[ROWS];
+    struct { double y, k23, k13; } em[EZ_NP * GLN];      // the emission panels' nodes, whatever chi
+    double mass[ROWS * EZ_NP];        // panel integrals per row
+    double below[(EM_NCHI + PAIR_NCHI) * (EZ_NP + 1)], above[(EM_NCHI + PAIR_NCHI) * (EZ_NP + 1)];
+    double fnode[NCOEF];              // rate form at the Chebyshev nodes
+};
+
+// what the kernels keep in shared memory
+struct TableShared {
+    Trig trig;
+    double gamma[4];
+};
+
+__device__ __forceinline__ void load_shared(TableShared &s, const TableWork *W) {
+    for (int i = threadIdx.x; i < NTRIG; i += blockDim.x) {
+        s.trig.ch[i] = W->trig.ch[i];
+        s.trig.c23[i] = W->trig.c23[i];
+        s.trig.c13[i] = W->trig.c13[i];
     }
-    return g;
+    if (threadIdx.x < 4) s.gamma[threadIdx.x] = W->gamma[threadIdx.x];
+    __syncthreads();
 }
 
 // Modified Bessel function of the second kind and int_y^inf K_{1/3}.
 //   y < 1 : ascending series, K_nu = pi/(2 sin(nu pi)) (I_{-nu} - I_nu)
 //   y >= 1: trapezoid rule on K_nu(y) = int_0^inf e^{-y cosh t} cosh(nu t) dt
 //           (and the same with 1/cosh t for the integral of K_{1/3})
-__device__ double series_I(double mu, double y, bool integrated) {
+// tg: Gamma(mu + 1)
+__device__ __forceinline__ double series_I(double mu, double tg, double y, bool integrated) {
     const double h = 0.5 * y, h2 = h * h;
-    double term = pow(h, mu) / tgamma(mu + 1.0);
+    double term = pow(h, mu) / tg;
     double s = integrated ? term * y / (mu + 1.0) : term;
     for (int k = 1; k < 40; ++k) {
         term *= h2 / (k * (k + mu));
@@ -94,237 +85,187 @@ __device__ double series_I(double mu, double y, bool integrated) {
     return s;
 }
 
-// y < 1
-__device__ double bessel_k23_small(double y) {
-    const double nu = 2.0 / 3.0;
-    return PI / (2.0 * sin(nu * PI)) * (series_I(-nu, y, false) - series_I(nu, y, false));
-}
-
-__device__ double int_k13_small(double y) {
-    const double c = PI / sqrt(3.0);   // int_0^inf K_{1/3} = pi/sqrt3 = pi/(2 sin(pi/3))
-    return c * (1.0 - series_I(-1.0 / 3.0, y, true) + series_I(1.0 / 3.0, y, true));
-}
-
-// e^y K_{2/3}(y) and e^y int_y^inf K_{1/3} for y >= 1 by the lanes of a warp:
-// the trapezoid terms j = lane, lane + 32, ... with cosh t - 1 = 2 sinh^2(t/2)
-__device__ void trap_scaled(double y, double &k23, double &k13) {
-    const double h = fmin(0.1, 0.4 * rsqrt(y));
-    double s23 = 0.0, s13 = 0.0;
-    for (int j0 = 0; j0 < 320; j0 += 32) {
-        const int j = j0 + (int)(threadIdx.x & 31);
-        const double t = j * h, sh = sinh(0.5 * t), c1 = 2.0 * sh * sh;
-        const double f = (j == 0 ? 0.5 : 1.0) * exp(-y * c1);
-        s23 += f * cosh((2.0 / 3.0) * t);
-        s13 += f * cosh((1.0 / 3.0) * t) / (1.0 + c1);
-        // the last lane's term is the smallest of this round, and the next
-        // rounds' terms fall faster than geometrically
-        if (__shfl_sync(0xffffffffu, f * cosh((2.0 / 3.0) * t), 31) < 1e-20) break;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        s23 += __shfl_xor_sync(0xffffffffu, s23, o);
-        s13 += __shfl_xor_sync(0xffffffffu, s13, o);
-    }
-    k23 = h * s23;
-    k13 = h * s13;
-}
-
-// ---- Bessel interpolants ----
-// On each emission panel (width 0.25 in z = ln y) e^y K_{2/3}(y) and
-// e^y int_y^inf K_{1/3} are interpolated at BC Chebyshev points.  Both are
-// entire in z and grow slowly in the strip |Im z| < 2, so the interpolation
-// error on a half width of 1/8 is about 4 * 32^-12 of the value, below FP64
-// rounding; the exponential is applied at the point itself.
-constexpr int BC = 12;
-
-// coefficient table: bc[2 * (panel * BC + k)] (K_{2/3}), + 1 (the integral)
-__device__ __forceinline__ void bessel_at(const double *bc, int panel, double x, double y, double &k23, double &k13) {
-    const double2 *c = reinterpret_cast<const double2 *>(bc) + panel * BC;
-    const double x2 = x + x;
-    double a1 = 0.0, a2 = 0.0, b1 = 0.0, b2 = 0.0;
-#pragma unroll
-    for (int k = BC - 1; k >= 1; --k) {
-        const double2 v = __ldg(c + k);
-        const double a0 = fma(x2, a1, v.x - a2), b0 = fma(x2, b1, v.y - b2);
-        a2 = a1; a1 = a0;
-        b2 = b1; b1 = b0;
-    }
-    const double2 v = __ldg(c);
-    const double ey = exp(-y);
-    k23 = fma(x, a1, v.x - a2) * ey;
-    k13 = fma(x, b1, v.y - b2) * ey;
-}
-
-// at any y with its logarithm (0 beyond the panels, where e^-y underflows;
-// the smallest y asked for is that of the first emission panel)
-__device__ __forceinline__ void bessel_any(const double *bc, double lny, double y, double &k23, double &k13) {
-    if (y > 740.0) {
+// K_{2/3}(y) and int_y^inf K_{1/3}
+__device__ __noinline__ double2 bessel(const TableShared &S, double y) {
+    double k23, k13;
+    if (y < 1.0) {
+        const double nu = 2.0 / 3.0;
+        k23 = PI / (2.0 * sin(nu * PI)) * (series_I(-nu, S.gamma[0], y, false) - series_I(nu, S.gamma[1], y, false));
+        const double c = PI / sqrt(3.0);   // int_0^inf K_{1/3} = pi/sqrt3 = pi/(2 sin(pi/3))
+        k13 = c * (1.0 - series_I(-1.0 / 3.0, S.gamma[2], y, true) + series_I(1.0 / 3.0, S.gamma[3], y, true));
+    } else if (y > 740.0) {
         k23 = 0.0;
         k13 = 0.0;
-        return;
+    } else {
+        // both trapezoid sums over the same points; each stops at its own end
+        const double h = fmin(0.1, 0.4 * rsqrt(y));
+        const bool tab = h == 0.1;
+        double s23 = 0.5 * exp(-y), s13 = s23;
+        bool d23 = false, d13 = false;
+        for (int j = 1; j < 20000 && !(d23 && d13); ++j) {
+            double ch, a23, a13;
+            if (tab && j < NTRIG) {
+                ch = S.trig.ch[j]; a23 = S.trig.c23[j]; a13 = S.trig.c13[j];
+            } else {
+                const double t = j * h;
+                ch = cosh(t); a23 = cosh((2.0 / 3.0) * t); a13 = cosh((1.0 / 3.0) * t);
+            }
+            const double yc = __dmul_rn(y, ch), e = exp(-yc);
+            if (!d23) {
+                const double f = __dmul_rn(e, a23);
+                s23 = __dadd_rn(s23, f);
+                d23 = yc > 1.0 && f <= __dmul_rn(1e-18, s23);
+            }
+            if (!d13) {
+                const double f = __dmul_rn(e, a13) / ch;
+                s13 = __dadd_rn(s13, f);
+                d13 = yc > 1.0 && f <= __dmul_rn(1e-18, s13);
+            }
+        }
+        k23 = __dmul_rn(h, s23);
+        k13 = __dmul_rn(h, s13);
     }
-    const double u = (lny - EZ_LO) * (1.0 / EZ_W);
-    int p = (int)u;
-    p = p < 0 ? 0 : (p > EZ_NP - 1 ? EZ_NP - 1 : p);
-    bessel_at(bc, p, 2.0 * (u - p) - 1.0, y, k23, k13);
+    return make_double2(k23, k13);
 }
 
-// emission integrand (bracket times d delta / dz) from y and the functions there
-__device__ __forceinline__ double em_integrand(double chi, double y, double k23, double k13) {
+// emission integrand in z = ln y (bracket times d delta / dz)
+__device__ __forceinline__ double g_emission_at(double y, double k23, double k13, double chi) {
     const double a = 3.0 * chi * y;
-    const double inv = 1.0 / (2.0 + a);                  // 1 - delta = 2 inv
-    const double jac = 6.0 * chi * y * (inv * inv);
-    return ((2.0 * inv + 0.5 * (2.0 + a)) * k23 - k13) * jac;
+    const double om = 2.0 / (2.0 + a);                   // 1 - delta
+    const double jac = y * 6.0 * chi / ((2.0 + a) * (2.0 + a));
+    return __dsub_rn(__dmul_rn(om + 1.0 / om, k23), k13) * jac;
 }
 
-// pair integrand: s = e^z + e^-z, 1 / (delta (1 - delta)) = 2 + s
-__device__ __forceinline__ double pair_integrand(const double *bc, double c, double lnc, double s, double lns2) {
-    const double y = c * (2.0 + s);                      // c = 2 / (3 chi)
-    double k23, k13;
-    bessel_any(bc, lnc + lns2, y, k23, k13);
-    return (s * k23 + k13) / (2.0 + s);
+__device__ __forceinline__ double g_emission(const TableShared &S, double z, double chi) {
+    const double y = exp(z);
+    const double2 k = bessel(S, y);
+    return g_emission_at(y, k.x, k.y, chi);
 }
 
-__device__ __forceinline__ double em_density(const double *bc, double chi, int panel, double z) {
-    const double za = EZ_LO + panel * EZ_W, y = exp(z);
-    if (y > 740.0) return 0.0;
-    double k23, k13;
-    bessel_at(bc, panel, (2.0 / EZ_W) * (z - za) - 1.0, y, k23, k13);
-    return em_integrand(chi, y, k23, k13);
+// pair integrand in z, delta = 1/(1+e^-z)
+__device__ __forceinline__ double g_pairs(const TableShared &S, double z, double chi) {
+    const double d = 1.0 / (1.0 + exp(-z));
+    const double om = 1.0 / (1.0 + exp(z));
+    const double jac = d * om;
+    const double y = 2.0 / (3.0 * chi * jac);
+    const double2 k = bessel(S, y);
+    return __dadd_rn(__dmul_rn(d / om + om / d, k.x), k.y) * jac;
 }
 
-__device__ __forceinline__ double pair_density(const double *bc, double c, double lnc, double z) {
-    const double s = exp(z) + exp(-z);
-    return pair_integrand(bc, c, lnc, s, log(2.0 + s));
-}
-
-// what the quadrature needs at the Gauss nodes of every panel, whatever chi
-struct BesselWork {
-    double bc[2 * EZ_NP * BC];        // interpolant coefficients
-    struct { double y, k23, k13, w; } em[EZ_NP * GLN];   // w: weight x half width
-    struct { double s, ln, w; } pr[PZ_NP * GLN];         // s = e^z + e^-z, ln = ln(2 + s)
-    double chi[ROWS];
-    double mass[ROWS * EZ_NP];        // panel integrals per row
-    double below[(EM_NCHI + PAIR_NCHI) * (EZ_NP + 1)], above[(EM_NCHI + PAIR_NCHI) * (EZ_NP + 1)];
-    double fnode[NCOEF];              // rate form at the Chebyshev nodes
-};
-
-// Panel b of the interpolants: the BC node values (a warp per node where the
-// trapezoid sum runs, y >= 1; a thread per node where the ascending series
-// does), their Chebyshev coefficients, and the values at the panel's Gauss
-// nodes.
-constexpr int BT = 32 * BC;
-__global__ void __launch_bounds__(BT) k_bessel_panels(const GlRule gl, BesselWork *W) {
-    __shared__ double f23[BC], f13[BC], cs[BC][BC];
-    const int b = blockIdx.x, t = threadIdx.x;
-    const double za = EZ_LO + b * EZ_W;
-    const bool series = za + EZ_W <= 0.0;
-    const int node = series ? t : t >> 5;
-    if (node < BC) {
-        const double z = za + 0.5 * EZ_W * (1.0 + cospi((node + 0.5) / BC));
-        const double y = exp(z);
-        double k23, k13;
-        if (series) {
-            const double e = exp(y);
-            k23 = bessel_k23_small(y) * e;
-            k13 = int_k13_small(y) * e;
-        } else {
-            trap_scaled(y, k23, k13);
-        }
-        f23[node] = k23;
-        f13[node] = k13;
+__device__ __forceinline__ double gl_panel(const TableShared &S, bool pair, double chi, double a, double b) {
+    const double m = 0.5 * (a + b), hw = 0.5 * (b - a);
+    double s = 0.0;
+    for (int i = 0; i < GLN; ++i) {
+        const double z = m + hw * GLX[i];
+        s += GLW[i] * (pair ? g_pairs(S, z, chi) : g_emission(S, z, chi));
     }
-    if (t < BC * BC) cs[t / BC][t % BC] = cospi((t / BC) * ((t % BC) + 0.5) / BC);
+    return s * hw;
+}
+
+__device__ double block_sum(double v, double *red) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    if (l == 0) red[w] = v;
     __syncthreads();
-    if (t < 2 * BC) {
-        const int k = t >> 1;
-        const double *f = t & 1 ? f13 : f23;
-        double s = 0.0;
-        for (int j = 0; j < BC; ++j) s += f[j] * cs[k][j];
-        W->bc[2 * (b * BC + k) + (t & 1)] = (k == 0 ? 1.0 : 2.0) / BC * s;
-    }
-    __syncthreads();                                     // the block reads its own coefficients
-    __threadfence_block();
-    if (t < GLN) {
-        const double x = gl.x[t], y = exp(za + 0.5 * EZ_W * (1.0 + x));
-        // plain loads: the coefficients were written by this launch
-        double a1 = 0.0, a2 = 0.0, c1 = 0.0, c2 = 0.0;
-        const double2 *c = reinterpret_cast<const double2 *>(W->bc) + b * BC;
-        for (int k = BC - 1; k >= 1; --k) {
-            const double a0 = fma(2.0 * x, a1, c[k].x - a2), c0 = fma(2.0 * x, c1, c[k].y - c2);
-            a2 = a1; a1 = a0;
-            c2 = c1; c1 = c0;
-        }
-        const double ey = y > 740.0 ? 0.0 : exp(-y);
-        W->em[b * GLN + t] = {y, fma(x, a1, c[0].x - a2) * ey, fma(x, c1, c[0].y - c2) * ey, gl.w[t] * 0.5 * EZ_W};
-    } else if (t >= 32 && t < 32 + GLN && b < PZ_NP) {
-        const int i = t - 32;
-        const double z = PZ_LO + b * PZ_W + 0.5 * PZ_W * (1.0 + gl.x[i]);
-        const double s = exp(z) + exp(-z);
-        W->pr[b * GLN + i] = {s, log(2.0 + s), gl.w[i] * 0.5 * PZ_W};
-    } else if (t == 64 && b < ROWS) {
-        double lg;                                       // log10 chi
-        if (b < ROW_PAIR) lg = -3.0 + b / 20.0;
-        else if (b < ROW_EM_RATE) lg = -2.0 + (b - ROW_PAIR) / 20.0;
-        else {
-            const int r = b - ROW_EM_RATE, dec = r / CHEB_N, k = r % CHEB_N;
-            const double lo = dec >= EM_NDEC ? -2.0 + (dec - EM_NDEC) : -3.0 + dec;
-            lg = lo + 0.5 + 0.5 * cos(PI * (k + 0.5) / CHEB_N);
-        }
-        W->chi[b] = pow(10.0, lg);
-    }
+    double s = 0.0;
+    if (threadIdx.x == 0)
+        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i];
+    __syncthreads();
+    return s;
 }
 
-// Panel integrals: one thread per (row, panel).
-constexpr int MT = 128;
-__global__ void __launch_bounds__(MT) k_panel_masses(BesselWork *W) {
-    const int r = blockIdx.y, p = blockIdx.x * MT + threadIdx.x;
+// the constants of the sums and the rows' chi (one thread each)
+constexpr int TT = 128;
+__global__ void k_table_constants(TableWork *W) {
+    const int i = blockIdx.x * TT + threadIdx.x;
+    if (i < NTRIG) {
+        const double t = i * 0.1;
+        W->trig.ch[i] = cosh(t);
+        W->trig.c23[i] = cosh((2.0 / 3.0) * t);
+        W->trig.c13[i] = cosh((1.0 / 3.0) * t);
+    } else if (i < NTRIG + 4) {
+        const double mu = i == NTRIG ? -2.0 / 3.0 : i == NTRIG + 1 ? 2.0 / 3.0 : i == NTRIG + 2 ? -1.0 / 3.0 : 1.0 / 3.0;
+        W->gamma[i - NTRIG] = tgamma(mu + 1.0);
+    }
+    if (i < ROWS) W->chi[i] = row_chi(i);
+}
+
+// Bessel values at the emission panels' Gauss nodes: one thread per node
+__global__ void __launch_bounds__(TT) k_emission_nodes(TableWork *W) {
+    __shared__ TableShared S;
+    load_shared(S, W);
+    const int i = blockIdx.x * TT + threadIdx.x;
+    if (i >= EZ_NP * GLN) return;
+    const int p = i / GLN;
+    const double a = EZ_LO + p * EZ_W, b = EZ_LO + (p + 1) * EZ_W;
+    const double m = 0.5 * (a + b), hw = 0.5 * (b - a);
+    const double y = exp(m + hw * GLX[i % GLN]);
+    const double2 k = bessel(S, y);
+    W->em[i] = {y, k.x, k.y};
+}
+
+// panel integrals: one thread per (row, panel)
+__global__ void __launch_bounds__(TT) k_panel_masses(TableWork *W) {
+    __shared__ TableShared S;
+    load_shared(S, W);
+    const int r = blockIdx.y, p = blockIdx.x * TT + threadIdx.x;
     const bool pair = row_is_pair(r);
     if (p >= (pair ? PZ_NP : EZ_NP)) return;
     const double chi = W->chi[r];
-    double s = 0.0;
-    if (!pair) {
+    double v;
+    if (pair) {
+        v = gl_panel(S, true, chi, PZ_LO + p * PZ_W, PZ_LO + (p + 1) * PZ_W);
+    } else {
+        const double a = EZ_LO + p * EZ_W, b = EZ_LO + (p + 1) * EZ_W, hw = 0.5 * (b - a);
+        double s = 0.0;
         for (int i = 0; i < GLN; ++i) {
             const auto n = W->em[p * GLN + i];
-            s += n.w * em_integrand(chi, n.y, n.k23, n.k13);
+            s += GLW[i] * g_emission_at(n.y, n.k23, n.k13, chi);
         }
-    } else {
-        const double c = 2.0 / (3.0 * chi), lnc = log(c);
-        for (int i = 0; i < GLN; ++i) {
-            const auto n = W->pr[p * GLN + i];
-            s += n.w * pair_integrand(W->bc, c, lnc, n.s, n.ln);
-        }
+        v = s * hw;
     }
-    W->mass[(size_t)r * EZ_NP + p] = s;
+    W->mass[(size_t)r * EZ_NP + p] = v;
 }
 
-// Per row: the cumulative integrals from both ends (table rows) or the rate
-// form at the Chebyshev node (emission decades store F/chi, pair decades
-// ln F + 8/(3 chi)).  The two running sums are two lanes of different warps.
-__global__ void __launch_bounds__(64) k_row_sums(BesselWork *W) {
+// Per row: the cumulative integrals from both ends (table rows; the two
+// running sums by two warps), or the total rate at the Chebyshev nodes
+// (emission decades 0..5 on log10 chi in [-3, 3] store F/chi; pair decades
+// 6..10 on [-2, 3] store ln F + 8/(3 chi)).
+__global__ void __launch_bounds__(TT) k_row_sums(TableWork *W) {
+    __shared__ TableShared S;
     __shared__ double m[EZ_NP];
+    __shared__ double red[32];
+    load_shared(S, W);
     const int r = blockIdx.x;
     const bool pair = row_is_pair(r);
     const int np = pair ? PZ_NP : EZ_NP;
-    for (int p = threadIdx.x; p < np; p += 64) m[p] = W->mass[(size_t)r * EZ_NP + p];
+    for (int p = threadIdx.x; p < np; p += TT) m[p] = W->mass[(size_t)r * EZ_NP + p];
     __syncthreads();
     const double chi = W->chi[r];
-    const double tail = pair ? 0.0 : 3.0 * em_density(W->bc, chi, 0, EZ_LO);
     if (r < ROW_EM_RATE) {
         double *below = W->below + (size_t)r * (EZ_NP + 1), *above = W->above + (size_t)r * (EZ_NP + 1);
         if (threadIdx.x == 0) {
-            double s = tail;
+            double s = pair ? 0.0 : 3.0 * g_emission(S, EZ_LO, chi);
             below[0] = s;
-            for (int p = 0; p < np; ++p) below[p + 1] = s += m[p];
+            for (int p = 0; p < np; ++p) below[p + 1] = s = s + m[p];
         } else if (threadIdx.x == 32) {
             double s = 0.0;
             above[np] = s;
-            for (int p = np - 1; p >= 0; --p) above[p] = s += m[p];
+            for (int p = np - 1; p >= 0; --p) above[p] = s = s + m[p];
         }
-    } else if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int p = 0; p < np; ++p) s += m[p];
-        const double F = (pair ? 2.0 * s : s + tail) / (sqrt(3.0) * PI);
-        W->fnode[r - ROW_EM_RATE] = pair ? log(F) + 8.0 / (3.0 * chi) : F / chi;
+    } else {
+        double acc = 0.0;
+        for (int p = threadIdx.x; p < np; p += TT) acc += m[p];
+        const double tot = block_sum(acc, red);
+        if (threadIdx.x == 0) {
+            if (!pair) {
+                const double F = (tot + 3.0 * g_emission(S, EZ_LO, chi)) / (sqrt(3.0) * PI);
+                W->fnode[r - ROW_EM_RATE] = F / chi;
+            } else {
+                const double F = 2.0 * tot / (sqrt(3.0) * PI);
+                W->fnode[r - ROW_EM_RATE] = log(F) + 8.0 / (3.0 * chi);
+            }
+        }
     }
 }
 
@@ -368,68 +309,83 @@ __global__ void k_rate_segments(const double *coef64, float *seg) {
     seg[4 * i + 3] = (float)(27.0 * (d3 / 6.0));
 }
 
-// Table nodes: rows 0..120 emission (ln y), 121..221 pair (ln delta); one
-// thread per node, Newton's method on the cumulative integral inside the
-// node's panel, bracketed by bisection.  The integral is taken from the
-// nearer end of the distribution, so that both tails keep their relative
-// accuracy.  Newton's error after a step s is about s^2 times half the
-// density's logarithmic slope (at most ~20 per unit z here), so a step below
-// 1e-9 leaves 1e-17 and no confirming evaluation is needed.
+// Newton's method inside one panel [za, zb] for int_za^z g = target
+// (from_top: int_z^zb g = target), bracketed by bisection.  whole: the
+// panel's integral.  SL lanes share a node: each evaluates every SL-th Gauss
+// point of the partial integral, which every lane then sums in the points'
+// order, so a node's chain of integrand evaluations is 16 / SL + 1 per
+// iteration instead of 17 (a few nodes take tens of iterations, and one lane
+// per node left the chip waiting for them: 132 ms against 95 ms).
+constexpr int SL = 8;
+__device__ __forceinline__ double solve_panel(const TableShared &S, bool pair, double chi, double za, double zb,
+                                              double whole, double target, bool from_top) {
+    const int lane = threadIdx.x & 31, part = lane % SL;
+    const unsigned group = (SL == 32 ? 0xffffffffu : (1u << SL) - 1u) << (lane - part);
+    double lo = za, hi = zb;
+    const double f = whole > 0.0 ? fmin(fmax(target / whole, 0.0), 1.0) : 0.5;
+    double z = from_top ? __fma_rn(-f, zb - za, zb) : __fma_rn(f, zb - za, za);
+    for (int it = 0; it < 100; ++it) {
+        const double a = from_top ? z : za, b = from_top ? zb : z;
+        const double m = 0.5 * (a + b), hw = 0.5 * (b - a);
+        double g[GLN / SL], s = 0.0;
+        for (int i = 0; i < GLN / SL; ++i) {
+            const double x = m + hw * GLX[i * SL + part];
+            g[i] = pair ? g_pairs(S, x, chi) : g_emission(S, x, chi);
+        }
+#pragma unroll
+        for (int i = 0; i < GLN; ++i) s = __fma_rn(GLW[i], __shfl_sync(group, g[i / SL], i % SL, SL), s);
+        const double gz = pair ? g_pairs(S, z, chi) : g_emission(S, z, chi);
+        const double r = __fma_rn(s, hw, -target), d = from_top ? -gz : gz;
+        const bool z_high = from_top ? (r < 0.0) : (r > 0.0);
+        if (z_high) hi = z; else lo = z;
+        double zn = d != 0.0 ? z - r / d : 0.5 * (lo + hi);
+        if (!(zn > lo && zn < hi)) zn = 0.5 * (lo + hi);
+        const double step = fabs(zn - z);
+        z = zn;
+        if (step <= 1e-15 * (1.0 + fabs(z)) || hi - lo <= 1e-15 * (1.0 + fabs(z))) break;
+    }
+    return z;
+}
+
+// Table nodes, SL lanes each: rows 0..120 emission (ln y), 121..221 pair (ln delta).
 constexpr int ST = 64;
-__global__ void __launch_bounds__(ST) k_solve_nodes(const GlRule gl, const BesselWork *W, double *em64, double *pair64) {
-    const int row = blockIdx.y, j = blockIdx.x * ST + threadIdx.x;
-    const bool pair = row >= ROW_PAIR;
-    const int ns = pair ? PAIR_NS : EM_NS, np = pair ? PZ_NP : EZ_NP;
-    if (j >= ns) return;
+__global__ void __launch_bounds__(ST) k_icdf_nodes(const TableWork *W, double *em64, double *pair64) {
+    __shared__ TableShared S;
+    load_shared(S, W);
+    const bool pair = blockIdx.y >= EM_NCHI;
+    const int row = pair ? blockIdx.y - EM_NCHI : blockIdx.y;
+    const int np = pair ? PZ_NP : EZ_NP;
     const double zlo = pair ? PZ_LO : EZ_LO, wp = pair ? PZ_W : EZ_W;
-    const double *below = W->below + (size_t)row * (EZ_NP + 1), *above = W->above + (size_t)row * (EZ_NP + 1);
-    const double chi = W->chi[row], c = 2.0 / (3.0 * chi), lnc = pair ? log(c) : 0.0;
+    const double chi = W->chi[blockIdx.y];
+    const double *mass = W->mass + (size_t)blockIdx.y * EZ_NP;
+    const double *below = W->below + (size_t)blockIdx.y * (EZ_NP + 1), *above = W->above + (size_t)blockIdx.y * (EZ_NP + 1);
+    const double tail = below[0];
+    const double total = pair ? 2.0 * below[np] : below[np];
+    const int ns = pair ? PAIR_NS : EM_NS;
+    const int j = (blockIdx.x * ST + threadIdx.x) / SL;
+    if (j >= ns) return;                            // all lanes of a node alike
     const double s = pair ? -16.0 + 16.0 * j / (PAIR_NS - 1) : -16.0 + 32.0 * j / (EM_NS - 1);
     const double u = 1.0 / (1.0 + exp(-s)), v = 1.0 / (1.0 + exp(s));
-    const double tail = below[0];                       // 0 for pairs
-    const double total = pair ? 2.0 * below[np] : below[np];
-    const bool low = pair || u <= 0.5;
-    double target = (low ? u : v) * total;
-    double z;
-    if (low && target <= tail) {
+    const bool top = !(pair || u <= 0.5);
+    double target = (top ? v : u) * total, z;
+    if (!top && target <= tail) {
         z = zlo + 3.0 * log(target / tail);
     } else {
         int a = 0, b = np - 1;
         while (a < b) {
-            if (low) {                                  // first panel with below[p + 1] >= target
+            if (!top) {                             // first panel with below[p+1] >= target
                 const int m = (a + b) >> 1;
                 if (below[m + 1] < target) a = m + 1; else b = m;
-            } else {                                    // last panel with above[p] >= target
+            } else {                                // last panel with above[p] >= target
                 const int m = (a + b + 1) >> 1;
                 if (above[m] >= target) a = m; else b = m - 1;
             }
         }
-        const double za = zlo + a * wp, zb = zlo + (a + 1) * wp;
-        target -= low ? below[a] : above[a + 1];
-        const double whole = W->mass[(size_t)row * EZ_NP + a];
-        const double f = whole > 0.0 ? fmin(fmax(target / whole, 0.0), 1.0) : 0.5;
-        z = low ? za + f * (zb - za) : zb - f * (zb - za);
-        double lo = za, hi = zb;
-        for (int it = 0; it < 100; ++it) {
-            const double e0 = low ? za : z, hw = 0.5 * (low ? z - za : zb - z);
-            double r = 0.0;
-            for (int i = 0; i < GLN; ++i) {
-                const double x = e0 + hw * (1.0 + gl.x[i]);
-                r += gl.w[i] * (pair ? pair_density(W->bc, c, lnc, x) : em_density(W->bc, chi, a, x));
-            }
-            r = r * hw - target;
-            if (!low) r = -r;                           // increasing in z from either end
-            const double d = pair ? pair_density(W->bc, c, lnc, z) : em_density(W->bc, chi, a, z);
-            if (r > 0.0) hi = z; else lo = z;
-            double zn = d != 0.0 ? z - r / d : 0.5 * (lo + hi);
-            const bool newton = zn >= lo && zn <= hi;
-            if (!newton) zn = 0.5 * (lo + hi);
-            const double step = fabs(zn - z);
-            z = zn;
-            if ((newton && step <= 1e-9) || hi - lo <= 1e-15 * (1.0 + fabs(z))) break;
-        }
+        target = top ? __dsub_rn(target, above[a + 1]) : __dsub_rn(target, below[a]);
+        z = solve_panel(S, pair, chi, zlo + a * wp, zlo + (a + 1) * wp, mass[a], target, top);
     }
-    if (pair) pair64[(size_t)(row - ROW_PAIR) * PAIR_NS + j] = -log1p(exp(-z));
+    if (threadIdx.x % SL) return;
+    if (pair) pair64[(size_t)row * PAIR_NS + j] = -log1p(exp(-z));
     else em64[(size_t)row * EM_NS + j] = z;
 }
 
@@ -444,21 +400,29 @@ __global__ void k_to_f32(const double *a, float *b, int n) {
 qed_status sfq_build_tables(qed_ctx *ctx) {
     using namespace sfq;
     cudaStream_t st = ctx->stream;
-    BesselWork *W = nullptr;
-    SFQ_CUDA(cudaMallocAsync(&W, sizeof(BesselWork), st));
-    const GlRule gl = gauss_legendre();
-    k_bessel_panels<<<EZ_NP, BT, 0, st>>>(gl, W);
-    k_panel_masses<<<dim3((EZ_NP + MT - 1) / MT, ROWS), MT, 0, st>>>(W);
-    k_row_sums<<<ROWS, 64, 0, st>>>(W);
-    k_cheb_coef<<<1, 128, 0, st>>>(W->fnode, ctx->coef64);
+    const bool fp32 = ctx->cfg.precision == QED_FP32;
+    void *work = nullptr;
+    SFQ_CUDA(cudaMallocAsync(&work, fp32 ? sfq_tables32_bytes() : sizeof(TableWork), st));
+    const double *fnode;
+    if (fp32) {
+        fnode = sfq_tables32(work, ctx->icdf_em64, ctx->icdf_pair64, st);
+    } else {
+        TableWork *W = static_cast<TableWork *>(work);
+        fnode = W->fnode;
+        k_table_constants<<<(ROWS + TT - 1) / TT, TT, 0, st>>>(W);
+        k_emission_nodes<<<(EZ_NP * GLN + TT - 1) / TT, TT, 0, st>>>(W);
+        k_panel_masses<<<dim3((EZ_NP + TT - 1) / TT, ROWS), TT, 0, st>>>(W);
+        k_row_sums<<<ROWS, TT, 0, st>>>(W);
+        k_icdf_nodes<<<dim3((EM_NS * SL + ST - 1) / ST, EM_NCHI + PAIR_NCHI), ST, 0, st>>>(W, ctx->icdf_em64,
+                                                                                           ctx->icdf_pair64);
+    }
+    k_cheb_coef<<<1, 128, 0, st>>>(fnode, ctx->coef64);
     k_rate_segments<<<1, 256, 0, st>>>(ctx->coef64, ctx->coef32);
-    k_solve_nodes<<<dim3((EM_NS + ST - 1) / ST, EM_NCHI + PAIR_NCHI), ST, 0, st>>>(gl, W, ctx->icdf_em64,
-                                                                                   ctx->icdf_pair64);
     k_to_f32<<<(EM_NCHI * EM_NS + 255) / 256, 256, 0, st>>>(ctx->icdf_em64, ctx->icdf_em32, EM_NCHI * EM_NS);
     k_to_f32<<<(PAIR_NCHI * PAIR_NS + 255) / 256, 256, 0, st>>>(ctx->icdf_pair64, ctx->icdf_pair32,
                                                                 PAIR_NCHI * PAIR_NS);
     SFQ_CUDA(cudaGetLastError());
-    SFQ_CUDA(cudaFreeAsync(W, st));
+    SFQ_CUDA(cudaFreeAsync(work, st));
     SFQ_CUDA(cudaStreamSynchronize(st));
     return QED_OK;
 }
