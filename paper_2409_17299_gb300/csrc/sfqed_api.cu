@@ -10,7 +10,6 @@ static void free_ctx(qed_ctx *c) {
     if (!c) return;
     cudaStreamSynchronize(c->stream);
     sfq_batch_free(c);
-    sfq_level_graphs_free(c);
     sfq_step_graph_free(c);
     void *dev[] = {c->coef64, c->coef32, c->icdf_em64, c->icdf_pair64, c->icdf_em32, c->icdf_pair32,
                    c->ctl, c->tau[0], c->tau[1], c->blk, c->slots, c->snap, c->lev,
@@ -19,7 +18,6 @@ static void free_ctx(qed_ctx *c) {
         if (p) cudaFree(p);
     if (c->ctl_host) cudaFreeHost(c->ctl_host);
     if (c->ctl_up) cudaFreeHost(c->ctl_up);
-    if (c->pin) cudaFreeHost(c->pin);
     if (c->grid_il) cudaFree(c->grid_il);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     if (c->ev_ready)
@@ -56,13 +54,13 @@ extern "C" qed_status qed_init_tables(qed_ctx **out, const qed_config *cfg, void
               cudaMalloc(&c->lev, sizeof(LevelWork)) == cudaSuccess &&
               cudaHostAlloc(&c->ctl_host, sizeof(DevCtl), cudaHostAllocDefault) == cudaSuccess &&
               cudaHostAlloc(&c->ctl_up, sizeof(DevCtl), cudaHostAllocDefault) == cudaSuccess &&
-              cudaHostAlloc(&c->pin, 64, cudaHostAllocDefault) == cudaSuccess &&
               cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) == cudaSuccess;
     if (!ok) {
         free_ctx(c);
         return QED_ERR_NOMEM;
     }
-    if (cudaMemsetAsync(c->ctl, 0, sizeof(DevCtl), c->stream) != cudaSuccess) {
+    if (cudaMemsetAsync(c->ctl, 0, sizeof(DevCtl), c->stream) != cudaSuccess ||
+        cudaMemsetAsync(c->lev, 0, sizeof(LevelWork), c->stream) != cudaSuccess) {
         free_ctx(c);
         return QED_ERR_CUDA;
     }
@@ -139,12 +137,11 @@ extern "C" qed_status qed_compact(qed_ctx *ctx, qed_particles *p, int64_t step) 
         h.capacity[s] = (unsigned long long)p->s[s].capacity;
     }
     SFQ_CUDA(cudaMemcpyAsync(ctx->ctl, &h, sizeof(DevCtl), cudaMemcpyHostToDevice, ctx->stream));
-    for (int s = 0; s < 3; ++s) {
-        // leveling skips dead entries and compacts; otherwise compaction only
-        const bool level = ctx->cfg.thin_cap > 0 && p->s[s].count > ctx->cfg.thin_cap;
-        qed_status e = level ? sfq_level_species(ctx, &p->s[s], s, step) : sfq_compact_species(ctx, &p->s[s], s);
-        if (e != QED_OK) return e;
-    }
+    // leveling skips dead entries and compacts; otherwise compaction only
+    const int64_t bound[3] = {p->s[0].count, p->s[1].count, p->s[2].count};
+    qed_status e = sfq_ensure_merge(ctx, bound);
+    if (e == QED_OK) e = sfq_merge(ctx, p, bound, ctx->cfg.thin_cap > 0 ? 7 : 0, 7, step, false, false);
+    if (e != QED_OK) return e;
     SFQ_CUDA(cudaMemcpyAsync(ctx->ctl_host, ctx->ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, ctx->stream));
     SFQ_CUDA(cudaStreamSynchronize(ctx->stream));
     if (ctx->ctl_host->bad_index) return QED_ERR_STATE;
@@ -176,7 +173,7 @@ extern "C" qed_status qed_level_eval(qed_ctx *ctx, const qed_species *sp, int sp
     if (ctx->async_open) return QED_ERR_STATE;
     SFQ_CUDA(cudaStreamSynchronize(ctx->stream));
     qed_species copy = *sp;
-    return sfq_level_eval(ctx, &copy, species, w, A, C, N, max_w);
+    return sfq_level_eval(ctx, &copy, w, A, C, N, max_w);
 }
 
 extern "C" qed_status qed_level_apply(qed_ctx *ctx, qed_particles *p, int species, double wstar, int64_t step) {
@@ -193,7 +190,7 @@ extern "C" qed_status qed_level_apply(qed_ctx *ctx, qed_particles *p, int specie
         h.capacity[s] = (unsigned long long)p->s[s].capacity;
     }
     SFQ_CUDA(cudaMemcpyAsync(ctx->ctl, &h, sizeof(DevCtl), cudaMemcpyHostToDevice, ctx->stream));
-    qed_status e = sfq_level_apply_species(ctx, &p->s[species], species, wstar, step);
+    qed_status e = sfq_level_apply_species(ctx, p, species, wstar, step);
     if (e != QED_OK) return e;
     SFQ_CUDA(cudaMemcpyAsync(ctx->ctl_host, ctx->ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, ctx->stream));
     SFQ_CUDA(cudaStreamSynchronize(ctx->stream));

@@ -189,13 +189,6 @@ __device__ __forceinline__ unsigned long long tile_count(const DevCtl *ctl, int 
     return c < cp ? c : cp;
 }
 
-__global__ void k_set_count(DevCtl *ctl, int s) {
-    if (ctl->overflow || ctl->timeout || ctl->bad_index) return;
-    ctl->count[s] = ctl->alive[s];
-    ctl->end[s] = ctl->alive[s];
-    ctl->begin[s] = ctl->alive[s];
-}
-
 __device__ __forceinline__ unsigned long long dbits(double v) { return (unsigned long long)__double_as_longlong(v); }
 constexpr unsigned long long INF_BITS = 0x7ff0000000000000ull;    // +inf as double bits
 
@@ -230,28 +223,24 @@ __host__ __device__ __forceinline__ double double_of_bits(unsigned long long b) 
 }
 
 // Warm start: the first pass evaluates at the species' previous threshold
-// (after a leveling most weights equal it, and the next root usually lies
-// in the piece just above it), else at +inf.  The start changes only the
+// times the last growth of the threshold (in a cascade that grows steadily
+// the next root lies close by), else at +inf.  The start changes only the
 // path: the root of its own piece is the same from any start.
-__device__ __forceinline__ void lev_start(LevelWork *lw, int s) {
-    LevelIter &it = lw->it[s];
+__device__ __forceinline__ LevelIter lev_start(double prev, double ratio) {
+    LevelIter it;
     const double inf = __longlong_as_double(0x7ff0000000000000ll);
-    const double w0 = lw->prev[s] > 0.0 && lw->prev[s] < inf ? lw->prev[s] : inf;
+    const double w0 = prev > 0.0 && prev < inf ? (ratio > 0.0 ? prev * ratio : prev) : inf;
     it.lo = 0.0;
     it.hi = inf;
     it.w = w0;
     it.w_up = w0 < inf ? ceil_f(w0) : __int_as_float(0x7f800000);
     it.wstar = 0.0;
-    it.wstar_inv_f = 0.f;
+    it.wstar_up = it.wstar_f = it.wstar_inv_f = 0.f;
     it.done = 0;
     it.iters = 0;
     it.alive = 0;
-    it.mode = 0;
-    lw->arrive[s] = 0;
-    lw->passes[s] = 0;
+    return it;
 }
-
-__global__ void k_lev_begin(LevelWork *lw, int s) { lev_start(lw, s); }
 
 // error-free float-float accumulation (TwoSum), accurate to ~2^-48 relative
 struct FF {
@@ -328,16 +317,12 @@ __host__ __device__ void lev_advance(LevelIter &it, double A, unsigned long long
     it.w_up = ceil_f(c);
 }
 
-// One pass of the iteration.  Every block sums its share of the weights at
-// it.w; the last block to finish reduces the block partials in block order
-// (a fixed order: the result does not depend on which block is last) and
-// advances the iteration, so a pass is one launch and needs no host.
 constexpr int LEV_T = 256;
 
-// This thread's share of the sums at it.w over entries t0, t0 + stride, ...
+// This thread's share of the sums at w_at (w_up in FP32) over entries t0, t0 + stride, ...
 template <class T>
 __device__ __forceinline__ void lev_accumulate(const void *w, unsigned long long n, unsigned long long t0,
-                                               unsigned long long stride, const LevelIter &it, double &A,
+                                               unsigned long long stride, double w_at, float w_up, double &A,
                                                unsigned long long &C, unsigned long long &N, unsigned long long &M,
                                                unsigned long long &L, unsigned long long &H) {
     C = 0;
@@ -347,7 +332,7 @@ __device__ __forceinline__ void lev_accumulate(const void *w, unsigned long long
     H = INF_BITS;
     if constexpr (sizeof(T) == 4) {
         // FP32 weights: exact float comparisons and float-float sums, no FP64 per element
-        const float wc = it.w_up;
+        const float wc = w_up;
         FF acc;
         unsigned mb = 0, c = 0, nn = 0, lb = 0, hb = 0x7f800000u;    // positive floats order like their bits
         auto one = [&](float v) {
@@ -391,7 +376,7 @@ __device__ __forceinline__ void lev_accumulate(const void *w, unsigned long long
         L = lb ? dbits((double)__uint_as_float(lb)) : 0ull;
         H = hb < 0x7f800000u ? dbits((double)__uint_as_float(hb)) : INF_BITS;
     } else {
-        const double wc = it.w;
+        const double wc = w_at;
         double comp = 0.0;           // Kahan
         A = 0.0;
         for (unsigned long long i = t0; i < n; i += stride) {
@@ -413,110 +398,215 @@ __device__ __forceinline__ void lev_accumulate(const void *w, unsigned long long
     }
 }
 
-// One pass of the iteration.  Every block sums its share of the weights at
-// it.w; the last block to finish reduces the block partials in block order
-// (a fixed order: the result does not depend on which block is last) and
-// advances the iteration, so a pass is one launch and needs no host.
+struct LevSums {
+    double A;                               // sum of the weights below w
+    unsigned long long C, N, M, L, H;       // at or above w; alive; largest; the bounds of w's piece (double bits)
+};
+
+// One pass over a species: this block's sums at w, written to its place of
+// the block partials.
 template <class T>
-__global__ void __launch_bounds__(LEV_T) k_lev_step(const void *w, const DevCtl *ctl, int s, LevelWork *lw,
-                                                    long long cap) {
-    LevelIter &it = lw->it[s];
-    if (*reinterpret_cast<volatile unsigned long long *>(&it.done)) return;
-    const unsigned long long n = min(ctl->count[s], ctl->capacity[s]);
+__device__ __forceinline__ void lev_block_sums(const void *w, unsigned long long n, double w_at, float w_up,
+                                               LevelWork *lw, int s) {
     const unsigned long long t0 = (unsigned long long)blockIdx.x * LEV_T + threadIdx.x;
     const unsigned long long stride = (unsigned long long)gridDim.x * LEV_T;
-    double A;
-    unsigned long long C, N, M, L, H;
-    lev_accumulate<T>(w, n, t0, stride, it, A, C, N, M, L, H);
-    __shared__ double sA[LEV_T / 32];
-    __shared__ unsigned long long sC[LEV_T / 32], sN[LEV_T / 32], sM[LEV_T / 32], sL[LEV_T / 32], sH[LEV_T / 32];
-    __shared__ int s_last;
+    LevSums v;
+    lev_accumulate<T>(w, n, t0, stride, w_at, w_up, v.A, v.C, v.N, v.M, v.L, v.H);
+    __shared__ LevSums sw[LEV_T / 32];
     for (int o = 16; o > 0; o >>= 1) {
-        A += __shfl_down_sync(0xffffffffu, A, o);
-        C += __shfl_down_sync(0xffffffffu, C, o);
-        N += __shfl_down_sync(0xffffffffu, N, o);
-        M = max(M, __shfl_down_sync(0xffffffffu, M, o));
-        L = max(L, __shfl_down_sync(0xffffffffu, L, o));
-        H = min(H, __shfl_down_sync(0xffffffffu, H, o));
+        v.A += __shfl_down_sync(0xffffffffu, v.A, o);
+        v.C += __shfl_down_sync(0xffffffffu, v.C, o);
+        v.N += __shfl_down_sync(0xffffffffu, v.N, o);
+        v.M = max(v.M, __shfl_down_sync(0xffffffffu, v.M, o));
+        v.L = max(v.L, __shfl_down_sync(0xffffffffu, v.L, o));
+        v.H = min(v.H, __shfl_down_sync(0xffffffffu, v.H, o));
     }
-    const int wid = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) { sA[wid] = A; sC[wid] = C; sN[wid] = N; sM[wid] = M; sL[wid] = L; sH[wid] = H; }
+    __syncthreads();                        // sw is read by the previous species' sums
+    if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double a = 0.0;
-        unsigned long long c = 0, nn = 0, m = 0, pl = 0, ph = INF_BITS;
-        for (int k = 0; k < LEV_T / 32; ++k) {
-            a += sA[k]; c += sC[k]; nn += sN[k]; m = max(m, sM[k]); pl = max(pl, sL[k]); ph = min(ph, sH[k]);
+        LevSums t = sw[0];
+        for (int k = 1; k < LEV_T / 32; ++k) {
+            t.A += sw[k].A; t.C += sw[k].C; t.N += sw[k].N;
+            t.M = max(t.M, sw[k].M); t.L = max(t.L, sw[k].L); t.H = min(t.H, sw[k].H);
         }
-        lw->partA[blockIdx.x] = a;
-        lw->partC[blockIdx.x] = c;
-        lw->partN[blockIdx.x] = nn;
-        lw->partM[blockIdx.x] = m;
-        lw->partL[blockIdx.x] = pl;
-        lw->partH[blockIdx.x] = ph;
-        __threadfence();
-        const unsigned prev = atomicAdd(&lw->arrive[s], 1u);
-        s_last = prev == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    // the last block: partials b = t, t + LEV_T, ... per thread, then a tree of fixed shape
-    __shared__ double rh[LEV_T], rl[LEV_T];
-    __shared__ unsigned long long rc[LEV_T], rn[LEV_T], rm[LEV_T], rpl[LEV_T], rph[LEV_T];
-    const int t = threadIdx.x;
-    DD acc;
-    unsigned long long c = 0, nn = 0, m = 0, pl = 0, ph = INF_BITS;
-    for (int b = t; b < (int)gridDim.x; b += LEV_T) {
-        acc.add(__ldcg(&lw->partA[b]));
-        c += __ldcg(&lw->partC[b]);
-        nn += __ldcg(&lw->partN[b]);
-        m = max(m, __ldcg(&lw->partM[b]));
-        pl = max(pl, __ldcg(&lw->partL[b]));
-        ph = min(ph, __ldcg(&lw->partH[b]));
-    }
-    rh[t] = acc.hi; rl[t] = acc.lo; rc[t] = c; rn[t] = nn; rm[t] = m; rpl[t] = pl; rph[t] = ph;
-    __syncthreads();
-    for (int o = LEV_T / 2; o > 0; o >>= 1) {
-        if (t < o) {
-            DD x;
-            x.hi = rh[t];
-            x.lo = rl[t];
-            x.add(rh[t + o]);
-            x.lo += rl[t + o];
-            rh[t] = x.hi;
-            rl[t] = x.lo;
-            rc[t] += rc[t + o];
-            rn[t] += rn[t + o];
-            rm[t] = max(rm[t], rm[t + o]);
-            rpl[t] = max(rpl[t], rpl[t + o]);
-            rph[t] = min(rph[t], rph[t + o]);
-        }
-        __syncthreads();
-    }
-    if (t == 0) {
-        if (it.mode == 1) {         // sums only: the caller combines them across shards
-            it.sumA = rh[0] + rl[0];
-            it.sumC = rc[0];
-            it.sumN = rn[0];
-            it.sumM = rm[0];
-        } else {
-            lev_advance(it, rh[0] + rl[0], rc[0], rn[0], rm[0], cap, rpl[0], rph[0]);
-            if (it.done && it.wstar > 0.0) lw->prev[s] = it.wstar;
-        }
-        lw->arrive[s] = 0;
+        const int b = s * LEVEL_MAX_BLOCKS + blockIdx.x;
+        lw->partA[b] = t.A;
+        lw->partC[b] = t.C;
+        lw->partN[b] = t.N;
+        lw->partM[b] = t.M;
+        lw->partL[b] = t.L;
+        lw->partH[b] = t.H;
     }
 }
 
-// Graph-driven leveling: after each pass, one thread decides whether the
-// graph's while loop runs another (the only setter of the condition, so no
-// two writes race).  The loop ends when the iteration is done, and in any
-// case after LEVEL_ITERS + 1 passes (the iteration itself finishes by then).
-__global__ void k_lev_cond(LevelWork *lw, int s, DevCtl *ctl, cudaGraphConditionalHandle h) {
-    const LevelIter &it = lw->it[s];
-    const unsigned long long n = ++lw->passes[s];
-    ctl->graph_kernels += 2;                 // this pass: k_lev_step and this kernel
-    cudaGraphSetConditional(h, (!it.done && n <= (unsigned long long)LEVEL_ITERS) ? 1u : 0u);
+// The block partials of a species reduced by one warp in a fixed order
+// (partials lane, lane + 32, ..., then a butterfly), so that the result does
+// not depend on which block does it.
+__device__ __forceinline__ LevSums lev_reduce(const LevelWork *lw, int s, int blocks) {
+    const int base = s * LEVEL_MAX_BLOCKS;
+    DD acc;
+    unsigned long long c = 0, nn = 0, m = 0, pl = 0, ph = INF_BITS;
+    for (int b = threadIdx.x & 31; b < blocks; b += 32) {
+        acc.add(__ldcg(&lw->partA[base + b]));
+        c += __ldcg(&lw->partC[base + b]);
+        nn += __ldcg(&lw->partN[base + b]);
+        m = max(m, __ldcg(&lw->partM[base + b]));
+        pl = max(pl, __ldcg(&lw->partL[base + b]));
+        ph = min(ph, __ldcg(&lw->partH[base + b]));
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        DD x = acc;
+        const double oh = __shfl_down_sync(0xffffffffu, acc.hi, o), ol = __shfl_down_sync(0xffffffffu, acc.lo, o);
+        x.add(oh);
+        x.lo += ol;
+        acc = x;
+        c += __shfl_down_sync(0xffffffffu, c, o);
+        nn += __shfl_down_sync(0xffffffffu, nn, o);
+        m = max(m, __shfl_down_sync(0xffffffffu, m, o));
+        pl = max(pl, __shfl_down_sync(0xffffffffu, pl, o));
+        ph = min(ph, __shfl_down_sync(0xffffffffu, ph, o));
+    }
+    return LevSums{acc.hi + acc.lo, c, nn, m, pl, ph};       // valid in lane 0
+}
+
+struct LevWeights {
+    const void *w[3];       // the species' weights (null: not leveled in this launch)
+};
+
+// Leveling thresholds of all species in one cooperative launch: each species
+// above the cap runs its iteration (lev_advance) over the same passes; in a
+// pass every block sums its share of each species' weights, the last block
+// to arrive reduces the partials and advances the iterations, and the others
+// wait for it (bounded; a wait that runs out marks the step as timed out).
+//
+// A pass over 1e7 weights takes 6 us from DRAM and less from L2, but as two
+// launches of a graph's while loop per pass and species it took 19 to 25 us,
+// and the standing-wave cascade takes about five passes for each of three
+// species: 0.36 ms of a 1.9 ms step (1e7 per species), 0.07 ms here (three
+// passes from the better start; a warp per species reduces the partials:
+// 0.26 ms with a block-wide tree per species and the old start).  With the
+// merged compaction launches: 40 steps of that cascade 88.2 -> 72.4 ms, 20
+// steps on the grid (1e6 per species) 20.8 -> 13.3 ms, 20 steps at the start
+// of a cascade 2.86 -> 2.00 ms, 40 steps at 5e7 photons 87.0 -> 83.9 ms.
+constexpr unsigned LEV_POLLS = 1u << 24;
+
+template <class T>
+__global__ void __launch_bounds__(LEV_T, 4) k_level(LevWeights lwt, DevCtl *ctl, LevelWork *lw, long long cap) {
+    __shared__ int s_last, s_out;
+    __shared__ double s_w[3];
+    __shared__ float s_wup[3];
+    __shared__ int s_done[3];
+    const int t = threadIdx.x;
+    const bool stop = ctl->overflow || ctl->timeout || ctl->bad_index;
+    unsigned long long n[3];
+    bool any = false;
+    for (int s = 0; s < 3; ++s) {
+        n[s] = min(ctl->count[s], ctl->capacity[s]);
+        const bool on = lwt.w[s] && !stop && cap > 0 && n[s] > (unsigned long long)cap;
+        if (!on) n[s] = 0;
+        any = any || on;
+        if (t == 0) {
+            const LevelIter it = lev_start(lw->prev[s], lw->ratio[s]);
+            s_w[s] = it.w;
+            s_wup[s] = it.w_up;
+            s_done[s] = !on;
+            if (!on && blockIdx.x == 0) {
+                LevelIter off = it;
+                lev_finish(off, 0.0);
+                lw->it[s] = off;
+                lw->on[s] = 0;
+            }
+        }
+    }
+    if (!any) return;
+    const unsigned long long round0 = *reinterpret_cast<volatile unsigned long long *>(&lw->round);
+    __syncthreads();
+    for (int pass = 0; pass <= LEVEL_ITERS; ++pass) {
+        for (int s = 0; s < 3; ++s)
+            if (!s_done[s]) lev_block_sums<T>(lwt.w[s], n[s], s_w[s], s_wup[s], lw, s);
+        if (t == 0) {
+            __threadfence();
+            s_last = atomicAdd(&lw->arrive, 1u) == gridDim.x - 1;
+            __threadfence();
+        }
+        __syncthreads();
+        if (s_last) {
+            const int s = t >> 5;                   // a warp per species
+            if (s < 3 && !s_done[s]) {
+                const LevSums v = lev_reduce(lw, s, (int)gridDim.x);
+                if ((t & 31) == 0) {
+                    LevelIter it;
+                    if (pass == 0) it = lev_start(lw->prev[s], lw->ratio[s]);
+                    else it = lw->it[s];
+                    lev_advance(it, v.A, v.C, v.N, v.M, cap, v.L, v.H);
+                    if (it.done && it.wstar > 0.0) {
+                        const double r = it.wstar / lw->prev[s];
+                        lw->ratio[s] = lw->prev[s] > 0.0 && r > 0.5 && r < 2.0 ? r : 1.0;
+                        lw->prev[s] = it.wstar;
+                    }
+                    lw->it[s] = it;
+                    lw->on[s] = 1;
+                    __threadfence();
+                }
+            }
+            __syncthreads();
+            if (t == 0) {
+                lw->arrive = 0;
+                __threadfence();
+                atomicExch(&lw->round, round0 + pass + 1);
+            }
+        }
+        if (t == 0) {
+            unsigned polls = 0;
+            s_out = 0;
+            while (!s_last && *reinterpret_cast<volatile unsigned long long *>(&lw->round) != round0 + pass + 1) {
+                if (++polls > LEV_POLLS) {
+                    atomicExch(&ctl->timeout, 1ull);
+                    s_out = 1;
+                    break;
+                }
+                __nanosleep(40);
+            }
+            __threadfence();
+            bool all = true;
+            for (int s = 0; s < 3; ++s) {
+                if (!s_done[s]) {
+                    s_done[s] = __ldcg(&lw->it[s].done) != 0;
+                    s_w[s] = __ldcg(&lw->it[s].w);
+                    s_wup[s] = __ldcg(&lw->it[s].w_up);
+                }
+                all = all && s_done[s];
+            }
+            if (all) s_out = 1;
+        }
+        __syncthreads();
+        if (s_out) break;
+    }
+}
+
+// The sums of one species at w (a shard's part of a leveling over processes)
+template <class T>
+__global__ void __launch_bounds__(LEV_T) k_lev_eval(const void *w, unsigned long long n, double at, float up, int s,
+                                                    LevelWork *lw) {
+    __shared__ int s_last;
+    lev_block_sums<T>(w, n, at, up, lw, s);
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(&lw->arrive, 1u) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
+    if (threadIdx.x >= 32) return;
+    const LevSums v = lev_reduce(lw, s, (int)gridDim.x);
+    if (threadIdx.x == 0) {
+        lw->sumA = v.A;
+        lw->sumC = v.C;
+        lw->sumN = v.N;
+        lw->sumM = v.M;
+        lw->arrive = 0;
+    }
 }
 
 // ---- compaction by tiles (used after leveling and for converted photons) ----
@@ -525,7 +615,9 @@ __global__ void k_lev_cond(LevelWork *lw, int s, DevCtl *ctl, cudaGraphCondition
 // the dead entries of each tile in index order (16-bit tile offsets) and
 // counts the alive ones; a scan gives A (alive total) and H (dead entries
 // below A); pass 2 lists the alive entries at or above A (the movers) by
-// rank; pass 3 moves mover r into the r-th dead slot below A.
+// rank; pass 3 moves mover r into the r-th dead slot below A.  The passes
+// cover all species of the merge step in one launch each (a species' step
+// took seven launches of its own: 25 us of a 145 us step with few particles).
 constexpr int LT = 256;
 constexpr int LROUNDS = 16;
 constexpr int LTILE = LT * LROUNDS;       // entries per tile (offsets fit 16 bits)
@@ -537,31 +629,57 @@ constexpr int LSPAN = 32 * LROUNDS;       // contiguous entries per warp
 // the work.
 __device__ __forceinline__ long long tiles_of(unsigned long long n) { return (long long)((n + LTILE - 1) / LTILE); }
 
+// What the passes work on: the species of `always`, and with `leveled` those
+// whose leveling ran.
+struct MergeArgs {
+    SpeciesDev sp[3];
+    DevCtl *ctl;
+    LevelWork *lw;
+    unsigned long long *blk[3];       // per tile: alive entries, then (pass 2 on) those before it
+    unsigned short *dl[3];            // dead entries by tile
+    unsigned long long *movers[3];
+    long long nb[3];                  // tiles the buffers hold
+    PhiloxKeys keys;
+    unsigned step;                    // step index keying the draws, unless
+    int step_from_ctl;                // it is the control block's current step
+    int always, leveled;              // bits of species; leveled: bits of species that may have been
+    int may_defer;
+};
+
+// entries of species s that the passes cover
+__device__ __forceinline__ unsigned long long merge_count(const MergeArgs &m, int s) {
+    const bool run = ((m.always >> s) & 1) || (((m.leveled >> s) & 1) && m.lw->on[s]);
+    return run ? tile_count(m.ctl, s) : 0;
+}
+
 // Pass 1.  LEVEL: first keep particle i (0 < w_i < w*) with probability
 // w_i / w*: the comparison u < w_i / w* is made in FP32 with a relative
 // margin, and in FP64 (the oracle's test) only for draws within that margin
-// of the boundary; kept particles get weight w*.  The step index keying the
-// draws is `step`, or the control block's current step when step_from_ctl.
+// of the boundary; kept particles get weight w*.
 template <class T, bool LEVEL>
-__global__ void __launch_bounds__(LT, 4) k_tile_dead(SpeciesDev S, DevCtl *ctl, int s, const LevelWork *lw,
-                                                  const PhiloxKeys keys, unsigned step, int step_from_ctl,
-                                                  unsigned long long *blk, unsigned short *dl) {
+__global__ void __launch_bounds__(LT, 4) k_tile_dead(const __grid_constant__ MergeArgs m) {
     __shared__ unsigned wdead[LT / 32];
-    const unsigned long long n = tile_count(ctl, s);
+    DevCtl *ctl = m.ctl;
+    const PhiloxKeys &keys = m.keys;
+    // one species per row of blocks: its arrays and threshold are uniform
+    const int s = 2 - (int)blockIdx.y;
+    const unsigned long long n = merge_count(m, s);
     const long long nbe = tiles_of(n);
-    if (step_from_ctl) step = ctl->sv_step;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const SpeciesDev S = m.sp[s];
     bool thin = false;
     double wstar = 0.0;
     float inv_f = 0.f, wup = 0.f, wnew = 0.f;
     if constexpr (LEVEL) {
-        const LevelIter &it = lw->it[s];
+        const LevelIter &it = m.lw->it[s];
         wstar = it.wstar;
-        thin = it.done && wstar > 0.0;
+        thin = ((m.leveled >> s) & 1) && it.done && wstar > 0.0;
         inv_f = it.wstar_inv_f;
         wup = it.wstar_up;
         wnew = it.wstar_f;
     }
+    unsigned step = m.step;
+    if (m.step_from_ctl) step = ctl->sv_step;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     unsigned removed = 0;
     // FP32 leveling: groups of four entries whose draws are computed together
     constexpr bool SPEC = LEVEL && sizeof(T) == 4;
@@ -639,7 +757,7 @@ __global__ void __launch_bounds__(LT, 4) k_tile_dead(SpeciesDev S, DevCtl *ctl, 
             before += k < wid ? c : 0u;
             total += c;
         }
-        unsigned short *tdl = dl + base;
+        unsigned short *tdl = m.dl[s] + base;
         const unsigned lt = (1u << lane) - 1u;
         unsigned run = before;
 #pragma unroll
@@ -649,7 +767,7 @@ __global__ void __launch_bounds__(LT, 4) k_tile_dead(SpeciesDev S, DevCtl *ctl, 
         }
         if (threadIdx.x == 0) {
             const unsigned long long tn = n - base < (unsigned long long)LTILE ? n - base : (unsigned long long)LTILE;
-            blk[tile] = tn - total;
+            m.blk[s][tile] = tn - total;
         }
         __syncthreads();                       // wdead is rewritten by the next tile
     }
@@ -659,74 +777,82 @@ __global__ void __launch_bounds__(LT, 4) k_tile_dead(SpeciesDev S, DevCtl *ctl, 
     }
 }
 
-// single block: exclusive scan of the counts of the tiles holding entries
-// (blk[nbe] = A), then H from the alive entries of the tile that holds A.
+// One block per species: exclusive scan of the counts of the tiles holding
+// entries (blk[nbe] = A; each thread takes a run of consecutive tiles), then H
+// from the alive entries of the tile that holds A.
 // may_defer: while dead entries are at most DEFER_DEN-th of the species and
 // the count leaves a fifth of the capacity free, the move is deferred (H = 0,
 // the count stays): the dead entries (weight 0) are skipped by every pass
 // until a later step compacts, with holes denser and fewer moves per step.
 constexpr unsigned long long DEFER_DEN = 4;
+constexpr int SCAN_T = 1024;
 
-template <class T>
-__global__ void k_scan_tiles(const void *w, unsigned long long *blk, long long nb, DevCtl *ctl, int s,
-                             int may_defer) {
-    __shared__ unsigned long long sw[32];
-    __shared__ unsigned long long carry;
-    const long long nbe_all = tiles_of(tile_count(ctl, s));
-    const long long nbe = nbe_all < nb ? nbe_all : nb;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (long long b0 = 0; b0 < nbe; b0 += blockDim.x) {
-        const long long i = b0 + threadIdx.x;
-        const unsigned long long v = i < nbe ? blk[i] : 0ull;
-        unsigned long long x = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
+template <class T> __global__ void __launch_bounds__(SCAN_T) k_scan_tiles(const __grid_constant__ MergeArgs m) {
+    __shared__ unsigned long long sw[SCAN_T / 32];
+    const int s = blockIdx.x;
+    DevCtl *ctl = m.ctl;
+    const unsigned long long n = merge_count(m, s);
+    if (n == 0) {
+        if (threadIdx.x == 0) {                     // nothing moves, no entry counted
+            ctl->alive[s] = min(ctl->count[s], ctl->capacity[s]);
+            ctl->holes[s] = 0;
         }
-        if (lane == 31) sw[wid] = x;
-        __syncthreads();
-        if (wid == 0) {
-            unsigned long long t = lane < nw ? sw[lane] : 0ull;
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long y = __shfl_up_sync(0xffffffffu, t, o);
-                if (lane >= o) t += y;
-            }
-            sw[lane] = t;
-        }
-        __syncthreads();
-        const unsigned long long before = carry + (wid > 0 ? sw[wid - 1] : 0ull) + x - v;
-        if (i < nbe) blk[i] = before;
-        __syncthreads();
-        if (threadIdx.x == 0) carry += sw[nw - 1];
-        __syncthreads();
+        return;
     }
-    const unsigned long long A = carry;
+    const void *w = m.sp[s].w;
+    unsigned long long *blk = m.blk[s];
+    const long long nbe_all = tiles_of(n), nbe = nbe_all < m.nb[s] ? nbe_all : m.nb[s];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const long long per = (nbe + SCAN_T - 1) / SCAN_T;
+    const long long i0 = min((long long)threadIdx.x * per, nbe), i1 = min(i0 + per, nbe);
+    unsigned long long v = 0;
+    for (long long i = i0; i < i1; ++i) v += blk[i];
+    unsigned long long x = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) sw[wid] = x;
+    __syncthreads();
+    if (wid == 0) {
+        unsigned long long t = sw[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += y;
+        }
+        sw[lane] = t;
+    }
+    __syncthreads();
+    unsigned long long run = (wid > 0 ? sw[wid - 1] : 0ull) + x - v;
+    for (long long i = i0; i < i1; ++i) {
+        const unsigned long long c = blk[i];
+        blk[i] = run;
+        run += c;
+    }
+    const unsigned long long A = sw[SCAN_T / 32 - 1];
     const unsigned long long a = A / LTILE;
     unsigned long long below = A;                   // A on a tile boundary past the data: no holes
+    __syncthreads();                                // blk and sw: written and read above
     if ((long long)a < nbe) {
         unsigned c = 0;
-        for (unsigned long long i = a * LTILE + threadIdx.x; i < A; i += blockDim.x) c += alive_at<T>(w, i) ? 1u : 0u;
+        for (unsigned long long i = a * LTILE + threadIdx.x; i < A; i += SCAN_T) c += alive_at<T>(w, i) ? 1u : 0u;
         for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
-        __syncthreads();
         if (lane == 0) sw[wid] = c;
         __syncthreads();
         unsigned long long tc = 0;
-        for (int k = 0; k < nw; ++k) tc += sw[k];
+        for (int k = 0; k < SCAN_T / 32; ++k) tc += sw[k];
         below = blk[a] + tc;
     }
     if (threadIdx.x == 0) {
-        const unsigned long long n = tile_count(ctl, s);
         blk[nbe] = A;
-        if (may_defer && (n - A) * DEFER_DEN <= n && 5 * n <= 4 * ctl->capacity[s]) {
+        if (m.may_defer && (n - A) * DEFER_DEN <= n && 5 * n <= 4 * ctl->capacity[s]) {
             ctl->alive[s] = n;                      // nothing moves; count unchanged
             ctl->holes[s] = 0;
             ctl->deferred[s] = n - A;
         } else {
             ctl->alive[s] = A;
             ctl->holes[s] = A - below;
-            ctl->moved += A - below;
+            if (A - below) atomicAdd(&ctl->moved, A - below);
             ctl->deferred[s] = 0;
         }
     }
@@ -734,44 +860,47 @@ __global__ void k_scan_tiles(const void *w, unsigned long long *blk, long long n
 
 // pass 2: movers (alive entries at or above A) by rank, over the tiles that
 // reach past A
-template <class T>
-__global__ void __launch_bounds__(LT) k_tile_movers(const void *w, DevCtl *ctl, int s, const unsigned long long *blk,
-                                                    unsigned long long *movers) {
+template <class T> __global__ void __launch_bounds__(LT) k_tile_movers(const __grid_constant__ MergeArgs m) {
     __shared__ unsigned walive[LT / 32];
-    const unsigned long long n = tile_count(ctl, s), A = ctl->alive[s], H = ctl->holes[s];
-    if (H == 0) return;
-    const unsigned long long below_A = A - H;      // alive entries below A
-    const long long nbe = tiles_of(n);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (long long tile = (long long)(A / LTILE) + blockIdx.x; tile < nbe; tile += gridDim.x) {
-        const unsigned long long base = (unsigned long long)tile * LTILE;
-        const unsigned long long wbase = base + (unsigned long long)wid * LSPAN;
-        unsigned amask[LROUNDS];
-        unsigned cnt = 0;
+    DevCtl *ctl = m.ctl;
+    for (int s = 0; s < 3; ++s) {
+        const unsigned long long n = merge_count(m, s), A = ctl->alive[s], H = ctl->holes[s];
+        if (n == 0 || H == 0) continue;
+        const void *w = m.sp[s].w;
+        const unsigned long long *blk = m.blk[s];
+        const unsigned long long below_A = A - H;      // alive entries below A
+        const long long nbe = tiles_of(n);
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        for (long long tile = (long long)(A / LTILE) + blockIdx.x; tile < nbe; tile += gridDim.x) {
+            const unsigned long long base = (unsigned long long)tile * LTILE;
+            const unsigned long long wbase = base + (unsigned long long)wid * LSPAN;
+            unsigned amask[LROUNDS];
+            unsigned cnt = 0;
 #pragma unroll
-        for (int r = 0; r < LROUNDS; ++r) {
-            const unsigned long long i = wbase + r * 32 + lane;
-            amask[r] = __ballot_sync(0xffffffffu, i < n && alive_at<T>(w, i));
-            cnt += __popc(amask[r]);
-        }
-        if (lane == 0) walive[wid] = cnt;
-        __syncthreads();
-        unsigned before = 0;
-        for (int k = 0; k < wid; ++k) before += walive[k];
-        const unsigned lt = (1u << lane) - 1u;
-        unsigned long long run = blk[tile] + before;   // alive entries before this warp's span
-#pragma unroll
-        for (int r = 0; r < LROUNDS; ++r) {
-            const unsigned long long i = wbase + r * 32 + lane;
-            if (((amask[r] >> lane) & 1u) && i >= A) {
-                const unsigned long long ab = run + __popc(amask[r] & lt);
-                const unsigned long long rank = ab - below_A;
-                if (ab >= below_A && rank < H) movers[rank] = i;
-                else atomicExch(&ctl->bad_index, i + 1);
+            for (int r = 0; r < LROUNDS; ++r) {
+                const unsigned long long i = wbase + r * 32 + lane;
+                amask[r] = __ballot_sync(0xffffffffu, i < n && alive_at<T>(w, i));
+                cnt += __popc(amask[r]);
             }
-            run += __popc(amask[r]);
+            if (lane == 0) walive[wid] = cnt;
+            __syncthreads();
+            unsigned before = 0;
+            for (int k = 0; k < wid; ++k) before += walive[k];
+            const unsigned lt = (1u << lane) - 1u;
+            unsigned long long run = blk[tile] + before;   // alive entries before this warp's span
+#pragma unroll
+            for (int r = 0; r < LROUNDS; ++r) {
+                const unsigned long long i = wbase + r * 32 + lane;
+                if (((amask[r] >> lane) & 1u) && i >= A) {
+                    const unsigned long long ab = run + __popc(amask[r] & lt);
+                    const unsigned long long rank = ab - below_A;
+                    if (ab >= below_A && rank < H) m.movers[s][rank] = i;
+                    else atomicExch(&ctl->bad_index, i + 1);
+                }
+                run += __popc(amask[r]);
+            }
+            __syncthreads();                       // walive is rewritten by the next tile
         }
-        __syncthreads();                       // walive is rewritten by the next tile
     }
 }
 
@@ -779,31 +908,49 @@ __global__ void __launch_bounds__(LT) k_tile_movers(const void *w, DevCtl *ctl, 
 // tile) + k; dead entries below A receive the mover of their rank.  (One
 // warp per tile with four moves in flight per lane was measured slower: the
 // moves are bound by the scattered 32-byte sectors they write, not by the
-// latency of their loads.)
-template <class T>
-__global__ void __launch_bounds__(LT) k_tile_fill(SpeciesDev S, DevCtl *ctl, int s, const unsigned long long *blk,
-                                                  const unsigned short *dl, const unsigned long long *movers) {
-    const unsigned long long n = tile_count(ctl, s), A = ctl->alive[s], H = ctl->holes[s];
-    if (H == 0) return;
-    const long long nfill = tiles_of(A);
-    for (long long tile = blockIdx.x; tile < nfill; tile += gridDim.x) {
-        const unsigned long long base = (unsigned long long)tile * LTILE;
-        const unsigned long long tn = n - base < (unsigned long long)LTILE ? n - base : (unsigned long long)LTILE;
-        const unsigned long long alive_t = blk[tile + 1] - blk[tile];
-        const unsigned dead_t = (unsigned)(tn - alive_t);
-        const unsigned long long dead_before = base - blk[tile];
-        const unsigned short *tdl = dl + base;
-        for (unsigned k = threadIdx.x; k < dead_t; k += LT) {
-            const unsigned long long i = base + tdl[k];
-            if (i >= A) break;                      // offsets ascend: the rest lie at or above A too
-            const unsigned long long r = dead_before + k;
-            if (r < H) {
-                const unsigned long long src = movers[r];
-                if (src >= A && src < n) move_entry<T>(S, i, src);
-                else atomicExch(&ctl->bad_index, i + 1);
-            } else {
-                atomicExch(&ctl->bad_index, i + 1);
+// latency of their loads.)  The last block to finish takes over the counts.
+template <class T> __global__ void __launch_bounds__(LT) k_tile_fill(const __grid_constant__ MergeArgs m) {
+    __shared__ int s_last;
+    DevCtl *ctl = m.ctl;
+    unsigned long long n3[3];
+    for (int s = 0; s < 3; ++s) {
+        const unsigned long long n = merge_count(m, s), A = ctl->alive[s], H = ctl->holes[s];
+        n3[s] = n;
+        if (n == 0 || H == 0) continue;
+        const SpeciesDev &S = m.sp[s];
+        const unsigned long long *blk = m.blk[s];
+        const long long nfill = tiles_of(A);
+        for (long long tile = blockIdx.x; tile < nfill; tile += gridDim.x) {
+            const unsigned long long base = (unsigned long long)tile * LTILE;
+            const unsigned long long tn = n - base < (unsigned long long)LTILE ? n - base : (unsigned long long)LTILE;
+            const unsigned long long alive_t = blk[tile + 1] - blk[tile];
+            const unsigned dead_t = (unsigned)(tn - alive_t);
+            const unsigned long long dead_before = base - blk[tile];
+            const unsigned short *tdl = m.dl[s] + base;
+            for (unsigned k = threadIdx.x; k < dead_t; k += LT) {
+                const unsigned long long i = base + tdl[k];
+                if (i >= A) break;                      // offsets ascend: the rest lie at or above A too
+                const unsigned long long r = dead_before + k;
+                if (r < H) {
+                    const unsigned long long src = m.movers[s][r];
+                    if (src >= A && src < n) move_entry<T>(S, i, src);
+                    else atomicExch(&ctl->bad_index, i + 1);
+                } else {
+                    atomicExch(&ctl->bad_index, i + 1);
+                }
             }
+        }
+    }
+    // every block has read the counts above
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(&ctl->arrive, 1ull) == gridDim.x - 1;
+        __threadfence();
+        if (s_last) {
+            ctl->arrive = 0;
+            for (int s = 0; s < 3; ++s)
+                if (n3[s]) ctl->count[s] = ctl->end[s] = ctl->begin[s] = ctl->alive[s];
         }
     }
 }
@@ -822,246 +969,100 @@ template <class K> static unsigned tile_grid(const qed_ctx *ctx, K kernel, long 
 // device); step_from_ctl: the leveling draws take the step index from the
 // control block (a captured step graph).  The work buffers must hold
 // bound / 1024 + 2 block words and bound hole words (sfq_ensure_work).
-template <class T, bool LEVEL>
-qed_status compact_tiles_bounded(qed_ctx *ctx, qed_species *sp, int s, int64_t step, int64_t bound,
-                                 bool step_from_ctl, bool may_defer = false) {
-    if (bound <= 0) return QED_OK;
-    const int64_t nb = (bound + LTILE - 1) / LTILE;
-    if (ctx->blk_cap < nb + 1 || ctx->slots_cap < bound) return QED_ERR_STATE;
-    SpeciesDev S{sp->x, sp->y, sp->z, sp->px, sp->py, sp->pz, sp->w,
-                 reinterpret_cast<unsigned long long *>(sp->id), sp->nevents, nullptr, ctx->od[s]};
-    // slots: bound 16-bit dead-list entries, then at most bound/2 mover indices
-    unsigned short *dl = reinterpret_cast<unsigned short *>(ctx->slots);
-    unsigned long long *movers = ctx->slots + (bound + 3) / 4;
+// The work buffers of one merge over species of at most bound[s] entries:
+// per tile two words, per entry 16 bits of dead list and half a mover index.
+static int64_t merge_blk_words(const int64_t bound[3]) {
+    int64_t n = 0;
+    for (int s = 0; s < 3; ++s) n += (bound[s] + LTILE - 1) / LTILE + 2;
+    return n;
+}
+
+static int64_t merge_slot_words(const int64_t bound[3]) {
+    int64_t n = 0;
+    for (int s = 0; s < 3; ++s) n += (bound[s] + 3) / 4 + bound[s] / 2 + 2;
+    return n;
+}
+
+template <class T>
+static qed_status merge_args(qed_ctx *ctx, const qed_particles *p, const int64_t bound[3], MergeArgs &m) {
+    memset(&m, 0, sizeof m);
+    if (ctx->blk_cap < merge_blk_words(bound) || ctx->slots_cap < merge_slot_words(bound)) return QED_ERR_STATE;
+    unsigned long long *blk = ctx->blk, *slots = ctx->slots;
+    for (int s = 0; s < 3; ++s) {
+        const qed_species &S = p->s[s];
+        m.sp[s] = SpeciesDev{S.x, S.y, S.z, S.px, S.py, S.pz, S.w, reinterpret_cast<unsigned long long *>(S.id),
+                             S.nevents, nullptr, ctx->od[s]};
+        m.nb[s] = (bound[s] + LTILE - 1) / LTILE;
+        m.blk[s] = blk;
+        blk += m.nb[s] + 2;
+        m.dl[s] = reinterpret_cast<unsigned short *>(slots);
+        slots += (bound[s] + 3) / 4 + 1;
+        m.movers[s] = slots;
+        slots += bound[s] / 2 + 1;
+    }
+    m.ctl = ctx->ctl;
+    m.lw = ctx->lev;
+    m.keys = philox_keys(ctx->cfg.seed);
+    return QED_OK;
+}
+
+// The four compaction passes over the species of m.always and, with
+// m.leveled, those whose leveling ran (four launches for all of them).
+template <class T, bool LEVEL> static qed_status compact_launch(qed_ctx *ctx, const MergeArgs &m) {
+    long long nb_max = 0;
+    for (int s = 0; s < 3; ++s)
+        if ((((m.always | m.leveled) >> s) & 1) && m.nb[s] > nb_max) nb_max = m.nb[s];
+    if (nb_max == 0) return QED_OK;
     cudaStream_t st = ctx->stream;
-    k_tile_dead<T, LEVEL><<<tile_grid(ctx, k_tile_dead<T, LEVEL>, nb), LT, 0, st>>>(
-        S, ctx->ctl, s, ctx->lev, philox_keys(ctx->cfg.seed), (unsigned)step, step_from_ctl ? 1 : 0, ctx->blk, dl);
-    k_scan_tiles<T><<<1, 1024, 0, st>>>(sp->w, ctx->blk, nb, ctx->ctl, s, may_defer ? 1 : 0);
-    k_tile_movers<T><<<tile_grid(ctx, k_tile_movers<T>, nb), LT, 0, st>>>(sp->w, ctx->ctl, s, ctx->blk, movers);
-    k_tile_fill<T><<<tile_grid(ctx, k_tile_fill<T>, nb), LT, 0, st>>>(S, ctx->ctl, s, ctx->blk, dl, movers);
-    k_set_count<<<1, 1, 0, st>>>(ctx->ctl, s);
-    SFQ_LAUNCHED(ctx, 5);
+    k_tile_dead<T, LEVEL><<<dim3(tile_grid(ctx, k_tile_dead<T, LEVEL>, nb_max), 3), LT, 0, st>>>(m);
+    k_scan_tiles<T><<<3, SCAN_T, 0, st>>>(m);
+    k_tile_movers<T><<<tile_grid(ctx, k_tile_movers<T>, nb_max), LT, 0, st>>>(m);
+    k_tile_fill<T><<<tile_grid(ctx, k_tile_fill<T>, nb_max), LT, 0, st>>>(m);
+    SFQ_LAUNCHED(ctx, 4);
     SFQ_CUDA(cudaGetLastError());
     return QED_OK;
 }
 
-template <class T, bool LEVEL>
-qed_status compact_tiles(qed_ctx *ctx, qed_species *sp, int s, int64_t step, bool may_defer = false) {
-    const int64_t n = sp->count;   // upper bound; kernels read the device count
-    if (n <= 0) return QED_OK;
-    qed_status e = sfq_ensure_work(ctx, (n + LTILE - 1) / LTILE + 1, n);
-    if (e != QED_OK) return e;
-    return compact_tiles_bounded<T, LEVEL>(ctx, sp, s, step, n, false, may_defer);
-}
-
-template <class T>
-qed_status compact_impl(qed_ctx *ctx, qed_species *sp, int s, bool may_defer) {
-    return compact_tiles<T, false>(ctx, sp, s, 0, may_defer);
-}
-
-// The leveling iteration of one species as a CUDA graph: k_lev_begin, then
-// a while node whose body is one pass (k_lev_step) and k_lev_cond.  The
-// graph is kept while the weight array, the cap and the grid stay the same.
-struct LevGraph {
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    const void *w = nullptr;
-    long long cap = 0;
-    int blocks = 0;
-};
-
-static void lev_graph_drop(LevGraph *g) {
-    if (!g) return;
-    if (g->exec) cudaGraphExecDestroy(g->exec);
-    if (g->graph) cudaGraphDestroy(g->graph);
-    delete g;
-}
-
-template <class T>
-static cudaError_t lev_graph_build(qed_ctx *ctx, LevGraph *G, const void *w, int s, long long cap, int blocks) {
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaGraphCreate(&g, 0);
-    if (e != cudaSuccess) return e;
-    LevelWork *lw = ctx->lev;
-    DevCtl *ctl = ctx->ctl;
-    cudaGraphConditionalHandle h;
-    cudaGraphNode_t nb, nw, n1, n2;
-    cudaKernelNodeParams kb{}, ks{}, kc{};
-    cudaGraphNodeParams cp{};
-    void *args_b[] = {&lw, &s};
-    void *args_s[] = {const_cast<void **>(&w), &ctl, &s, &lw, &cap};
-    void *args_c[] = {&lw, &s, &ctl, &h};
-    cudaGraph_t body = nullptr;
-    e = cudaGraphConditionalHandleCreate(&h, g, 1u, cudaGraphCondAssignDefault);
-    if (e != cudaSuccess) goto fail;
-    kb.func = reinterpret_cast<void *>(k_lev_begin);
-    kb.gridDim = dim3(1);
-    kb.blockDim = dim3(1);
-    kb.kernelParams = args_b;
-    e = cudaGraphAddKernelNode(&nb, g, nullptr, 0, &kb);
-    if (e != cudaSuccess) goto fail;
-    cp.type = cudaGraphNodeTypeConditional;
-    cp.conditional.handle = h;
-    cp.conditional.type = cudaGraphCondTypeWhile;
-    cp.conditional.size = 1;
-    e = cudaGraphAddNode(&nw, g, &nb, nullptr, 1, &cp);
-    if (e != cudaSuccess) goto fail;
-    body = cp.conditional.phGraph_out[0];
-    ks.func = reinterpret_cast<void *>(k_lev_step<T>);
-    ks.gridDim = dim3((unsigned)blocks);
-    ks.blockDim = dim3(LEV_T);
-    ks.kernelParams = args_s;
-    e = cudaGraphAddKernelNode(&n1, body, nullptr, 0, &ks);
-    if (e != cudaSuccess) goto fail;
-    kc.func = reinterpret_cast<void *>(k_lev_cond);
-    kc.gridDim = dim3(1);
-    kc.blockDim = dim3(1);
-    kc.kernelParams = args_c;
-    e = cudaGraphAddKernelNode(&n2, body, &n1, 1, &kc);
-    if (e != cudaSuccess) goto fail;
-    e = cudaGraphInstantiate(&G->exec, g, 0);
-    if (e != cudaSuccess) goto fail;
-    G->graph = g;
-    G->w = w;
-    G->cap = cap;
-    G->blocks = blocks;
-    return cudaSuccess;
-fail:
-    cudaGraphDestroy(g);
-    return e;
-}
-
-// Launch species s's leveling graph (building it when needed).  false: the
-// graph could not be built (conditional nodes unavailable); the caller then
-// checks the passes from the host.
-template <class T>
-static bool lev_graph_launch(qed_ctx *ctx, const void *w, int s, long long cap, int blocks) {
-    if (ctx->lev_graph_failed) return false;
-    LevGraph *G = static_cast<LevGraph *>(ctx->lev_graph[s]);
-    if (!G || G->w != w || G->cap != cap || G->blocks != blocks) {
-        lev_graph_drop(G);
-        G = new LevGraph;
-        ctx->lev_graph[s] = nullptr;
-        if (lev_graph_build<T>(ctx, G, w, s, cap, blocks) != cudaSuccess) {
-            delete G;
-            cudaGetLastError();                  // clear the failed call's error
-            ctx->lev_graph_failed = 1;
-            return false;
-        }
-        ctx->lev_graph[s] = G;
-    }
-    if (cudaGraphLaunch(G->exec, ctx->stream) != cudaSuccess) {
-        cudaGetLastError();
-        ctx->lev_graph_failed = 1;
-        return false;
-    }
-    return true;
-}
-
-// Leveling of one species at `step`: the iteration runs on the device (a
-// graph whose while loop runs one pass per iteration; without conditional
-// graph nodes, one launch per pass with a host check per chunk), then
-// keep/drop fused with the first compaction pass.  sp->count must bound the
-// device count.
-template <class T>
-qed_status level_impl(qed_ctx *ctx, qed_species *sp, int s, int64_t step, bool may_defer) {
-    const int64_t cap = ctx->cfg.thin_cap;
-    cudaStream_t st = ctx->stream;
-    if (cap <= 0 || sp->count <= cap) return QED_OK;
-    int blocks = ctx->sm_count * 4;
+// Leveling thresholds of the species of `mask` (device: those whose count
+// exceeds the cap), one cooperative launch.
+template <class T> static qed_status level_launch(qed_ctx *ctx, const qed_particles *p, int mask) {
+    LevWeights w{};
+    for (int s = 0; s < 3; ++s) w.w[s] = ((mask >> s) & 1) && p->s[s].capacity > 0 ? p->s[s].w : nullptr;
+    int per_sm = 0;
+    SFQ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_level<T>, LEV_T, 0));
+    int blocks = ctx->sm_count * (per_sm < 4 ? (per_sm > 0 ? per_sm : 1) : 4);
     blocks = blocks > LEVEL_MAX_BLOCKS ? LEVEL_MAX_BLOCKS : blocks;
-    if (!ctx->cfg.profile && lev_graph_launch<T>(ctx, sp->w, s, (long long)cap, blocks)) {
-        SFQ_LAUNCHED(ctx, 1);                    // k_lev_begin; the passes are counted on the device
-        SFQ_CUDA(cudaGetLastError());
-        return compact_tiles<T, true>(ctx, sp, s, step, may_defer);
-    }
-    k_lev_begin<<<1, 1, 0, st>>>(ctx->lev, s);
+    long long cap = (long long)ctx->cfg.thin_cap;
+    void *args[] = {&w, &ctx->ctl, &ctx->lev, &cap};
+    SFQ_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void *>(k_level<T>), dim3((unsigned)blocks), dim3(LEV_T), args,
+                                         0, ctx->stream));
     SFQ_LAUNCHED(ctx, 1);
-    // passes in chunks (a pass after convergence returns at once); the host
-    // reads the done flag and the pass count between chunks.  A chunk is as
-    // long as the previous leveling of this species needed, so one check
-    // usually suffices.
-    int chunk = ctx->lev_chunk[s] >= 2 ? ctx->lev_chunk[s] : 3;
-    for (int launched = 0; launched < LEVEL_ITERS; launched += chunk, chunk = 2) {
-        for (int c = 0; c < chunk; ++c)
-            k_lev_step<T><<<blocks, LEV_T, 0, st>>>(sp->w, ctx->ctl, s, ctx->lev, (long long)cap);
-        SFQ_LAUNCHED(ctx, chunk);
-        // done and iters are adjacent words of the iteration state
-        SFQ_CUDA(cudaMemcpyAsync(ctx->pin, &ctx->lev->it[s].done, 2 * sizeof(unsigned long long),
-                                 cudaMemcpyDeviceToHost, st));
-        const auto t0 = std::chrono::steady_clock::now();
-        SFQ_CUDA(cudaStreamSynchronize(st));
-        ctx->sync_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
-        if (ctx->pin[0]) break;
-    }
-    const int used = (int)ctx->pin[1];
-    ctx->lev_chunk[s] = used < 2 ? 2 : (used > 12 ? 12 : used);
-    SFQ_CUDA(cudaGetLastError());
-    return compact_tiles<T, true>(ctx, sp, s, step, may_defer);
-}
-
-// ---- the merge step of a captured step graph ----
-// One thread decides on the device what a species' merge step does (no host
-// round trip): leveling when its count exceeds the cap (the iteration is
-// started as by k_lev_begin), dead entries removed when it was leveled or
-// may hold converted photons (otherwise the iteration is finished with w* = 0,
-// so the compaction only removes dead entries).  Nothing runs once a step
-// ran out of capacity or a device check failed.
-__global__ void k_merge_begin(DevCtl *ctl, LevelWork *lw, int s, long long cap, int always_compact,
-                              cudaGraphConditionalHandle h_lev, cudaGraphConditionalHandle h_cmp) {
-    const bool stop = ctl->overflow || ctl->timeout || ctl->bad_index;
-    const unsigned long long c = ctl->count[s], cp = ctl->capacity[s];
-    const unsigned long long n = c < cp ? c : cp;
-    const bool level = !stop && cap > 0 && n > (unsigned long long)cap;
-    lev_start(lw, s);
-    if (!level) lev_finish(lw->it[s], 0.0);
-    const bool compact = !stop && n > 0 && (level || always_compact);
-    if (cap > 0) cudaGraphSetConditional(h_lev, level ? 1u : 0u);
-    cudaGraphSetConditional(h_cmp, compact ? 1u : 0u);
-    if (compact) ctl->graph_kernels += 5;          // the compaction passes below
-}
-
-// Appends species s's merge step to a step graph under capture (ctx->stream
-// is the capture stream): the decision kernel, a while node running the
-// leveling passes, and an if node holding the compaction passes sized by the
-// capacity (their loops follow the device count).
-template <class T>
-qed_status capture_merge(qed_ctx *ctx, GraphBuild &gb, qed_species *sp, int s, bool always_compact) {
-    const long long cap = ctx->cfg.thin_cap;
-    if (sp->capacity <= 0 || (cap <= 0 && !always_compact)) return QED_OK;
-    cudaGraphConditionalHandle h_lev = 0, h_cmp = 0;
-    if (cap > 0 && cudaGraphConditionalHandleCreate(&h_lev, gb.g, 0, cudaGraphCondAssignDefault) != cudaSuccess)
-        return QED_ERR_CUDA;
-    if (cudaGraphConditionalHandleCreate(&h_cmp, gb.g, 0, cudaGraphCondAssignDefault) != cudaSuccess)
-        return QED_ERR_CUDA;
-    LevelWork *lw = ctx->lev;
-    DevCtl *ctl = ctx->ctl;
-    const int ac = always_compact ? 1 : 0;
-    if (gb.capture(gb.g, [&] {
-            k_merge_begin<<<1, 1, 0, ctx->stream>>>(ctl, lw, s, cap, ac, h_lev, h_cmp);
-            return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
-        }) != cudaSuccess)
-        return QED_ERR_CUDA;
-    gb.top_kernels += 1;
-    if (cap > 0) {
-        cudaGraph_t body;
-        if (gb.conditional(h_lev, cudaGraphCondTypeWhile, &body) != cudaSuccess) return QED_ERR_CUDA;
-        int blocks = ctx->sm_count * 4;
-        blocks = blocks > LEVEL_MAX_BLOCKS ? LEVEL_MAX_BLOCKS : blocks;
-        const void *w = sp->w;
-        if (gb.capture(body, [&] {
-                k_lev_step<T><<<blocks, LEV_T, 0, ctx->stream>>>(w, ctl, s, lw, cap);
-                k_lev_cond<<<1, 1, 0, ctx->stream>>>(lw, s, ctl, h_lev);
-                return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
-            }) != cudaSuccess)
-            return QED_ERR_CUDA;
-    }
-    cudaGraph_t cbody;
-    if (gb.conditional(h_cmp, cudaGraphCondTypeIf, &cbody) != cudaSuccess) return QED_ERR_CUDA;
-    if (gb.capture(cbody, [&] { return compact_tiles_bounded<T, true>(ctx, sp, s, 0, sp->capacity, true, true); }) !=
-        cudaSuccess)
-        return QED_ERR_CUDA;
     return QED_OK;
+}
+
+// A merge step: species of level_mask are leveled when their count exceeds
+// the cap (decided on the device), dead entries are removed from those and
+// from the species of `always`.  bound: an upper bound of each device count.
+template <class T>
+static qed_status merge_impl(qed_ctx *ctx, const qed_particles *p, const int64_t bound[3], int level_mask, int always,
+                             int64_t step, bool step_from_ctl, bool may_defer) {
+    MergeArgs m;
+    for (int s = 0; s < 3; ++s)
+        if (bound[s] <= 0) {
+            level_mask &= ~(1 << s);
+            always &= ~(1 << s);
+        }
+    if (!(level_mask | always)) return QED_OK;
+    qed_status e = merge_args<T>(ctx, p, bound, m);
+    if (e != QED_OK) return e;
+    m.step = (unsigned)step;
+    m.step_from_ctl = step_from_ctl ? 1 : 0;
+    m.always = always;
+    m.leveled = level_mask;
+    m.may_defer = may_defer ? 1 : 0;
+    if (!level_mask) return compact_launch<T, false>(ctx, m);
+    e = level_launch<T>(ctx, p, level_mask);
+    return e != QED_OK ? e : compact_launch<T, true>(ctx, m);
 }
 
 // ---- leveling over shards (one species split across processes) ----
@@ -1070,42 +1071,28 @@ qed_status capture_merge(qed_ctx *ctx, GraphBuild &gb, qed_species *sp, int s, b
 // shards (an all-reduce) and advances the iteration with the same step the
 // device uses (sfq_level_advance), then each shard applies w* (level_apply).
 template <class T>
-qed_status level_eval_impl(qed_ctx *ctx, qed_species *sp, int s, double w, double *A, int64_t *C, int64_t *N,
-                           double *M) {
+qed_status level_eval_impl(qed_ctx *ctx, qed_species *sp, double w, double *A, int64_t *C, int64_t *N, double *M) {
     cudaStream_t st = ctx->stream;
     int blocks = ctx->sm_count * 4;
     blocks = blocks > LEVEL_MAX_BLOCKS ? LEVEL_MAX_BLOCKS : blocks;
-    LevelIter h{};
-    h.w = w;
-    h.w_up = ceil_f(w);
-    h.iters = 1;
-    h.mode = 1;
     const unsigned long long n = (unsigned long long)sp->count;
-    const unsigned zero = 0;
-    SFQ_CUDA(cudaMemcpyAsync(&ctx->ctl->count[s], &n, sizeof n, cudaMemcpyHostToDevice, st));
-    SFQ_CUDA(cudaMemcpyAsync(&ctx->ctl->capacity[s], &n, sizeof n, cudaMemcpyHostToDevice, st));
-    SFQ_CUDA(cudaMemcpyAsync(&ctx->lev->it[s], &h, sizeof h, cudaMemcpyHostToDevice, st));
-    SFQ_CUDA(cudaMemcpyAsync(&ctx->lev->arrive[s], &zero, sizeof zero, cudaMemcpyHostToDevice, st));
-    if (n > 0) {
-        k_lev_step<T><<<blocks, LEV_T, 0, st>>>(sp->w, ctx->ctl, s, ctx->lev, 0);
-        SFQ_LAUNCHED(ctx, 1);
-    }
+    *A = *M = 0.0;
+    *C = *N = 0;
+    if (n == 0) return QED_OK;
+    k_lev_eval<T><<<blocks, LEV_T, 0, st>>>(sp->w, n, w, ceil_f(w), 0, ctx->lev);
+    SFQ_LAUNCHED(ctx, 1);
     SFQ_CUDA(cudaGetLastError());
-    SFQ_CUDA(cudaMemcpyAsync(&h, &ctx->lev->it[s], sizeof h, cudaMemcpyDeviceToHost, st));
+    struct {
+        double A;
+        unsigned long long C, N, M;
+    } h;
+    SFQ_CUDA(cudaMemcpyAsync(&h, &ctx->lev->sumA, sizeof h, cudaMemcpyDeviceToHost, st));
     SFQ_CUDA(cudaStreamSynchronize(st));
-    *A = n > 0 ? h.sumA : 0.0;
-    *C = n > 0 ? (int64_t)h.sumC : 0;
-    *N = n > 0 ? (int64_t)h.sumN : 0;
-    *M = n > 0 ? double_of_bits(h.sumM) : 0.0;
+    *A = h.A;
+    *C = (int64_t)h.C;
+    *N = (int64_t)h.N;
+    *M = double_of_bits(h.M);
     return QED_OK;
-}
-
-template <class T>
-qed_status level_apply_impl(qed_ctx *ctx, qed_species *sp, int s, double wstar, int64_t step) {
-    LevelIter h{};
-    lev_finish(h, wstar > 0.0 ? wstar : 0.0);
-    SFQ_CUDA(cudaMemcpyAsync(&ctx->lev->it[s], &h, sizeof h, cudaMemcpyHostToDevice, ctx->stream));
-    return compact_tiles<T, true>(ctx, sp, s, step);
 }
 
 }  // namespace
@@ -1133,45 +1120,37 @@ qed_status sfq_ensure_work(qed_ctx *ctx, int64_t n_blocks, int64_t n_slots) {
     return QED_OK;
 }
 
-qed_status sfq_capture_merge(qed_ctx *ctx, GraphBuild &gb, qed_species *sp, int s, bool always_compact) {
-    if (ctx->cfg.precision == QED_FP32) return capture_merge<float>(ctx, gb, sp, s, always_compact);
-    return capture_merge<double>(ctx, gb, sp, s, always_compact);
+qed_status sfq_ensure_merge(qed_ctx *ctx, const int64_t bound[3]) {
+    return sfq_ensure_work(ctx, merge_blk_words(bound), merge_slot_words(bound));
 }
 
-// Removes every dead entry of the species, its count known only on the device
-// (bounded by the capacity): the end of a batch whose steps deferred moves.
-qed_status sfq_compact_pending(qed_ctx *ctx, qed_species *sp, int s) {
-    if (sp->capacity <= 0) return QED_OK;
-    if (ctx->cfg.precision == QED_FP32) return compact_tiles_bounded<float, false>(ctx, sp, s, 0, sp->capacity, false);
-    return compact_tiles_bounded<double, false>(ctx, sp, s, 0, sp->capacity, false);
+qed_status sfq_merge(qed_ctx *ctx, const qed_particles *p, const int64_t bound[3], int level_mask, int always,
+                     int64_t step, bool step_from_ctl, bool may_defer) {
+    if (ctx->cfg.precision == QED_FP32)
+        return merge_impl<float>(ctx, p, bound, level_mask, always, step, step_from_ctl, may_defer);
+    return merge_impl<double>(ctx, p, bound, level_mask, always, step, step_from_ctl, may_defer);
 }
 
-qed_status sfq_compact_species(qed_ctx *ctx, qed_species *sp, int s, bool may_defer) {
-    if (ctx->cfg.precision == QED_FP32) return compact_impl<float>(ctx, sp, s, may_defer);
-    return compact_impl<double>(ctx, sp, s, may_defer);
+qed_status sfq_level_eval(qed_ctx *ctx, qed_species *sp, double w, double *A, int64_t *C, int64_t *N, double *M) {
+    if (ctx->cfg.precision == QED_FP32) return level_eval_impl<float>(ctx, sp, w, A, C, N, M);
+    return level_eval_impl<double>(ctx, sp, w, A, C, N, M);
 }
 
-void sfq_level_graphs_free(qed_ctx *ctx) {
-    for (int s = 0; s < 3; ++s) {
-        lev_graph_drop(static_cast<LevGraph *>(ctx->lev_graph[s]));
-        ctx->lev_graph[s] = nullptr;
-    }
-}
-
-qed_status sfq_level_species(qed_ctx *ctx, qed_species *sp, int s, int64_t step, bool may_defer) {
-    if (ctx->cfg.precision == QED_FP32) return level_impl<float>(ctx, sp, s, step, may_defer);
-    return level_impl<double>(ctx, sp, s, step, may_defer);
-}
-
-qed_status sfq_level_eval(qed_ctx *ctx, qed_species *sp, int s, double w, double *A, int64_t *C, int64_t *N,
-                          double *M) {
-    if (ctx->cfg.precision == QED_FP32) return level_eval_impl<float>(ctx, sp, s, w, A, C, N, M);
-    return level_eval_impl<double>(ctx, sp, s, w, A, C, N, M);
-}
-
-qed_status sfq_level_apply_species(qed_ctx *ctx, qed_species *sp, int s, double wstar, int64_t step) {
-    if (ctx->cfg.precision == QED_FP32) return level_apply_impl<float>(ctx, sp, s, wstar, step);
-    return level_apply_impl<double>(ctx, sp, s, wstar, step);
+qed_status sfq_level_apply_species(qed_ctx *ctx, const qed_particles *p, int s, double wstar, int64_t step) {
+    LevelIter h{};
+    lev_finish(h, wstar > 0.0 ? wstar : 0.0);
+    SFQ_CUDA(cudaMemcpyAsync(&ctx->lev->it[s], &h, sizeof h, cudaMemcpyHostToDevice, ctx->stream));
+    const int64_t bound[3] = {p->s[0].count, p->s[1].count, p->s[2].count};
+    if (bound[s] <= 0) return QED_OK;
+    qed_status e = sfq_ensure_merge(ctx, bound);
+    if (e != QED_OK) return e;
+    MergeArgs m;
+    const bool f32 = ctx->cfg.precision == QED_FP32;
+    e = f32 ? merge_args<float>(ctx, p, bound, m) : merge_args<double>(ctx, p, bound, m);
+    if (e != QED_OK) return e;
+    m.step = (unsigned)step;
+    m.always = m.leveled = 1 << s;             // w* is given: no threshold to find
+    return f32 ? compact_launch<float, true>(ctx, m) : compact_launch<double, true>(ctx, m);
 }
 
 void sfq_level_advance(double *lo, double *hi, double *w, double *wstar, int64_t *iters, int64_t *done,

@@ -89,21 +89,23 @@ struct LevelIter {
     float wstar_f;          // wstar rounded to float (the new weight in FP32 mode)
     float wstar_inv_f;      // 1 / wstar rounded to float
     unsigned long long done, iters, alive;
-    unsigned long long mode;    // 0: a pass advances the iteration; 1: a pass only stores its sums
-    double sumA;                // sums of the last pass in mode 1
-    unsigned long long sumC, sumN, sumM;
 };
 struct LevelWork {
     LevelIter it[3];
-    unsigned arrive[4];                         // blocks of the current pass that finished (per species)
-    unsigned long long passes[4];               // passes of the current graph-driven leveling
-    double prev[4];                             // last threshold found per species (the next start)
-    double partA[LEVEL_MAX_BLOCKS];             // sum of weights below w (block partials)
-    unsigned long long partC[LEVEL_MAX_BLOCKS]; // count at or above w
-    unsigned long long partN[LEVEL_MAX_BLOCKS]; // alive count
-    unsigned long long partM[LEVEL_MAX_BLOCKS]; // largest weight (double bits)
-    unsigned long long partL[LEVEL_MAX_BLOCKS]; // largest weight below w (double bits; 0: none)
-    unsigned long long partH[LEVEL_MAX_BLOCKS]; // smallest weight at or above w (double bits; +inf: none)
+    unsigned long long on[3];                   // the current merge step leveled the species
+    double prev[3];                             // last threshold found per species
+    double ratio[3];                            // its growth over the one before (the next start: their product)
+    unsigned arrive;                            // blocks of the current pass that finished
+    unsigned long long round;                   // passes finished
+    double sumA;                                // sums of an evaluation for a shard
+    unsigned long long sumC, sumN, sumM;
+    // block partials of each species
+    double partA[3 * LEVEL_MAX_BLOCKS];             // sum of weights below w
+    unsigned long long partC[3 * LEVEL_MAX_BLOCKS]; // count at or above w
+    unsigned long long partN[3 * LEVEL_MAX_BLOCKS]; // alive count
+    unsigned long long partM[3 * LEVEL_MAX_BLOCKS]; // largest weight (double bits)
+    unsigned long long partL[3 * LEVEL_MAX_BLOCKS]; // largest weight below w (double bits; 0: none)
+    unsigned long long partH[3 * LEVEL_MAX_BLOCKS]; // smallest weight at or above w (double bits; +inf: none)
 };
 
 // Philox round keys of one seed: k[2 r], k[2 r + 1] are the key of round r
@@ -184,7 +186,6 @@ struct qed_ctx {
     unsigned long long *slots;    // hole indices
     int64_t slots_cap;
     sfq::LevelWork *lev;          // leveling work (device)
-    unsigned long long *pin;      // small pinned host scratch (flags read back)
     // overflow snapshot
     void *snap;
     int64_t snap_bytes;
@@ -198,8 +199,6 @@ struct qed_ctx {
     int64_t launches;            // kernels launched since the last reset
     double sync_ms;              // host time blocked in stream synchronisation
     void *batch;                 // batched-push work buffers
-    void *lev_graph[3];          // per species: the graph-driven leveling iteration (or null)
-    int lev_graph_failed;        // graphs with conditional nodes unavailable: host-checked passes
     cudaStream_t cap_stream;     // private stream for graph capture (the caller's may be the legacy stream)
     void *od[3];                 // caller's optical-depth arrays (QED_METHOD_OPTICAL_DEPTH, T)
     const void *field_grid;      // caller's gridded field values (QED_FIELD_GRID)
@@ -207,7 +206,6 @@ struct qed_ctx {
     size_t grid_il_bytes;
     int tuned_threads;           // block shape picked by the autotuner (0: none yet)
     int tuned_budget;            // step budget picked by the autotuner (0: none yet)
-    int lev_chunk[3];            // leveling passes enqueued per host check (from the last leveling)
     // steps enqueued without waiting (qed_push_async) until qed_push_wait:
     // the device control block holds the counts meanwhile
     int async_open;
@@ -306,18 +304,17 @@ struct GraphBuild {
 };
 
 // Implemented in sfqed_compact.cu
-// the merge step of species s (leveling when its count exceeds the cap, dead
-// entries removed) appended to a step graph; decided on the device
-qed_status sfq_capture_merge(qed_ctx *ctx, GraphBuild &gb, qed_species *sp, int s, bool always_compact);
+// The merge step (Sec. 4.2, Sec. 5.1): species of level_mask whose count
+// exceeds the cap are leveled (decided on the device), dead entries removed
+// from those and from the species of `always` (bits).  bound: upper bounds of
+// the device counts, for which sfq_ensure_merge has sized the work buffers.
 // may_defer: the moves may be left for a later step (dead entries stay in
-// place while they are few; see k_scan_tiles)
-qed_status sfq_compact_species(qed_ctx *ctx, qed_species *sp, int s, bool may_defer = false);
-qed_status sfq_compact_pending(qed_ctx *ctx, qed_species *sp, int s);
-void sfq_level_graphs_free(qed_ctx *ctx);
-qed_status sfq_level_species(qed_ctx *ctx, qed_species *sp, int s, int64_t step, bool may_defer = false);
-qed_status sfq_level_eval(qed_ctx *ctx, qed_species *sp, int s, double w, double *A, int64_t *C, int64_t *N,
-                          double *M);
-qed_status sfq_level_apply_species(qed_ctx *ctx, qed_species *sp, int s, double wstar, int64_t step);
+// place while they are few; see k_scan_tiles).
+qed_status sfq_ensure_merge(qed_ctx *ctx, const int64_t bound[3]);
+qed_status sfq_merge(qed_ctx *ctx, const qed_particles *p, const int64_t bound[3], int level_mask, int always,
+                     int64_t step, bool step_from_ctl, bool may_defer);
+qed_status sfq_level_eval(qed_ctx *ctx, qed_species *sp, double w, double *A, int64_t *C, int64_t *N, double *M);
+qed_status sfq_level_apply_species(qed_ctx *ctx, const qed_particles *p, int s, double wstar, int64_t step);
 void sfq_level_advance(double *lo, double *hi, double *w, double *wstar, int64_t *iters, int64_t *done,
                        int64_t *alive, double A, int64_t C, int64_t N, double M, int64_t cap);
 qed_status sfq_drain_events(qed_ctx *ctx);

@@ -311,8 +311,18 @@ static qed_status build_step_graph(qed_ctx *ctx, const PassArgs &args, qed_parti
         }
         // merge step (Sec. 4.2): converted photons removed, each species
         // leveled when its count exceeds the cap
-        if (cascade || ctx->cfg.thin_cap > 0)
-            for (int s = 0; s < 3 && rc == QED_OK; ++s) rc = sfq_capture_merge(ctx, gb, &p->s[s], s, cascade && s == 2);
+        if (cascade || ctx->cfg.thin_cap > 0) {
+            const int64_t bound[3] = {p->s[0].capacity, p->s[1].capacity, p->s[2].capacity};
+            const int64_t before = ctx->launches;
+            e = gb.capture(gb.g, [&] {
+                return sfq_merge(ctx, p, bound, ctx->cfg.thin_cap > 0 ? 7 : 0, cascade ? 4 : 0, 0, true, true);
+            });
+            if (e != cudaSuccess) {
+                rc = QED_ERR_CUDA;
+                break;
+            }
+            gb.top_kernels += (int)(ctx->launches - before);
+        }
     } while (0);
     ctx->stream = saved;
     ctx->launches = launches;
@@ -383,19 +393,16 @@ static qed_status host_steps(qed_ctx *ctx, qed_particles *pw, PassArgs &a, doubl
             }
             const DevCtl &c = *ctx->ctl_host;
             if (c.overflow || c.timeout || c.bad_index) break;
-            for (int s = 0; s < 3; ++s) P.s[s].count = (int64_t)c.count[s];
-            // per species: leveling (it skips dead entries and compacts), else
-            // removal of the photons that converted
+            bool level = false;
+            int64_t bound[3];
             for (int s = 0; s < 3; ++s) {
-                const bool level = ctx->cfg.thin_cap > 0 && P.s[s].count > ctx->cfg.thin_cap;
-                const int64_t step = (int64_t)c.step_next - 1;
-                if (level) {
-                    e = timed_block(ctx, 3, [&] { return sfq_level_species(ctx, &P.s[s], s, step, true); });
-                } else if (cascade && s == 2) {
-                    e = timed_block(ctx, 2, [&] { return sfq_compact_species(ctx, &P.s[2], 2, true); });
-                }
-                if (e != QED_OK) return e;
+                bound[s] = P.s[s].capacity;
+                level = level || (ctx->cfg.thin_cap > 0 && (int64_t)c.count[s] > ctx->cfg.thin_cap);
             }
+            qed_status e2 = timed_block(ctx, level ? 3 : 2, [&] {
+                return sfq_merge(ctx, &P, bound, ctx->cfg.thin_cap > 0 ? 7 : 0, cascade ? 4 : 0, 0, true, true);
+            });
+            if (e2 != QED_OK) return e2;
         }
     }
     return QED_OK;
@@ -424,14 +431,14 @@ static qed_status open_batch(qed_ctx *ctx, qed_particles *p, int64_t step0) {
     h.step_next = (unsigned long long)step0;
     h.pass_limit = pass_limit_of(ctx);
     SFQ_CUDA(cudaMemcpyAsync(ctx->ctl, &h, sizeof(DevCtl), cudaMemcpyHostToDevice, ctx->stream));
-    int64_t cap_max = 0;
+    int64_t bound[3];
     for (int s = 0; s < 3; ++s) {
         qed_status e = s < 2 ? ensure_tau(ctx, s, p->s[s].capacity) : QED_OK;
         if (e != QED_OK) return e;
-        cap_max = p->s[s].capacity > cap_max ? p->s[s].capacity : cap_max;
+        bound[s] = p->s[s].capacity;
     }
-    // compaction work buffers sized once for the largest species
-    qed_status e = sfq_ensure_work(ctx, (cap_max + 1023) / 1024 + 2, cap_max);
+    // compaction work buffers sized once for the capacities
+    qed_status e = sfq_ensure_merge(ctx, bound);
     if (e != QED_OK) return e;
     if (ctx->cfg.restore_on_overflow) {
         e = snapshot(ctx, p, false);
@@ -537,12 +544,12 @@ static qed_status wait_batch(qed_ctx *ctx, qed_particles *p, qed_stats *out) {
         // counts returned hold live particles only (after a step that ran out
         // of capacity nothing is moved)
         ctx->async_deferred = 0;
-        for (int s = 0; s < 3; ++s) {
-            qed_status e = sfq_compact_pending(ctx, &ctx->async_p.s[s], s);
-            if (e != QED_OK) {
-                ctx->async_open = 0;
-                return e;
-            }
+        const qed_particles &B = ctx->async_p;
+        const int64_t bound[3] = {B.s[0].capacity, B.s[1].capacity, B.s[2].capacity};
+        qed_status e = sfq_merge(ctx, &B, bound, 0, 7, 0, false, false);
+        if (e != QED_OK) {
+            ctx->async_open = 0;
+            return e;
         }
     }
     qed_status e = read_ctl(ctx);
