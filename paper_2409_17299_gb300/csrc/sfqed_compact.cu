@@ -690,18 +690,29 @@ __global__ void __launch_bounds__(LT, 4) k_tile_dead(const __grid_constant__ Mer
         const unsigned long long wbase = base + (unsigned long long)wid * LSPAN;
         unsigned mask[LROUNDS];
         unsigned cnt = 0;
-#pragma unroll
-        for (int c0 = 0; c0 < LROUNDS; c0 += G) {
-            // weights and (leveling) ids of G entries issued together: at
-            // the cap nearly every entry is below w* and needs its id
-            T v[G];
-            unsigned long long idv[G];
+        // weights and (leveling) ids of G entries issued together, and those of
+        // the next G before this group's draws and stores.  Read-only loads:
+        // an entry's weight is read once, by the thread that may then store it,
+        // and the compiler need not keep the loads behind the stores.
+        T v[G], vn[G];
+        unsigned long long idv[G], idn[G];
+        auto load = [&](int c0, T (&vv)[G], unsigned long long (&ii)[G]) {
 #pragma unroll
             for (int r = 0; r < G; ++r) {
                 const unsigned long long i = wbase + (c0 + r) * 32 + lane;
-                v[r] = i < n ? ld<T>(S.w, i) : (T)0;
-                idv[r] = (LEVEL && thin && i < n) ? S.id[i] : 0ull;
+                vv[r] = i < n ? __ldg(reinterpret_cast<const T *>(S.w) + i) : (T)0;
+                ii[r] = (LEVEL && thin && i < n) ? __ldg(S.id + i) : 0ull;
             }
+        };
+        load(0, vn, idn);
+#pragma unroll
+        for (int c0 = 0; c0 < LROUNDS; c0 += G) {
+#pragma unroll
+            for (int r = 0; r < G; ++r) {
+                v[r] = vn[r];
+                idv[r] = idn[r];
+            }
+            if (c0 + G < LROUNDS) load(c0 + G, vn, idn);
             bool below[G];
 #pragma unroll
             for (int r = 0; r < G; ++r) {

@@ -156,6 +156,7 @@ struct PassArgs {
     float dt_f_gt;          // smallest float above dt (FP32 first-iteration event test)
     unsigned long long seed;
     PhiloxKeys keys;        // round keys of seed (event draws)
+    PhiloxKeys child_keys;  // round keys of the children's ids
     int pass;               // 0: particles present at the step start (tau = 0)
     int soft_filter;
     int fly_newborns;       // newborns are pushed to the end of their birth step (cascades)

@@ -84,6 +84,11 @@ __device__ __forceinline__ bool before_step_end(double tau, double dt) {
     return __double_as_longlong(tau) < __double_as_longlong(dt);
 }
 
+// the step in the working precision (FP32: rounded once on the host)
+template <class T> __device__ __forceinline__ T dt_of(const PassArgs &a);
+template <> __device__ __forceinline__ float dt_of<float>(const PassArgs &a) { return a.dt_f; }
+template <> __device__ __forceinline__ double dt_of<double>(const PassArgs &a) { return a.dt; }
+
 template <class T> __device__ __forceinline__ T t_inf();
 template <> __device__ __forceinline__ double t_inf<double>() { return __longlong_as_double(0x7ff0000000000000ll); }
 template <> __device__ __forceinline__ float t_inf<float>() { return __int_as_float(0x7f800000); }
@@ -319,7 +324,7 @@ __device__ __forceinline__ void pair_create(const PassArgs &a, const StepTime &t
     em = em < (T)1 ? (T)1 : em;
     ep = ep < (T)1 ? (T)1 : ep;
     const T pm = f_sqrt((em - (T)1) * (em + (T)1)), pp = f_sqrt((ep - (T)1) * (ep + (T)1));
-    const uint4 rid = event_draw(a.seed ^ CHILD_KEY_XOR, id, tm.step, k);
+    const uint4 rid = event_draw(a.child_keys, id, tm.step, k);
     const unsigned long long se = warp_append(&ctl->count[0], 1);
     const unsigned long long sp = warp_append(&ctl->count[1], 1);
     if (se < ctl->capacity[0]) {
@@ -370,27 +375,34 @@ __device__ __forceinline__ bool photon_flight(const PassArgs &a, const StepTime 
     T lam;
     if constexpr (sizeof(T) == 4) lam = alpha_r * inv * rate_pair<T>(s_coef, chi);
     else lam = alpha_r / k0 * rate_pair<T>(s_coef, chi);     // the oracle's rounding
+    // the remaining time of the step, and with FP32 clocks inside a step the
+    // margin within which the FP64 test decides (as in the lepton pass)
+    T h, marg = (T)0;
+    if constexpr (FRESH) h = dt_of<T>(a);
+    else {
+        h = (T)(a.dt - tau);
+        if constexpr (sizeof(T) == 4) marg = fmaf(h, 0x1p-20f, a.dt_f * 0x1p-40f);
+    }
     uint4 r = make_uint4(0, 0, 0, 0);
     T dth = t_inf<T>();
     if (lam > lam_skip<T>(a)) {
         r = event_draw(a.keys, id, tm.step, 0u);
         T uw, vw;
         Uniform<T>::draw(r.x, r.y, uw, vw);
-        dth = f_div(Uniform<T>::neglog(uw, vw), lam);
+        // -ln u >= 1 - u = v: with v above lambda h (by a margin far above every
+        // rounding involved) the photon reaches the step end, and neither the
+        // logarithm nor the division is needed.  About one photon in a
+        // thousand converts per step, so nearly every warp ends here.
+        if (!(vw > lam * ((h + marg) * (T)(1.0 + 1e-4)))) dth = f_div(Uniform<T>::neglog(uw, vw), lam);
     }
     bool no_event;
-    T h;
-    if constexpr (FRESH && sizeof(T) == 4) { no_event = dth >= a.dt_f_gt; h = a.dt_f; }
-    else if constexpr (FRESH) { no_event = dth > a.dt; h = a.dt; }
+    if constexpr (FRESH && sizeof(T) == 4) no_event = dth >= a.dt_f_gt;
+    else if constexpr (FRESH) no_event = dth > a.dt;
     else if constexpr (sizeof(T) == 4) {
-        // as in the lepton pass: the FP64 test decided in FP32 outside a margin
-        const float rf = __double2float_rn(a.dt - tau);
-        const float marg = fmaf(rf, 0x1p-20f, a.dt_f * 0x1p-40f);
-        if (dth > rf + marg) no_event = true;
-        else if (dth < rf - marg) no_event = false;
+        if (dth > h + marg) no_event = true;
+        else if (dth < h - marg) no_event = false;
         else no_event = tau + (double)dth > a.dt;
-        h = rf;
-    } else { no_event = tau + (double)dth > a.dt; h = (T)(a.dt - tau); }
+    } else no_event = tau + (double)dth > a.dt;
     if (no_event) {
         x[0] += nx * h; x[1] += ny * h; x[2] += nz * h;
         return false;
@@ -527,7 +539,7 @@ __device__ __forceinline__ void stack_round(const LeptonCtx<T> &c, LeptonStack<T
     if (event) {
         T kv[3];
         if (recoil<T>(c.a, p, gam, p2, delta, om, kv)) {
-            const uint4 rid = event_draw(c.a.seed ^ CHILD_KEY_XOR, id, c.tm.step, k);
+            const uint4 rid = event_draw(c.a.child_keys, id, c.tm.step, k);
             if (c.a.fly_newborns) fly_newborn<T>(c, q, pos, E, B, x, kv, tau, w, rid, gen + 1u, ps);
             else append_photon<T>(c.a, c.ctl, c.cap_ph, x, kv, w, rid);
         }
@@ -844,11 +856,6 @@ template <class T> __device__ __forceinline__ T od_exp1(const uint4 &r) {
     return Uniform<T>::neglog(u, v);
 }
 
-// the step in the working precision (FP32: rounded once on the host)
-template <class T> __device__ __forceinline__ T dt_of(const PassArgs &a);
-template <> __device__ __forceinline__ float dt_of<float>(const PassArgs &a) { return a.dt_f; }
-template <> __device__ __forceinline__ double dt_of<double>(const PassArgs &a) { return a.dt; }
-
 // od after this step's decrement, drawn first when not drawn yet.  The
 // product is rounded on its own (no contraction), as in the oracle.
 template <class T>
@@ -903,7 +910,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_lepton_od(Pas
             const T delta = sample_emission<T>(c.icdf, chi, ue, ve, &om);
             T kv[3];
             if (recoil<T>(a, p, gam, p2, delta, om, kv))
-                append_photon<T>(a, ctl, c.cap_ph, x, kv, w, event_draw(a.seed ^ CHILD_KEY_XOR, id, tm.step, 0u));
+                append_photon<T>(a, ctl, c.cap_ph, x, kv, w, event_draw(a.child_keys, id, tm.step, 0u));
             od = od_exp1<T>(r);
             k = 1;
         }
@@ -1010,7 +1017,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_photon_od(Pas
                 em = em < (T)1 ? (T)1 : em;
                 ep = ep < (T)1 ? (T)1 : ep;
                 const T pm = f_sqrt((em - (T)1) * (em + (T)1)), pp = f_sqrt((ep - (T)1) * (ep + (T)1));
-                const uint4 rid = event_draw(a.seed ^ CHILD_KEY_XOR, id, tm.step, 0u);
+                const uint4 rid = event_draw(a.child_keys, id, tm.step, 0u);
                 const unsigned long long se = warp_append(&ctl->count[0], 1);
                 const unsigned long long sp = warp_append(&ctl->count[1], 1);
                 if (se < cap_e) {

@@ -524,6 +524,7 @@ static qed_status enqueue_steps(qed_ctx *ctx, const qed_field_desc *field, doubl
     a.dt_f_gt = (double)a.dt_f > dt ? a.dt_f : nextafterf(a.dt_f, INFINITY);
     a.seed = ctx->cfg.seed;
     a.keys = philox_keys(ctx->cfg.seed);
+    a.child_keys = philox_keys(ctx->cfg.seed ^ CHILD_KEY_XOR);
     a.soft_filter = ctx->cfg.soft_photon_filter;
     a.fly_newborns = cascade && ctx->cfg.event_method == QED_METHOD_SUBSTEP ? 1 : 0;
 
