@@ -837,6 +837,184 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_photon_pass(P
 }
 
 
+#if !SFQ_GRID
+// The FP32 photon pass in a field that does not depend on the position
+// (uniform, rotating E), two consecutive photons per thread.  A photon is a
+// chain of some 250 dependent instructions (a scheduler issued in 65% of the
+// cycles with one photon per thread and 32 warps per SM); the chains of two
+// photons interleave, and copies, shared-memory reads and stores move two
+// photons at a time.  Both photons' arithmetic is written out with explicit
+// rounding where the compiler could fuse either way.  5e7 photons, rotating E:
+// 40 steps of its cascade 82.2 -> 77.1 ms; two blocks per SM (106 registers) as fast as three (spills).
+// In the standing wave the two sine and cosine evaluations do not interleave
+// (their argument reduction branches): 40 steps took 72.1 ms against 71.6 with
+// one photon per thread, which stays the rule there and on the grid.
+__device__ __forceinline__ void cp_async8z(void *smem, const void *gmem, unsigned bytes) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(gmem), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async16z(void *smem, const void *gmem, unsigned bytes) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(gmem), "r"(bytes) : "memory");
+}
+
+__global__ void __launch_bounds__(256, 2) k_photon_pass2(const __grid_constant__ PassArgs a) {
+    DevCtl *ctl = a.ctl;
+    constexpr int NT = 256;
+    const unsigned n = (unsigned)ctl->end[2];
+    const unsigned pairs = (n + 1) / 2;
+    __shared__ __align__(16) float s_coef[RateWords<float>::N];
+    __shared__ StepTime s_tm;
+    if (blockIdx.x * NT < pairs) {
+        for (int i = threadIdx.x; i < RateWords<float>::N; i += NT) s_coef[i] = reinterpret_cast<const float *>(a.coef)[i];
+        if (threadIdx.x == 0) s_tm = load_step_time(a);
+        __syncthreads();
+        const StepTime &tm = s_tm;
+        const unsigned step = tm.step;
+        const float *icdf = reinterpret_cast<const float *>(a.icdf_pair);
+        const SpeciesDev &S = a.sp[2];
+        PassStats ps;
+        const Phase<float> ph0 = time_phase<float, StepTime>(tm, 0.0);
+        const float *tab = s_coef + 4 * EM_NSEG;
+        const float skip = a.lam_skip_f, h = a.dt_f;
+        const float alpha_r = (float)(ALPHA * RS);
+        // two buffers per thread: the next pair's copies run under this pair's work
+        __shared__ __align__(16) float2 stg[2][7][NT];         // w x y z kx ky kz
+        __shared__ __align__(16) ulonglong2 sid[2][NT];
+        const unsigned stride = gridDim.x * NT;
+        const int t = threadIdx.x;
+        auto stage = [&](unsigned j, int buf) {
+            const unsigned i = 2 * j, b = i + 1 < n ? 8u : 4u;     // an odd last photon: nothing read past the count
+            cp_async8z(&stg[buf][0][t], reinterpret_cast<const float *>(S.w) + i, b);
+            cp_async8z(&stg[buf][1][t], reinterpret_cast<const float *>(S.x) + i, b);
+            cp_async8z(&stg[buf][2][t], reinterpret_cast<const float *>(S.y) + i, b);
+            cp_async8z(&stg[buf][3][t], reinterpret_cast<const float *>(S.z) + i, b);
+            cp_async8z(&stg[buf][4][t], reinterpret_cast<const float *>(S.px) + i, b);
+            cp_async8z(&stg[buf][5][t], reinterpret_cast<const float *>(S.py) + i, b);
+            cp_async8z(&stg[buf][6][t], reinterpret_cast<const float *>(S.pz) + i, b);
+            cp_async16z(&sid[buf][t], S.id + i, 2 * b);
+        };
+        const unsigned j0 = blockIdx.x * NT + threadIdx.x;
+        if (j0 < pairs) stage(j0, 0);
+        cp_async_commit();
+        int buf = 0;
+        for (unsigned j = j0; j < pairs; j += stride, buf ^= 1) {
+            if (j + stride < pairs) stage(j + stride, buf ^ 1);
+            cp_async_commit();
+            cp_async_wait_prev();                // this thread's copies of pair j have landed
+            float w[2], x[3][2], k[3][2];
+            unsigned long long id[2];
+            {
+                float2 v;
+                v = stg[buf][0][t]; w[0] = v.x; w[1] = v.y;              // zero-filled past the count: dead
+                for (int c = 0; c < 3; ++c) { v = stg[buf][1 + c][t]; x[c][0] = v.x; x[c][1] = v.y; }
+                for (int c = 0; c < 3; ++c) { v = stg[buf][4 + c][t]; k[c][0] = v.x; k[c][1] = v.y; }
+                const ulonglong2 u = sid[buf][t];
+                id[0] = u.x; id[1] = u.y;
+            }
+            float k0[2], inv[2], nd[3][2], chi[2], lam[2];
+            bool fly[2], due[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                k0[q] = f_sqrt(sum_sq<true>(k[0][q], k[1][q], k[2][q]));
+                inv[q] = f_div(1.0f, k0[q]);
+                fly[q] = w[q] > 0.f && k0[q] > 0.f;
+                for (int c = 0; c < 3; ++c) nd[c][q] = __fmul_rn(k[c][q], inv[q]);
+            }
+            // chi of both photons, case by case
+            if (a.field_zero == 1 && a.field_kind == QED_FIELD_ROTATING_E) {
+                const float e0 = a.prm_f[0] * ph0.c, e1 = a.prm_f[0] * ph0.s;
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const float ax = diff_of_products(k[1][q], 0.f, k[2][q], e1);
+                    const float ay = diff_of_products(k[2][q], e0, k[0][q], 0.f);
+                    const float az = diff_of_products(k[0][q], e1, k[1][q], e0);
+                    chi[q] = f_sqrt(sum_sq<true>(ax, ay, az)) * (float)(1.0 / RS);
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const float xq[3] = {x[0][q], x[1][q], x[2][q]}, kq[3] = {k[0][q], k[1][q], k[2][q]};
+                    float E[3], B[3];
+                    field_at<float>(a, xq, ph0, E, B);
+                    chi[q] = photon_chi<float, true>(k0[q], kq, E, B, ps.n64, a.field_zero);
+                }
+            }
+            // rates (rate_pair<float>, its last piece's continuation apart)
+            bool beyond = false;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const float u = piece_coord(chi[q], 2 * RSEG);
+                beyond = beyond || u >= (float)PAIR_NSEG;
+                const int i = u > 0.f ? min((int)u, PAIR_NSEG - 1) : 0;
+                const float F = f_exp(__fsub_rn(piece_eval(tab, i, __fsub_rn(u, (float)i)), f_div(8.0f / 3.0f, chi[q])));
+                lam[q] = __fmul_rn(__fmul_rn(alpha_r, inv[q]), chi[q] >= (float)PAIR_CHI_MIN ? F : 0.f);
+            }
+            if (beyond)
+                for (int q = 0; q < 2; ++q) lam[q] = __fmul_rn(__fmul_rn(alpha_r, inv[q]), rate_pair<float>(s_coef, chi[q]));
+            due[0] = fly[0] && lam[0] > skip;
+            due[1] = fly[1] && lam[1] > skip;
+            float uw[2], vw[2];
+            uint4 r[2];
+            if (due[0] || due[1]) {
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    r[q] = event_draw(a.keys, id[q], step, 0u);
+                    Uniform<float>::draw(r[q].x, r[q].y, uw[q], vw[q]);
+                    // as in photon_flight: above this the photon reaches the step end
+                    due[q] = due[q] && !(vw[q] > lam[q] * (h * (float)(1.0 + 1e-4)));
+                }
+            }
+            if (due[0] || due[1]) {
+                for (int q = 0; q < 2; ++q) {
+                    if (!due[q]) continue;
+                    const float dth = f_div(Uniform<float>::neglog(q ? uw[1] : uw[0], q ? vw[1] : vw[0]), q ? lam[1] : lam[0]);
+                    if (dth >= a.dt_f_gt) {
+                        due[q] = false;
+                        continue;
+                    }
+                    const float kq[3] = {q ? k[0][1] : k[0][0], q ? k[1][1] : k[1][0], q ? k[2][1] : k[2][0]};
+                    const float nq[3] = {q ? nd[0][1] : nd[0][0], q ? nd[1][1] : nd[1][0], q ? nd[2][1] : nd[2][0]};
+                    float xq[3] = {q ? x[0][1] : x[0][0], q ? x[1][1] : x[1][0], q ? x[2][1] : x[2][0]};
+                    for (int c = 0; c < 3; ++c) xq[c] = __fmaf_rn(nq[c], dth, xq[c]);
+                    const uint4 rq = q ? r[1] : r[0];
+                    pair_create<float>(a, tm, icdf, xq, kq, q ? k0[1] : k0[0], nq[0], nq[1], nq[2], (double)dth,
+                                       q ? w[1] : w[0], q ? id[1] : id[0], 0u, make_uint2(rq.z, rq.w), ps.n64,
+                                       [](int, unsigned) {});
+                    const unsigned i = 2 * j + q;
+                    st<float>(S.w, i, 0.f);       // the photon is eliminated
+                    S.nev[i] += 1u;
+                    ++ps.pr;
+                    ps.mx = 1u;
+                    for (int c = 0; c < 3; ++c) { if (q) x[c][1] = xq[c]; else x[c][0] = xq[c]; }
+                }
+            } else {
+                due[0] = due[1] = false;
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                ps.ph += w[q] > 0.f ? 1 : 0;
+                if (fly[q] && !due[q])
+                    for (int c = 0; c < 3; ++c) x[c][q] = __fmaf_rn(nd[c][q], h, x[c][q]);
+            }
+            // a dead photon's place is written back as it was read
+            if (2 * j + 1 < n) {
+                if (w[0] > 0.f || w[1] > 0.f) {
+                    reinterpret_cast<float2 *>(S.x)[j] = make_float2(x[0][0], x[0][1]);
+                    reinterpret_cast<float2 *>(S.y)[j] = make_float2(x[1][0], x[1][1]);
+                    reinterpret_cast<float2 *>(S.z)[j] = make_float2(x[2][0], x[2][1]);
+                }
+            } else if (w[0] > 0.f) {
+                st<float>(S.x, 2 * j, x[0][0]); st<float>(S.y, 2 * j, x[1][0]); st<float>(S.z, 2 * j, x[2][0]);
+            }
+        }
+        __syncwarp();
+        flush_stats(ctl, ps);
+    }
+    if (last_block(ctl) && threadIdx.x < 2) ctl->born[threadIdx.x] = count_now(ctl, threadIdx.x);
+}
+#endif
+
 // ---- the accumulated-optical-depth method (QED_METHOD_OPTICAL_DEPTH) ----
 // Per particle and step: the rate at the step start; an optical depth not
 // drawn yet (od <= 0) is drawn as -ln u from Philox(id, step, OD_DRAW); od
@@ -1131,8 +1309,16 @@ template <class T>
 qed_status launch_pass(qed_ctx *ctx, PassArgs &a, bool photons, cudaGraphConditionalHandle h, int loop) {
     qed_status e = QED_OK;
     if (a.pass == 0 && photons) {
-        const int bp = resident_blocks(ctx, k_photon_pass<T>, 256);
-        e = timed_launch(ctx, 1, [&] { k_photon_pass<T><<<bp, 256, 0, ctx->stream>>>(a); });
+#if !SFQ_GRID
+        if (sizeof(T) == 4 && a.field_kind != QED_FIELD_STANDING_CP) {
+            const int bp = resident_blocks(ctx, k_photon_pass2, 256);
+            e = timed_launch(ctx, 1, [&] { k_photon_pass2<<<bp, 256, 0, ctx->stream>>>(a); });
+        } else
+#endif
+        {
+            const int bp = resident_blocks(ctx, k_photon_pass<T>, 256);
+            e = timed_launch(ctx, 1, [&] { k_photon_pass<T><<<bp, 256, 0, ctx->stream>>>(a); });
+        }
         if (e != QED_OK) return e;
         SFQ_LAUNCHED(ctx, 1);
     }
