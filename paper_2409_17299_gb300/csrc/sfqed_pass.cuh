@@ -743,6 +743,96 @@ __global__ void __launch_bounds__(LB<T>, (sizeof(T) == 4 && !MLP ? 3 : 2))
     }
 }
 
+// Several steps of an emission run (photons recorded, no leveling): nothing
+// couples the leptons between steps, so one launch carries them through all
+// steps of a call.  A block holds a lepton per thread in registers; per step
+// those without an event are pushed to the step end, the others go through
+// the stack as in the pass above and come back through the species arrays.
+// The arithmetic per particle and step is that of the pass, as are the draws.
+//
+// A launch per step is bound by its latency where the ensemble is small: the
+// step-begin kernel, the tables' staging and the block's last, partly filled
+// rounds took 80 us per step for 16384 electrons in FP64 (49 us here).
+template <class T>
+__global__ void __launch_bounds__(LB<T>, 2) k_lepton_steps(const __grid_constant__ PassArgs a, unsigned long long step0,
+                                                           int nsteps) {
+    constexpr int NT = LB<T>;
+    DevCtl *ctl = a.ctl;
+    __shared__ __align__(16) T s_coef[RateWords<T>::N];
+    __shared__ LeptonStack<T> q;
+    __shared__ StepTime s_tm;
+    __shared__ Phase<T> s_ph;
+    __shared__ int s_stop;
+    const unsigned n0 = (unsigned)min(ctl->count[0], ctl->capacity[0]), n1 = (unsigned)min(ctl->count[1], ctl->capacity[1]);
+    const unsigned n = n0 + n1;
+    if (blockIdx.x * NT >= n) return;
+    for (int i = threadIdx.x; i < RateWords<T>::N; i += NT) s_coef[i] = reinterpret_cast<const T *>(a.coef)[i];
+    if (threadIdx.x < 3) q.pushed[threadIdx.x] = 0;
+    PassStats ps;
+    MlpInf ms{nullptr, nullptr, nullptr};
+    StackPos pos{0, 0, 0};
+    auto next_iteration = [&] {                  // as in the pass: sizes after this iteration's pushes
+        const int nx = pos.it == 2 ? 0 : pos.it + 1;
+        if (threadIdx.x == 0) q.pushed[nx] = 0;
+        __syncthreads();
+        pos.n += q.pushed[pos.it];
+        pos.it = nx;
+    };
+    for (unsigned base = blockIdx.x * NT; base < n; base += gridDim.x * NT) {
+        const unsigned j = base + threadIdx.x;
+        const int s = j < n0 ? 0 : 1;
+        const unsigned i = s == 0 ? j : j - n0;
+        const SpeciesDev &S = a.sp[s];
+        const unsigned idx = i | ((unsigned)s << 31);
+        T w = (T)0, x[3], p[3];
+        unsigned long long id = 0;
+        if (j < n) {
+            w = ld<T>(S.w, i);
+            x[0] = ld<T>(S.x, i); x[1] = ld<T>(S.y, i); x[2] = ld<T>(S.z, i);
+            p[0] = ld<T>(S.px, i); p[1] = ld<T>(S.py, i); p[2] = ld<T>(S.pz, i);
+            id = __ldg(S.id + i);
+        }
+        const T qch = s == 0 ? (T)-1 : (T)1;
+        for (int it = 0; it < nsteps; ++it) {
+            if (threadIdx.x == 0) {
+                // the step's time and index as the step-begin kernel writes them
+                const double t_n = (double)(step0 + it) * a.dt;
+                s_tm.field_kind = a.field_kind;
+                s_tm.t_n = t_n;
+                s_tm.t_n_red_f = (float)fmod(t_n, 2.0 * 3.14159265358979323846);
+                s_tm.step = (unsigned)(step0 + it);
+                s_ph = time_phase<T, StepTime>(s_tm, 0.0);
+                s_stop = __ldcg(&ctl->overflow) != 0;
+            }
+            __syncthreads();
+            if (s_stop) break;                   // out of capacity: later steps do nothing
+            const LeptonCtx<T> c{a, ctl, s_coef, reinterpret_cast<const T *>(a.icdf_em), ctl->capacity[2], 0u,
+                                 (T)(ALPHA * RS), s_tm, s_ph};
+            bool away = false;
+            if (w > (T)0) {
+                double tau = 0.0;
+                ++ps.lep;
+                uint2 rz = make_uint2(0, 0);
+                away = advance<T, true>(c, x, p, qch, tau, id, 0u, rz, ps.n64);
+                if (away) stack_push<T>(q, pos, x, p, tau, id, w, idx, 0u, 0u, rz);
+            }
+            next_iteration();
+            while (pos.n > 0) {
+                stack_round<T, false>(c, q, pos, ps, ms);
+                next_iteration();
+            }
+            if (away) {                          // written by the thread that finished it, before the barrier
+                x[0] = ld<T>(S.x, i); x[1] = ld<T>(S.y, i); x[2] = ld<T>(S.z, i);
+                p[0] = ld<T>(S.px, i); p[1] = ld<T>(S.py, i); p[2] = ld<T>(S.pz, i);
+            }
+        }
+        if (w > (T)0) finish<T>(a, idx, x, p, 0u);
+        __syncthreads();                         // s_tm is rewritten by the next tile's first step
+    }
+    __syncwarp();
+    flush_stats(ctl, ps);
+}
+
 // Photon push: straight flight, pair creation at the event, the photon is
 // removed (weight 0) and the pair appended, its leptons left to the lepton
 // pass of the same step (the last block to finish closes their range).
@@ -1327,6 +1417,18 @@ qed_status launch_pass(qed_ctx *ctx, PassArgs &a, bool photons, cudaGraphConditi
     else
         e = a.pass == 0 ? launch_leptons<T, true, false>(ctx, a, h, loop) : launch_leptons<T, false, false>(ctx, a, h, loop);
     if (e != QED_OK) return e;
+    SFQ_CUDA(cudaGetLastError());
+    return QED_OK;
+}
+
+template <class T>
+qed_status launch_steps(qed_ctx *ctx, PassArgs &a, int64_t step0, int nsteps) {
+    const int bl = resident_blocks(ctx, k_lepton_steps<T>, LB<T>);
+    qed_status e = timed_launch(ctx, 0, [&] {
+        k_lepton_steps<T><<<bl, LB<T>, 0, ctx->stream>>>(a, (unsigned long long)step0, nsteps);
+    });
+    if (e != QED_OK) return e;
+    SFQ_LAUNCHED(ctx, 1);
     SFQ_CUDA(cudaGetLastError());
     return QED_OK;
 }

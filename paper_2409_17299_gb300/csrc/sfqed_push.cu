@@ -58,6 +58,13 @@ __global__ void k_step_begin(DevCtl *ctl, double dt) {
     ctl->spilled = 0;
 }
 
+// the control block after nsteps steps taken by one launch
+__global__ void k_advance_step(DevCtl *ctl, double dt, unsigned long long nsteps) {
+    ctl->step_next += nsteps;
+    ctl->sv_step = (unsigned)(ctl->step_next - 1);
+    ctl->sv_t_n = (double)(ctl->step_next - 1) * dt;
+}
+
 __global__ void k_set_step(DevCtl *ctl, unsigned long long step) { ctl->step_next = step; }
 
 // ---- component kernels for the parity tests ----
@@ -529,6 +536,14 @@ static qed_status enqueue_steps(qed_ctx *ctx, const qed_field_desc *field, doubl
     a.fly_newborns = cascade && ctx->cfg.event_method == QED_METHOD_SUBSTEP ? 1 : 0;
 
     ctx->async_deferred = 1;
+    if (!cascade && ctx->cfg.thin_cap == 0 && ctx->cfg.event_method == QED_METHOD_SUBSTEP && !a.mlp_w16 && nsteps > 1) {
+        // an emission run of several steps: one launch for all of them
+        a.pass = 0;
+        k_advance_step<<<1, 1, 0, ctx->stream>>>(ctx->ctl, dt, (unsigned long long)nsteps);
+        SFQ_LAUNCHED(ctx, 1);
+        if (field->kind == QED_FIELD_GRID) return pass_grid::launch_steps<T>(ctx, a, step0, nsteps);
+        return pass_analytic::launch_steps<T>(ctx, a, step0, nsteps);
+    }
     StepGraph *G = ctx->cfg.profile ? nullptr : step_graph_for<T>(ctx, a, p, dt);
     if (!G) return host_steps<T>(ctx, p, a, dt, nsteps);
     for (int it = 0; it < nsteps; ++it) SFQ_CUDA(cudaGraphLaunch(G->exec, ctx->stream));
