@@ -217,7 +217,7 @@ __device__ __forceinline__ void fused_emit(const FusedCtx &c, const EnsDev &e, u
     const T pa = f_sqrt((g_after - (T)1) * (g_after + (T)1));
     if (!(b.soft_filter && k0 < (T)2)) {
         const uint4 rid = event_draw(b.seed ^ CHILD_KEY_XOR, id, step, k);
-        const unsigned long long slot = warp_append(&b.ph_count[ens], 1);
+        const unsigned long long slot = warp_append_keyed(b.ph_count, ens);     // a round mixes ensembles
         if (slot < e.ph_cap) {
             const SpeciesDev &P = e.ph;
             st<T>(P.x, slot, x[0]); st<T>(P.y, slot, x[1]); st<T>(P.z, slot, x[2]);

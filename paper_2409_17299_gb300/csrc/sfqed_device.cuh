@@ -652,4 +652,16 @@ __device__ __forceinline__ unsigned long long warp_append(unsigned long long *co
     return base + (unsigned long long)below * n_each;
 }
 
+// The same where the lanes may append to different counters: the lanes of one
+// key share its counter.
+__device__ __forceinline__ unsigned long long warp_append_keyed(unsigned long long *counters, unsigned key) {
+    const unsigned mask = __match_any_sync(__activemask(), key);
+    const int lane = threadIdx.x & 31;
+    const int leader = __ffs(mask) - 1;
+    unsigned long long base = 0;
+    if (lane == leader) base = atomicAdd(&counters[key], (unsigned long long)__popc(mask));
+    base = __shfl_sync(mask, base, leader);
+    return base + (unsigned long long)__popc(mask & ((1u << lane) - 1u));
+}
+
 }  // namespace sfq
