@@ -138,6 +138,7 @@ struct PassArgs {
     SpeciesDev sp[3];
     DevCtl *ctl;
     const void *coef;       // NCOEF coefficients (T)
+    const float *coef32;    // NRATE32 words of the FP32 rate pieces
     const void *icdf_em;    // EM_NCHI * EM_NS (T)
     const void *icdf_pair;  // PAIR_NCHI * PAIR_NS (T)
     const __nv_bfloat16 *mlp_w16;   // surrogate network weights, or null (table sampler)

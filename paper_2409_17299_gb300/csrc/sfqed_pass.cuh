@@ -201,6 +201,7 @@ template <class T> struct LeptonCtx {
     const PassArgs &a;
     DevCtl *ctl;
     const T *coef;
+    const float *coef32;    // FP64 mode: the FP32 rate pieces (surely_flies)
     const T *icdf;
     unsigned long long cap_ph;
     unsigned gen_limit;     // generations a step may run (then it is marked as timed out)
@@ -362,6 +363,54 @@ __device__ __forceinline__ void pair_create(const PassArgs &a, const StepTime &t
 __device__ __forceinline__ float own(float v) { asm volatile("" : "+f"(v)); return v; }
 __device__ __forceinline__ double own(double v) { asm volatile("" : "+d"(v)); return v; }
 
+// FP64 mode: whether a photon surely reaches the step end, decided in FP32.
+// Converting takes -ln u <= lambda h, and -ln u >= v = 1 - u; with a bound of
+// lambda from above (chi bounded without cancellation, the FP32 rate form,
+// monotonic in chi, 1% on top, far above every rounding and the arguments'
+// own) v > lambda h decides, and neither chi, rate nor logarithm is needed in
+// FP64.  Photons it does not decide (those that convert and about as many
+// others) take the FP64 path, so what is computed is unchanged.  On GB300 an
+// FP64 instruction occupies its pipe 16 times as long as an FP32 one: the
+// photon pass at 5e5 photons in the standing wave took 265 us of a step, and 20 steps 18.6 ms; 15.4 ms with the bound.
+// chi_ub: an upper bound of chi; tab32: the FP32 rate pieces.
+__device__ __forceinline__ bool surely_flies(const PassArgs &a, const float *tab32, float chi_ub, float inv_k0, float h,
+                                             unsigned long long id, unsigned step) {
+    const float lam = (float)(ALPHA * RS) * inv_k0 * rate_pair<float>(tab32, chi_ub * 1.0001f);
+    const uint4 r = event_draw(a.keys, id, step, 0u);
+    float u, v;
+    Uniform<float>::draw(r.x, r.y, u, v);
+    return v > lam * h * 1.01f;
+}
+
+// chi R = |k0 E + k x B| without the part along k: at most |k x E| + |k x B|
+__device__ __forceinline__ float chi_bound(const float k[3], const float E[3], const float B[3]) {
+    const float ax = k[1] * E[2] - k[2] * E[1], ay = k[2] * E[0] - k[0] * E[2], az = k[0] * E[1] - k[1] * E[0];
+    const float bx = k[1] * B[2] - k[2] * B[1], by = k[2] * B[0] - k[0] * B[2], bz = k[0] * B[1] - k[1] * B[0];
+    const float e = fabsf(k[0]) + fabsf(k[1]) + fabsf(k[2]);      // the products' rounding: 2^-22 of their sizes
+    const float f = fabsf(E[0]) + fabsf(E[1]) + fabsf(E[2]) + fabsf(B[0]) + fabsf(B[1]) + fabsf(B[2]);
+    return (sqrtf(ax * ax + ay * ay + az * az) + sqrtf(bx * bx + by * by + bz * bz) + e * f * 0x1p-21f) * (float)(1.0 / RS);
+}
+
+// The same at the step start from the field's descriptor alone: in the
+// standing wave E and B lie along (0, cos t, sin t) with E^2 + B^2 = a0^2
+// everywhere, so chi R = a0 |k x (0, cos t, sin t)|, whatever x; a0 |k x
+// (cos t, sin t, 0)| in the rotating field.  The step's phase is taken from
+// the FP64 sine and cosine.
+__device__ __forceinline__ float chi_bound_start(const PassArgs &a, const Phase<double> &ph, const float k[3]) {
+    const float zero[3] = {0.f, 0.f, 0.f};
+    const float c = (float)ph.c, s = (float)ph.s, a0 = a.prm_f[0];
+    if (a.field_kind == QED_FIELD_ROTATING_E) {
+        const float E[3] = {a0 * c, a0 * s, 0.f};
+        return chi_bound(k, E, zero);
+    }
+    if (a.field_kind == QED_FIELD_STANDING_CP) {
+        const float E[3] = {0.f, a0 * c, a0 * s};
+        return chi_bound(k, E, zero);
+    }
+    const float E[3] = {a.prm_f[0], a.prm_f[1], a.prm_f[2]}, B[3] = {a.prm_f[3], a.prm_f[4], a.prm_f[5]};
+    return chi_bound(k, E, B);
+}
+
 // One waiting time of a photon of energy k0 and direction n at x, where the
 // field is (E, B), at clock tau (FRESH: the step start, tau = 0): the photon
 // flies to the step end (returns false) or to the point where it converts
@@ -436,7 +485,15 @@ __device__ __forceinline__ void fly_newborn(const LeptonCtx<T> &c, LeptonStack<T
         const T inv = f_div((T)1, k0);
         const T nx = kv[0] * inv, ny = kv[1] * inv, nz = kv[2] * inv;
         uint2 rz = make_uint2(0, 0);
-        if (photon_flight<T, false>(a, c.tm, c.coef, E, B, x, kv, k0, inv, nx, ny, nz, tau, id, rz, ps.n64)) {
+        bool flies = false;
+        if constexpr (sizeof(T) == 8) {
+            const float kf[3] = {(float)kv[0], (float)kv[1], (float)kv[2]}, Ef[3] = {(float)E[0], (float)E[1], (float)E[2]},
+                        Bf[3] = {(float)B[0], (float)B[1], (float)B[2]};
+            const double h = a.dt - tau;
+            flies = surely_flies(a, c.coef32, chi_bound(kf, Ef, Bf), (float)inv, (float)h, id, c.tm.step);
+            if (flies) { x[0] += nx * h; x[1] += ny * h; x[2] += nz * h; }
+        }
+        if (!flies && photon_flight<T, false>(a, c.tm, c.coef, E, B, x, kv, k0, inv, nx, ny, nz, tau, id, rz, ps.n64)) {
             alive = false;
             ++ps.pr;
             ps.mx = max(ps.mx, 1u);
@@ -589,7 +646,7 @@ __global__ void __launch_bounds__(LB<T>, (sizeof(T) == 4 && !MLP ? 3 : 2))
         __syncthreads();
         const unsigned gen_limit = (unsigned)ctl->pass_limit;
         const unsigned gen0 = FRESH ? 1u : (unsigned)ctl->step_passes + 1u;   // generation of the newborns waiting
-        const LeptonCtx<T> c{a, ctl, s_coef, reinterpret_cast<const T *>(a.icdf_em), ctl->capacity[2], gen_limit,
+        const LeptonCtx<T> c{a, ctl, s_coef, a.coef32, reinterpret_cast<const T *>(a.icdf_em), ctl->capacity[2], gen_limit,
                              (T)(ALPHA * RS), s_tm, time_phase<T, StepTime>(s_tm, 0.0)};
         // FP32 step-start pass: each thread stages its particle of the block's
         // next tile in shared memory while the block works on the current tile
@@ -806,7 +863,7 @@ __global__ void __launch_bounds__(LB<T>, 2) k_lepton_steps(const __grid_constant
             }
             __syncthreads();
             if (s_stop) break;                   // out of capacity: later steps do nothing
-            const LeptonCtx<T> c{a, ctl, s_coef, reinterpret_cast<const T *>(a.icdf_em), ctl->capacity[2], 0u,
+            const LeptonCtx<T> c{a, ctl, s_coef, a.coef32, reinterpret_cast<const T *>(a.icdf_em), ctl->capacity[2], 0u,
                                  (T)(ALPHA * RS), s_tm, s_ph};
             bool away = false;
             if (w > (T)0) {
@@ -846,6 +903,10 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_photon_pass(P
     __shared__ StepTime s_tm;
     if (blockIdx.x * NT < n) {
         for (int i = threadIdx.x; i < RateWords<T>::N; i += NT) s_coef[i] = reinterpret_cast<const T *>(a.coef)[i];
+        constexpr bool BOUND = sizeof(T) == 8 && !SFQ_GRID;
+        __shared__ __align__(16) float s_coef32[BOUND ? NRATE32 : 4];
+        if constexpr (BOUND)
+            for (int i = threadIdx.x; i < NRATE32; i += NT) s_coef32[i] = a.coef32[i];
         if (threadIdx.x == 0) s_tm = load_step_time(a);
         __syncthreads();
         const StepTime &tm = s_tm;
@@ -905,11 +966,21 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_photon_pass(P
             if (k0 > (T)0) {
                 const T inv = f_div((T)1, k0);
                 const T nx = kv[0] * inv, ny = kv[1] * inv, nz = kv[2] * inv;
+                bool flies = false;
+#if !SFQ_GRID
+                if constexpr (sizeof(T) == 8) {
+                    const float kf[3] = {(float)kv[0], (float)kv[1], (float)kv[2]};
+                    flies = surely_flies(a, s_coef32, chi_bound_start(a, ph0, kf), (float)inv, a.dt_f, id, tm.step);
+                }
+#endif
                 T E[3], B[3];
-                field_at<T>(a, x, ph0, E, B);
                 double tau = 0.0;
                 uint2 rz = make_uint2(0, 0);
-                if (photon_flight<T, true>(a, tm, s_coef, E, B, x, kv, k0, inv, nx, ny, nz, tau, id, rz, ps.n64)) {
+                if (flies) {
+                    const T h = dt_of<T>(a);
+                    x[0] += nx * h; x[1] += ny * h; x[2] += nz * h;
+                } else if (field_at<T>(a, x, ph0, E, B);
+                           photon_flight<T, true>(a, tm, s_coef, E, B, x, kv, k0, inv, nx, ny, nz, tau, id, rz, ps.n64)) {
                     pair_create<T>(a, tm, icdf, x, kv, k0, nx, ny, nz, tau, w, id, 0u, rz, ps.n64,
                                    [](int, unsigned) {});
                     st<T>(S.w, i, (T)0);       // the photon is eliminated
@@ -1144,7 +1215,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_lepton_od(Pas
     const unsigned long long b0 = ctl->begin[0], n0 = ctl->end[0] - b0;
     const unsigned long long b1 = ctl->begin[1], n1 = ctl->end[1] - b1;
     const unsigned long long n = n0 + n1;
-    const LeptonCtx<T> c{a, ctl, s_coef, reinterpret_cast<const T *>(a.icdf_em), ctl->capacity[2], 0u, (T)(ALPHA * RS),
+    const LeptonCtx<T> c{a, ctl, s_coef, a.coef32, reinterpret_cast<const T *>(a.icdf_em), ctl->capacity[2], 0u, (T)(ALPHA * RS),
                          tm, time_phase<T, StepTime>(tm, 0.0)};
     PassStats ps;
     for (unsigned long long j = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; j < n;

@@ -491,6 +491,7 @@ static qed_status enqueue_steps(qed_ctx *ctx, const qed_field_desc *field, doubl
     a.ctl = ctx->ctl;
     const bool f32 = sizeof(T) == 4;
     a.coef = f32 ? (const void *)ctx->coef32 : (const void *)ctx->coef64;
+    a.coef32 = ctx->coef32;
     a.icdf_em = f32 ? (const void *)ctx->icdf_em32 : (const void *)ctx->icdf_em64;
     a.icdf_pair = f32 ? (const void *)ctx->icdf_pair32 : (const void *)ctx->icdf_pair64;
     a.mlp_w16 = ctx->cfg.sampler == QED_SAMPLER_MLP ? ctx->mlp_w16 : nullptr;
