@@ -462,9 +462,10 @@ __device__ __forceinline__ float add_sr(float x, float dx, unsigned long long id
 // id, the step and its iteration k).  q = -1 (e-) or +1 (e+).  no_b: B = 0
 // wherever the field is evaluated (the rotation is the identity and is
 // skipped).  FP32 mode takes 1/gamma from the hardware reciprocal square root
-// and the rotation factor from the fast division.
+// and the rotation factor from the fast division.  SPLIT (FP64): the products
+// of the position update rounded on their own.
 // ---------------------------------------------------------------------------
-template <class T>
+template <class T, bool SPLIT = false>
 __device__ __forceinline__ void boris(T x[3], T p[3], T q, const T E[3], const T B[3], T h, bool no_b,
                                       unsigned long long id, unsigned step, unsigned k) {
     const T qh2 = (T)0.5 * q * h;
@@ -486,9 +487,15 @@ __device__ __forceinline__ void boris(T x[3], T p[3], T q, const T E[3], const T
     p[2] = m2 + qh2 * E[2];
     if constexpr (sizeof(T) == 8) {
         const double vh = h / sqrt(1.0 + p[0] * p[0] + p[1] * p[1] + p[2] * p[2]);
-        x[0] += p[0] * vh;
-        x[1] += p[1] * vh;
-        x[2] += p[2] * vh;
+        if constexpr (SPLIT) {
+            x[0] = __dadd_rn(x[0], __dmul_rn(p[0], vh));
+            x[1] = __dadd_rn(x[1], __dmul_rn(p[1], vh));
+            x[2] = __dadd_rn(x[2], __dmul_rn(p[2], vh));
+        } else {
+            x[0] += p[0] * vh;
+            x[1] += p[1] * vh;
+            x[2] += p[2] * vh;
+        }
     } else {
         const float vh = h * rsqrtf(1.0f + p[0] * p[0] + p[1] * p[1] + p[2] * p[2]);
         x[0] = add_sr(x[0], __fmul_rn(p[0], vh), id, step, 3u * k);

@@ -169,6 +169,7 @@ __device__ __forceinline__ void note_overflow(DevCtl *ctl, int s, unsigned long 
 // step: 87 us at 256 threads, 79 us at 128).
 template <class T> constexpr int LB = sizeof(T) == 4 ? 256 : 128;
 constexpr unsigned RESUME = 0x80000000u;   // stack item flag: no event pending (a newborn at its birth clock)
+constexpr unsigned START = 0x40000000u;    // with it: a lepton at the step start (its first waiting time to be drawn)
 
 template <class T> struct LeptonStack {
     static constexpr int Q = 2 * LB<T>;    // items: < LB left + LB pushed
@@ -233,9 +234,9 @@ __device__ __forceinline__ bool advance(const LeptonCtx<T> &c, T x[3], T p[3], T
     if constexpr (FRESH) field_at<T>(a, x, c.ph0, E, B);
     else field_tau<T>(a, c.tm, x, tau, E, B);
     T gam, chi, p2;
-    // after an event the copy of this code depends on what surrounds it: its
-    // sums are rounded explicitly
-    lepton_chi<T, !FRESH>(p, E, B, gam, chi, p2, n64, a.field_zero);
+    // in a round the copy of this code depends on what surrounds it: its sums
+    // are rounded explicitly
+    lepton_chi<T, !FRESH || sizeof(T) == 8>(p, E, B, gam, chi, p2, n64, a.field_zero);
     const T lam = p2 > (T)0 ? f_div(c.alpha_r, gam) * rate_em<T>(c.coef, chi) : (T)0;
     T dth = t_inf<T>();
     if (lam > lam_skip<T>(a)) {
@@ -354,6 +355,36 @@ __device__ __forceinline__ void pair_create(const PassArgs &a, const StepTime &t
     } else {
         note_overflow(ctl, 1, sp);
     }
+}
+
+// FP64 mode, a lepton at the step start: whether it surely has no event in the
+// step, decided in FP32 as for photons (surely_flies below).  The lepton is
+// then only pushed; the others go to the stack, where their waiting times are
+// drawn in FP64, densely.  The emission rate grows with chi too.  (One
+// emission in seven lepton-steps: 20 steps of the paper's test problem at
+// 5e5 photons 15.4 -> 12.5 ms, 200 steps of 16384 electrons 9.8 -> 8.8 ms.)
+__device__ __forceinline__ bool surely_calm(const LeptonCtx<double> &c, const double p[3], const double E[3],
+                                            const double B[3], unsigned long long id) {
+    const PassArgs &a = c.a;
+    const float k[3] = {(float)p[0], (float)p[1], (float)p[2]};
+    const float Ef[3] = {(float)E[0], (float)E[1], (float)E[2]}, Bf[3] = {(float)B[0], (float)B[1], (float)B[2]};
+    const float p2 = k[0] * k[0] + k[1] * k[1] + k[2] * k[2], gam = sqrtf(1.0f + p2);
+    // chi R <= |gamma E_perp| + |E along p| + |p x B|, each bounded with its rounding
+    const float ax = k[1] * Ef[2] - k[2] * Ef[1], ay = k[2] * Ef[0] - k[0] * Ef[2], az = k[0] * Ef[1] - k[1] * Ef[0];
+    const float bx = k[1] * Bf[2] - k[2] * Bf[1], by = k[2] * Bf[0] - k[0] * Bf[2], bz = k[0] * Bf[1] - k[1] * Bf[0];
+    const float e2 = Ef[0] * Ef[0] + Ef[1] * Ef[1] + Ef[2] * Ef[2];
+    const float sum = (fabsf(k[0]) + fabsf(k[1]) + fabsf(k[2])) *
+                      (fabsf(Ef[0]) + fabsf(Ef[1]) + fabsf(Ef[2]) + fabsf(Bf[0]) + fabsf(Bf[1]) + fabsf(Bf[2]));
+    float chi;
+    if (a.field_zero) chi = sqrtf(e2 + ax * ax + ay * ay + az * az + bx * bx + by * by + bz * bz);     // E.(p x B) = 0
+    else chi = sqrtf(e2 + ax * ax + ay * ay + az * az) + sqrtf(bx * bx + by * by + bz * bz);
+    chi = (chi + sum * 0x1p-21f) * (float)(1.0 / RS) * 1.0001f;
+    const float lam = (float)(ALPHA * RS) / gam * rate_em<float>(c.coef32, chi);
+    const uint4 r = event_draw(a.keys, id, c.tm.step, 0u);
+    float u, v;
+    Uniform<float>::draw(r.x, r.y, u, v);
+    // -ln u to 1e-6 in FP32, the rate bound's 1% aside
+    return Uniform<float>::neglog(u, v) > lam * a.dt_f * 1.01f;
 }
 
 // A copy of v that the compiler does not see through.  Sub-expressions shared
@@ -561,7 +592,8 @@ __device__ __forceinline__ void stack_round(const LeptonCtx<T> &c, LeptonStack<T
     }
     __syncthreads();                                // the popped places may now be pushed to
     const bool event = !(gen & RESUME);
-    gen &= ~RESUME;
+    const bool start = sizeof(T) == 8 && mine && (gen & START);
+    gen &= ~(RESUME | START);
     // the event at the particle's current point: chi there, energy fraction
     // from the inverse CDF (or the network: the whole warp evaluates it for
     // its 32 items on the tensor cores), then the kinematics
@@ -605,7 +637,10 @@ __device__ __forceinline__ void stack_round(const LeptonCtx<T> &c, LeptonStack<T
     }
     if (mine) {
         const T qch = (idx >> 31) ? (T)1 : (T)-1;
-        if (before_step_end(tau, c.a.dt) && advance<T, false>(c, x, p, qch, tau, id, k, rz, ps.n64)) {
+        bool again;
+        if (start) again = advance<T, true>(c, x, p, qch, tau, id, 0u, rz, ps.n64);
+        else again = before_step_end(tau, c.a.dt) && advance<T, false>(c, x, p, qch, tau, id, k, rz, ps.n64);
+        if (again) {
             stack_push<T>(q, pos, x, p, tau, id, w, idx, k, gen, rz);
         } else {
             finish<T>(c.a, idx, x, p, k);
@@ -720,7 +755,16 @@ __global__ void __launch_bounds__(LB<T>, (sizeof(T) == 4 && !MLP ? 3 : 2))
                         ++ps.lep;
                         uint2 rz = make_uint2(0, 0);
                         const T qch = s == 0 ? (T)-1 : (T)1;
-                        if (advance<T, true>(c, x, p, qch, tau, id, 0u, rz, ps.n64)) {
+                        if constexpr (sizeof(T) == 8) {
+                            T E[3], B[3];
+                            field_at<T>(a, x, c.ph0, E, B);
+                            if (surely_calm(c, p, E, B, id)) {
+                                boris<T, true>(x, p, qch, E, B, a.dt, a.field_zero == 1, id, c.tm.step, 0u);
+                                finish<T>(a, idx, x, p, 0u);
+                            } else {
+                                stack_push<T>(q, pos, x, p, tau, id, w, idx, 0u, RESUME | START, rz);
+                            }
+                        } else if (advance<T, true>(c, x, p, qch, tau, id, 0u, rz, ps.n64)) {
                             stack_push<T>(q, pos, x, p, tau, id, w, idx, 0u, 0u, rz);
                         } else {
                             finish<T>(a, idx, x, p, 0u);
@@ -870,8 +914,16 @@ __global__ void __launch_bounds__(LB<T>, 2) k_lepton_steps(const __grid_constant
                 double tau = 0.0;
                 ++ps.lep;
                 uint2 rz = make_uint2(0, 0);
-                away = advance<T, true>(c, x, p, qch, tau, id, 0u, rz, ps.n64);
-                if (away) stack_push<T>(q, pos, x, p, tau, id, w, idx, 0u, 0u, rz);
+                if constexpr (sizeof(T) == 8) {
+                    T E[3], B[3];
+                    field_at<T>(a, x, c.ph0, E, B);
+                    away = !surely_calm(c, p, E, B, id);
+                    if (away) stack_push<T>(q, pos, x, p, tau, id, w, idx, 0u, RESUME | START, rz);
+                    else boris<T, true>(x, p, qch, E, B, a.dt, a.field_zero == 1, id, c.tm.step, 0u);
+                } else {
+                    away = advance<T, true>(c, x, p, qch, tau, id, 0u, rz, ps.n64);
+                    if (away) stack_push<T>(q, pos, x, p, tau, id, w, idx, 0u, 0u, rz);
+                }
             }
             next_iteration();
             while (pos.n > 0) {

@@ -1,5 +1,5 @@
-"""FP64 photons whose flight to the step end is decided by a bound in FP32:
-against the oracle, decision by decision, over photon energies and directions
+"""FP64 photons whose flight to the step end, and FP64 leptons whose step
+without an event, is decided by a bound in FP32: against the oracle, decision by decision, over photon energies and directions
 from far below the pair threshold to chi of several hundred, in every analytic
 field (along and across the field, at rest-frame extremes)."""
 import numpy as np
@@ -46,3 +46,37 @@ def test_photons_fp64(kind, prm, n):
     assert np.array_equal(a["id"][i], b["id"][j])
     for c in ("x", "y", "z"):
         assert np.allclose(a[c][i], b[c][j], rtol=0, atol=1e-12)
+
+
+@pytest.mark.parametrize("kind,prm", FIELDS)
+@pytest.mark.parametrize("n,steps,photons", [(1, 3, 1), (129, 3, 0), (20000, 2, 1), (20000, 3, 0)])
+def test_leptons_fp64(kind, prm, n, steps, photons):
+    r = np.random.default_rng(n + steps)
+    k = np.exp(r.uniform(np.log(1e-4), np.log(1e5), n))
+    k[::11] = 0.0                                          # at rest
+    v = r.standard_normal((n, 3))
+    v[: n // 5] *= [1.0, 1e-9, 1e-9]
+    v *= (k / np.linalg.norm(v, axis=1))[:, None]
+    sp = []
+    for s in range(2):
+        d = {c: r.uniform(-40, 40, n) for c in ("x", "y", "z")}
+        d.update({c: v[:, i] for i, c in enumerate(("px", "py", "pz"))})
+        d.update(w=np.ones(n), id=np.arange(n, dtype=np.uint64) + (s << 40))
+        sp.append(d)
+    cap = [n + 50000, n + 50000, 400000]
+    g = q.Generator(q.make_config(precision=q.QED_FP64, seed=6, push_photons=photons))
+    ens = q.DeviceEnsemble.from_host(sp + [W._empty()], cap, q.QED_FP64)
+    st = g.push(ens, q.make_field(kind, prm), W.TWO_PI / 100, steps, 3, auto_grow=False)
+    g.close()
+    o = oracle.Ensemble.from_arrays(sp + [W._empty()], cap)
+    ost = oracle.push_and_generate(o, oracle.build_tables(),
+                                   oracle.make_cfg(seed=6, push_photons=photons, field_kind=kind, field_prm=prm),
+                                   W.TWO_PI / 100, steps, 3)
+    for key in ("particle_steps", "emit_events", "pair_events"):
+        assert st[key] == ost[key], key
+    for s in range(2):
+        a, b = ens.to_host(s), o.view(s)
+        i, j = np.argsort(a["id"]), np.argsort(b["id"])
+        assert np.array_equal(a["id"][i], b["id"][j]) and np.array_equal(a["nevents"][i], b["nevents"][j])
+        pa, pb = (np.stack([d[c][m] for c in ("px", "py", "pz")]) for d, m in ((a, i), (b, j)))
+        assert np.max(np.linalg.norm(pa - pb, axis=0) / np.maximum(np.linalg.norm(pb, axis=0), 1e-3)) < 1e-5
