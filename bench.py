@@ -41,12 +41,23 @@ sys.path.insert(0, ROOT)
 from paper_2409_17299_gb300 import workloads as W  # noqa: E402  (no CUDA, no method arithmetic)
 
 # algorithmic bytes per particle-step of the lepton pass (read x,y,z,px,py,pz,w + id;
-# write x,y,z,px,py,pz) and per emission (nevents update + photon record + birth clock)
+# write x,y,z,px,py,pz) and per emission (nevents update + photon record, written
+# once where the photon's flight ends)
 LEPTON_BYTES = {"fp32": 7 * 4 + 8 + 6 * 4, "fp64": 7 * 8 + 8 + 6 * 8}
-EMIT_BYTES = {"fp32": 8 + 7 * 4 + 8 + 4 + 8, "fp64": 8 + 7 * 8 + 8 + 4 + 8}
-# photon step: read w, x, k, id; write x.  Pair: photon weight cleared, two
+EMIT_BYTES = {"fp32": 8 + 7 * 4 + 8 + 4, "fp64": 8 + 7 * 8 + 8 + 4}
+# photon step: read w, x, k, id; write x (photons born in the step fly in the
+# lepton pass and move no bytes of their own).  Pair: photon weight cleared, two
 # lepton records (x, p, w, id, nevents, birth clock)
 PHOTON_BYTES = {"fp32": 4 + 3 * 4 + 3 * 4 + 8 + 3 * 4, "fp64": 8 + 3 * 8 + 3 * 8 + 8 + 3 * 8}
+
+
+def photon_pass_bytes(prec, tot):
+    """Algorithmic bytes of the photon pass: the photons present at the step
+    starts (each emission is one photon that flies in the lepton pass)."""
+    return (PHOTON_BYTES[prec] * max(0, tot["photon_steps"] - tot["emit_events"])
+            + PAIR_BYTES[prec] * tot["pair_events"])
+
+
 PAIR_BYTES = {"fp32": 4 + 2 * (7 * 4 + 8 + 4 + 8), "fp64": 8 + 2 * (7 * 8 + 8 + 4 + 8)}
 # optical-depth scheme, per particle-step: the same records plus the optical
 # depth (working precision) read and written
@@ -60,13 +71,15 @@ OD_PHOTON_BYTES = {"fp32": PHOTON_BYTES["fp32"] + 8, "fp64": PHOTON_BYTES["fp64"
 # profiles/k_photon_pass_fp32_rotating_e_cascade.md and
 # profiles/k_lepton_pass_fp32_rotating_e_cascade.md.  None when the kernel
 # changed since its capture.
-NCU_PHOTON_BYTES_PER_STEP = {"fp32": 47.6, "fp64": None}
-NCU_LEPTON_BYTES_PER_STEP = {"fp32": 80.1, "fp64": None}
+NCU_PHOTON_BYTES_PER_STEP = {"fp32": None, "fp64": None}
+NCU_LEPTON_BYTES_PER_STEP = {"fp32": None, "fp64": None}
 # FP64 FLOPs (2 DFMA + DADD + DMUL thread instructions) per particle-step of
 # the FP64 step-start passes at the rotating-E cascade's cap (0.3 emissions
 # per lepton-step): the launch's count over the particles it pushed, from one
-# ncu capture of the current kernels (profiles/fp64_passes_rotating_e_cascade.md)
-NCU_FP64_FLOP_PER_STEP = {"k_lepton_pass": 481.7, "k_photon_pass": 206.0}
+# ncu capture.  None: the kernels changed since their capture
+# (profiles/fp64_passes_rotating_e_cascade.md: 481.7 and 206.0 before most
+# particles' steps were decided in FP32)
+NCU_FP64_FLOP_PER_STEP = {"k_lepton_pass": None, "k_photon_pass": None}
 # algorithmic FLOPs per training sample of the 2-64-64-64-1 network: forward
 # 2 x (2*64 + 64*64 + 64*64 + 64) multiply-adds, backward the two 64x64 input
 # gradients, the two 64x64 weight gradients, W1's and W4's gradients
@@ -423,7 +436,7 @@ def gpu_run(args, w, precision, start, warm, steps, profile=False, mlp_params=No
     gen.close()
     del ens, flush
     torch.cuda.empty_cache()
-    st["lepton_launches"] = steps + st["passes"]
+    st["lepton_launches"] = steps
     st["counts_start"] = counts0
     st["gpu_idle_ms"] = idle
     st["host_enqueue_ms"] = host_in_loop * 1e3
@@ -736,7 +749,7 @@ def main():
                                   profile=True)
         pr = args.precision
         lb = LEPTON_BYTES[pr] * tot_mp["lepton_steps"] + EMIT_BYTES[pr] * tot_mp["emit_events"]
-        pb = PHOTON_BYTES[pr] * tot_mp["photon_steps"] + PAIR_BYTES[pr] * tot_mp["pair_events"]
+        pb = photon_pass_bytes(pr, tot_mp)
         lk, pk = tot_mp["kernel_ms"][0], tot_mp["kernel_ms"][1]
         mlp["roofline"] = {
             "k_lepton_pass (network sampler)": {"kernel_ms": lk, "achieved_gbs": lb / (lk / 1e3) / 1e9 if lk > 0 else None,
@@ -821,7 +834,7 @@ def main():
         return
     prec = args.precision
     lep_bytes = LEPTON_BYTES[prec] * tot["lepton_steps"] + EMIT_BYTES[prec] * tot["emit_events"]
-    ph_bytes = PHOTON_BYTES[prec] * tot["photon_steps"] + PAIR_BYTES[prec] * tot["pair_events"]
+    ph_bytes = photon_pass_bytes(prec, tot) if w.push_photons else 0
     lep_ms, ph_ms = tot["kernel_ms"][0], tot["kernel_ms"][1]
     launches = max(1, tot["lepton_launches"])
     kernels = {
@@ -1060,12 +1073,12 @@ def fp64_roofline(tot, hbm_peak):
     for k, ms, units, nbytes in (("k_lepton_pass", tot["kernel_ms"][0], tot["lepton_steps"],
                                   LEPTON_BYTES["fp64"] * tot["lepton_steps"] + EMIT_BYTES["fp64"] * tot["emit_events"]),
                                  ("k_photon_pass", tot["kernel_ms"][1], tot["photon_steps"],
-                                  PHOTON_BYTES["fp64"] * tot["photon_steps"] + PAIR_BYTES["fp64"] * tot["pair_events"])):
+                                  photon_pass_bytes("fp64", tot))):
         if ms <= 0:
             continue
-        fl = NCU_FP64_FLOP_PER_STEP[k] * units / (ms / 1e3)
+        fl = NCU_FP64_FLOP_PER_STEP[k] * units / (ms / 1e3) if NCU_FP64_FLOP_PER_STEP[k] else None
         gbs = nbytes / (ms / 1e3) / 1e9
-        out["kernels"][k] = {"kernel_ms": ms, "achieved": fl, "frac": fl / peak,
+        out["kernels"][k] = {"kernel_ms": ms, "achieved": fl, "frac": fl / peak if fl else None,
                              "flop_per_particle_step": NCU_FP64_FLOP_PER_STEP[k],
                              "hbm_gbs": gbs, "hbm_frac": gbs / hbm_peak}
     dom = max(out["kernels"], key=lambda k: out["kernels"][k]["kernel_ms"]) if out["kernels"] else None
