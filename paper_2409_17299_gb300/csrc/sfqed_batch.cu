@@ -297,8 +297,21 @@ __device__ __forceinline__ void fused_round(const FusedCtx &c, FusedStack<T, NT>
     __syncthreads();
 }
 
-template <class T, int NT>
-__global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT == 128 ? 7 : 1)) k_emission_fused(BatchArgs b) {
+// DENSE (FP32): 32 warps per SM at every block shape (64 registers, 32 bytes
+// spilled), for calls whose tiles fill the chip.  The rounds' barriers and
+// dependent instructions leave the issue slots 40% idle at 16 warps (86
+// registers, what the compiler takes by itself).  64 bunches of 250 to 250000
+// leptons, 50 steps, 256 threads: 8.15 ms with 16 warps, 6.56 with 24, 6.08
+// with 32, 6.65 with 40 (48 registers); 32 warps in blocks of 128: 6.10, of
+// 512: 6.43.  A call of which every block of the roomy kernel gets at most
+// one tile gains nothing from more warps and keeps that kernel (3 bunches of
+// 20 to 20000 leptons, 10 steps: 0.213 ms, dense 0.229).
+template <class T, int NT, bool DENSE> constexpr int fused_min_blocks() {
+    return sizeof(T) == 4 ? (DENSE ? 1024 / NT : NT == 128 ? 7 : 1) : 1;
+}
+
+template <class T, int NT, bool DENSE>
+__global__ void __launch_bounds__(NT, fused_min_blocks<T, NT, DENSE>()) k_emission_fused(BatchArgs b) {
     __shared__ __align__(16) T s_coef[RateWords<T>::N];
     __shared__ FusedStack<T, NT> q;
     __shared__ unsigned long long s_tile;
@@ -377,21 +390,32 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT == 128 ? 7 : 1)) k_e
     }
 }
 
-template <class T, int NT> static int fused_blocks(const qed_ctx *ctx) {
+template <class T, int NT, bool DENSE> static int fused_blocks(const qed_ctx *ctx) {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_emission_fused<T, NT>, NT, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_emission_fused<T, NT, DENSE>, NT, 0) != cudaSuccess ||
         per_sm < 1)
         per_sm = 1;
     if (ctx->cfg.blocks_per_sm > 0 && ctx->cfg.blocks_per_sm < per_sm) per_sm = ctx->cfg.blocks_per_sm;
     return ctx->sm_count * per_sm;
 }
 
+template <class T, int NT> static void launch_shape(const qed_ctx *ctx, const BatchArgs &b, cudaStream_t st) {
+    const int blocks = fused_blocks<T, NT, false>(ctx);
+    if constexpr (sizeof(T) == 4) {
+        if (b.n_tiles > (unsigned long long)blocks) {
+            k_emission_fused<T, NT, true><<<fused_blocks<T, NT, true>(ctx), NT, 0, st>>>(b);
+            return;
+        }
+    }
+    k_emission_fused<T, NT, false><<<blocks, NT, 0, st>>>(b);
+}
+
 template <class T>
 static cudaError_t launch_fused(const qed_ctx *ctx, int nt, const BatchArgs &b, cudaStream_t st) {
     switch (nt) {
-    case 128: k_emission_fused<T, 128><<<fused_blocks<T, 128>(ctx), 128, 0, st>>>(b); break;
-    case 512: k_emission_fused<T, 512><<<fused_blocks<T, 512>(ctx), 512, 0, st>>>(b); break;
-    default: k_emission_fused<T, 256><<<fused_blocks<T, 256>(ctx), 256, 0, st>>>(b); break;
+    case 128: launch_shape<T, 128>(ctx, b, st); break;
+    case 512: launch_shape<T, 512>(ctx, b, st); break;
+    default: launch_shape<T, 256>(ctx, b, st); break;
     }
     return cudaGetLastError();
 }
