@@ -96,8 +96,9 @@ typedef struct {
                                  step, one born of it in the same step, ...) a step may
                                  run; a step that needs more stops there and the call
                                  returns QED_ERR_TIMEOUT; 0 = 100000 */
-    int wait_polls;           /* polls of each grid barrier inside qed_train_surrogate
-                                 before the launch gives up (QED_ERR_TIMEOUT); 0 = 2^24 */
+    int wait_polls;           /* polls of each wait of one block for another inside
+                                 qed_train_surrogate before the launch gives up
+                                 (QED_ERR_TIMEOUT); 0 = 2^24 */
     int reserved[1];
 } qed_config;
 
@@ -272,10 +273,12 @@ qed_status qed_batch_shape(qed_ctx *ctx, int *threads, int *step_budget);
  * by the emission table, in batches of `batch` (a multiple of 128): forward
  * and backward passes on the tensor cores (tcgen05, accumulators in tensor
  * memory), Adam, learning rate decaying from lr to lr/100 (cosine).  Every
- * step runs inside one cooperative launch (one CTA per SM at most, a grid
- * barrier per step); the call allocates its scratch, blocks until the
- * launch ends and frees it.  *final_loss (may be NULL): mean squared error
- * over the last 16 batches.  QED_ERR_TIMEOUT if a grid barrier or a
+ * step runs inside one cooperative launch (one CTA per SM at most); the call
+ * blocks until the launch ends.  Its scratch (69 KB per CTA, 8 bytes per
+ * step) stays in the context until qed_destroy.  Gradients are summed over
+ * the CTAs in a fixed order: the same arguments give the same bits on the
+ * same GPU model.  *final_loss (may be NULL): mean squared error over the
+ * last 16 batches.  QED_ERR_TIMEOUT if a wait for another CTA's data or a
  * tensor-core wait inside the launch ran out (bounded waits); the
  * parameters are then left as they were before the call's first step
  * (the freshly initialised network). */

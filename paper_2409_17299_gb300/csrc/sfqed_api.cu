@@ -13,7 +13,7 @@ static void free_ctx(qed_ctx *c) {
     sfq_step_graph_free(c);
     void *dev[] = {c->coef64, c->coef32, c->icdf_em64, c->icdf_pair64, c->icdf_em32, c->icdf_pair32,
                    c->ctl, c->tau[0], c->tau[1], c->blk, c->slots, c->snap, c->lev,
-                   c->mlp_p, c->mlp_w16, c->mlp_loss};
+                   c->mlp_p, c->mlp_w16, c->mlp_scratch};
     for (void *p : dev)
         if (p) cudaFree(p);
     if (c->ctl_host) cudaFreeHost(c->ctl_host);

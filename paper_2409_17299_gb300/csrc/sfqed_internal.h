@@ -219,10 +219,11 @@ struct qed_ctx {
     int async_deferred;          // the open batch's steps may have left dead entries in place
     int step_graph_failed;       // conditional graph nodes unavailable: host-driven steps
     // surrogate network: FP32 master parameters, Adam moments and gradient
-    // (4 x 8577 floats), BF16 copy used by the kernels, loss accumulator
+    // (4 x 8577 floats), BF16 copy used by the kernels
     float *mlp_p;
     __nv_bfloat16 *mlp_w16;
-    float *mlp_loss;
+    void *mlp_scratch;           // work memory of the training and gradient calls
+    size_t mlp_scratch_bytes;
     int mlp_ready;
 };
 

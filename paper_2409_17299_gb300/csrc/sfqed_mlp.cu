@@ -6,8 +6,8 @@
 // It is trained on samples drawn from the table method itself; the table is
 // kept as the fallback outside the trained range.  Training (k_mlp_train
 // below): forward and backward products of 128-sample tiles on the tcgen05
-// tensor cores with accumulators in tensor memory, gradients summed in FP32,
-// Adam, all steps in one cooperative launch.
+// tensor cores with accumulators in tensor memory, gradients summed in FP32
+// in a fixed order, Adam, all steps in one cooperative launch.
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -25,12 +25,9 @@ namespace {
 // ---- training on the tensor cores (tcgen05, accumulators in tensor memory)
 //
 // One persistent cooperative kernel runs every optimizer step.  A CTA holds
-// 128 samples at a time (one per tensor-memory lane) and keeps, in shared
-// memory, its own copy of the FP32 parameters and Adam moments: every CTA
-// applies the same Adam update to the same summed gradient, so the copies
-// stay identical and one grid barrier per step suffices.  512 threads: the
-// four warps that share a lane quadrant split the 64 columns of their 32
-// samples, 16 each.
+// 128 samples at a time (one per tensor-memory lane).  512 threads: the four
+// warps that share a lane quadrant split the 64 columns of their 32 samples,
+// 16 each.
 //
 // Per tile of 128 samples (B = BF16 storage, as in the network the oracle
 // defines; Z and dy stay FP32):
@@ -43,9 +40,24 @@ namespace {
 // Layer 1 (2 -> 64) and layer 4 (64 -> 1) run on the CUDA cores.  The SiLU
 // derivatives are computed in the forward pass and kept in tensor memory
 // until the backward pass multiplies them in.  G1 and G2 accumulate over
-// the CTA's tiles of a step and are added to the step's gradient sum with
-// vector atomics.  Features and dy enter G2 as BF16 hi + lo pairs, so the
-// BF16 operand rounding leaves them exact to about 2^-17.
+// the CTA's tiles of a step.  Features and dy enter G2 as BF16 hi + lo pairs,
+// so the BF16 operand rounding leaves them exact to about 2^-17.
+//
+// The gradient sum has a fixed order: every CTA writes its share to a slot of
+// its own, and the CTA that owns a group of four parameters (a contiguous run
+// of groups each) adds the slots' values in the order of the CTAs, applies
+// Adam to them and hands the new BF16 weights to all CTAs.  Added by atomics
+// in the order of arrival, the sums differed in their last bits from run to
+// run, and the BF16 rounding of the weights carried that to 1e-4 of the loss
+// after 32 steps.  Slots and weights travel in 64-bit words that hold the
+// value and the step's tag, so that a word is complete when its tag is there:
+// a step takes two one-way exchanges and no grid barrier.  A slot is free
+// again when the weights of its step have arrived, since an owner sends them
+// after it has read every slot.
+// What a step costs (GB300, its chain of dependent phases; atomics and a grid
+// barrier before -> now): 10.2 -> 10.3 us with 1 CTA, 10.4 -> 10.9 with 8,
+// 10.9 -> 11.2 with 64, 14.1 -> 12.4 with 152, 19.3 -> 18.1 with two tiles
+// each; FP64 atomics, whose order matters no more, took 13.8 with 64.
 constexpr int TT = 512;                       // threads
 constexpr int TS = 128;                       // samples per tile = tensor-memory lanes
 constexpr int GSTRIDE = 8580;                 // MLP_NP rounded up to whole float4s
@@ -70,16 +82,17 @@ static_assert(MLP_B1 % 4 == 0 && MLP_W2 % 4 == 0 && MLP_B2 % 4 == 0 && MLP_W3 % 
 static_assert(TR_SMEM <= 227 * 1024, "shared memory");
 // tensor-memory columns: products, SiLU derivatives of layers 1 and 2, gradients
 constexpr uint32_t TM_COLS = 512, TZ = 0, TD1 = 64, TD2 = 128, TG1 = 256, TG2 = 416;
-constexpr uint32_t WAIT_POLLS = 1u << 22, BAR_POLLS = 1u << 24;      // defaults of the bounded waits
+constexpr uint32_t WAIT_POLLS = 1u << 22, WORD_POLLS = 1u << 24;     // defaults of the bounded waits
 // instruction descriptors: forward (A, B K-major), backward (B MN-major), gradients
 constexpr uint32_t ID_FWD = tc::idesc_bf16(128, 64, 0, 0), ID_BWD = tc::idesc_bf16(128, 64, 0, 1);
 constexpr uint32_t ID_G1 = tc::idesc_bf16(128, 144, 1, 1), ID_G2 = tc::idesc_bf16(128, 16, 1, 1);
 
 struct TrainArgs {
-    float *P, *M, *V;                         // parameters and moments (read at start, written back at the end)
-    float *gbuf;                              // three gradient sums of GSTRIDE floats (zero at launch); the gradient
-    __nv_bfloat16 *W16;
-    float *loss;                              // sum of squared errors of the counted steps
+    const float *P, *M, *V;                   // parameters and moments at the start
+    float *out;                               // the same at the end, GSTRIDE values each
+    uint64_t *slots;                          // per CTA GSTRIDE words (tag << 32 | gradient; no tag set at launch)
+    uint64_t *weights;                        // GSTRIDE / 2 words (tag << 32 | two BF16 weights; the same)
+    double *loss;                             // per CTA: sum of squared errors of the counted steps
     const float *icdf_em32;                   // target generator (the table method)
     const float *feat, *target;               // given samples, or null: draw them
     const float *sched;                       // per step: lr / bias correction 1, 1 / bias correction 2
@@ -88,9 +101,8 @@ struct TrainArgs {
     long long steps;                          // optimizer steps; 0: one gradient, no update
     long long tail_from;                      // steps from here on add to *loss
     float inv_total;                          // 1 / per_step
-    unsigned *bar;                            // grid-barrier arrivals (zero at launch)
-    uint32_t bar_polls;                       // polls of a grid barrier before the launch gives up
-    int *status;                              // 0 ok, 1 a barrier wait ran out, 2 an MMA wait ran out
+    uint32_t polls;                           // polls of a word before the launch gives up
+    int *status;                              // 0 ok, 1 a wait for a word ran out, 2 an MMA wait ran out
 };
 
 // table target for (log10 chi, logit u) in the FP32 table's own arithmetic
@@ -130,43 +142,53 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
     return *reinterpret_cast<const uint32_t *>(&h);
 }
 
-// fire-and-forget additions to global memory (no value returned)
-__device__ __forceinline__ void red_add(float *p, float a) {
-    asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(a) : "memory");
+// Tagged words, each written and read as a whole (also as an element of a vector).
+__device__ __forceinline__ uint64_t word(uint32_t tag, uint32_t v) { return (uint64_t)tag << 32 | v; }
+__device__ __forceinline__ uint64_t word(uint32_t tag, float v) { return word(tag, __float_as_uint(v)); }
+__device__ __forceinline__ void put_words(uint64_t *p, uint64_t a, uint64_t b) {
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
 }
-__device__ __forceinline__ void red_add2(float *p, float a, float b) {
-    asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
+__device__ __forceinline__ void put_words(uint64_t *p, uint64_t a, uint64_t b, uint64_t c, uint64_t d) {
+    asm volatile("st.relaxed.gpu.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
 }
-__device__ __forceinline__ void red_add4(float *p, float a, float b, float c, float d) {
-    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
-                 : "memory");
+struct Words2 {
+    uint64_t v[2];
+    __device__ __forceinline__ void get(const uint64_t *p) {
+        asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "l"(p) : "memory");
+    }
+    __device__ __forceinline__ bool tagged(uint32_t t) const {
+        return (uint32_t)(v[0] >> 32) == t && (uint32_t)(v[1] >> 32) == t;
+    }
+};
+struct Words4 {
+    uint64_t v[4];
+    __device__ __forceinline__ void get(const uint64_t *p) {
+        asm volatile("ld.relaxed.gpu.global.v4.b64 {%0, %1, %2, %3}, [%4];"
+                     : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(p) : "memory");
+    }
+    __device__ __forceinline__ bool tagged(uint32_t t) const {
+        return (uint32_t)(v[0] >> 32) == t && (uint32_t)(v[1] >> 32) == t && (uint32_t)(v[2] >> 32) == t &&
+               (uint32_t)(v[3] >> 32) == t;
+    }
+};
+// w, read from p, until every word carries the tag; false when the polls run
+// out (the status word says so) or another wait's did
+template <class W>
+__device__ __forceinline__ bool await_words(const uint64_t *p, uint32_t tag, W &w, uint32_t polls, int *status) {
+    for (uint32_t it = 0; !w.tagged(tag); ++it) {
+        if (it >= polls || ((it & 255u) == 255u && *reinterpret_cast<volatile int *>(status))) {
+            atomicCAS(status, 0, 1);
+            return false;
+        }
+        w.get(p);
+    }
+    return true;
 }
 
 __device__ __forceinline__ float sqrt_approx(float x) {
     float y;
     asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
-}
-
-// all CTAs arrive; false when a wait ran out (the status word says which)
-__device__ bool grid_sync(unsigned *bar, unsigned target, uint32_t polls, int *status, int *s_flag) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(bar, 1u);
-        unsigned v = 0;
-        for (uint32_t it = 0; it < polls; ++it) {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if (v >= target || *reinterpret_cast<volatile int *>(status)) break;
-        }
-        if (v < target) {
-            atomicCAS(status, 0, 1);
-            *s_flag = 1;
-        }
-        __threadfence();
-    }
-    __syncthreads();
-    return *reinterpret_cast<volatile int *>(s_flag) == 0;
 }
 
 // 16 activations of one sample row (units u0..u0+15): pre-activation z (with
@@ -203,7 +225,6 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train(TrainArgs a) {
     float4 *sf = reinterpret_cast<float4 *>(sm + SM_SF);
     uint64_t *mbar = reinterpret_cast<uint64_t *>(sm + SM_MISC);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(sm + SM_MISC + 8);
-    int *s_flag = reinterpret_cast<int *>(sm + SM_MISC + 12);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int quad = warp & 3, cq = warp >> 2;       // lane quadrant; column quarter
     const int r = quad * 32 + lane, u0 = cq * 16;    // sample row; first unit of this thread
@@ -223,10 +244,7 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train(TrainArgs a) {
         *reinterpret_cast<uint4 *>(sm + SM_ZERO + tid * 16) = make_uint4(0u, 0u, 0u, 0u);
     }
     if (warp == 0) tc::alloc(tslot, TM_COLS);
-    if (tid == 0) {
-        tc::mbar_init(mbar, 1);
-        *s_flag = 0;
-    }
+    if (tid == 0) tc::mbar_init(mbar, 1);
     tc::fence_proxy_smem();
     tc::fence_before_sync();
     __syncthreads();
@@ -303,8 +321,15 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train(TrainArgs a) {
     const long long tiles = (a.per_step + TS - 1) / TS;
     const long long nsteps = train ? a.steps : 1;
     bool drawn = false;                              // sf already holds the next tile's samples
+    // this CTA's groups of four parameters, taken `width` at a time by `shares`
+    // threads each, which share the slots
+    constexpr int NG = GSTRIDE / 4;
+    const int own = (NG + gridDim.x - 1) / gridDim.x, g_lo = blockIdx.x * own, g_n = max(0, min(own, NG - g_lo));
+    const int width = min(own, TT), shares = min(TT / width, (int)gridDim.x), share = tid / width;
+    uint64_t *slot = a.slots + (size_t)blockIdx.x * GSTRIDE;
+    double loss = 0.0;
     for (long long s = 0; s < nsteps && ok; ++s) {
-        float *g = a.gbuf + (train ? (s % 3) * GSTRIDE : 0);
+        const uint32_t tag = (uint32_t)(s + 1);
         float dysum = 0.f, sq = 0.f;
         bool first = true;
         for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
@@ -401,38 +426,55 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train(TrainArgs a) {
             first = false;
         }
         if (!ok) break;
-        if (!first) {
-            // row r of G1: dW3 row r and db3 (r < 64), or dW2 row r - 64 and db2;
-            // this thread's 16 columns of it
-            const bool lo = r < 64;
-            float *gw = g + (lo ? MLP_W3 + r * 64 : MLP_W2 + (r - 64) * 64) + u0;
-            float v[16];
-            tc::ld16(tl + TG1 + (lo ? 0u : 64u) + u0, v);
-#pragma unroll
-            for (int q = 0; q < 16; q += 4)
-                red_add4(gw + q, v[q], v[q + 1], v[q + 2], v[q + 3]);
-            if (cq == 0) {
-                float v8[8];
-                tc::ld8(tl + TG1 + 128, v8);
-                red_add(g + (lo ? MLP_B3 + r : MLP_B2 + (r - 64)), v8[0]);
-                tc::ld8(tl + TG2, v8);
-                if (lo) {
-                    red_add2(g + MLP_W1 + 2 * r, v8[0] + v8[1], v8[2] + v8[3]);
-                    red_add(g + MLP_B1 + r, v8[4]);
-                } else {
-                    red_add(g + MLP_W4 + (r - 64), v8[5] + v8[6]);
-                }
-            }
-        }
         if (cq == 0) {
             for (int o = 16; o > 0; o >>= 1) {
                 dysum += __shfl_down_sync(0xffffffffu, dysum, o);
                 sq += __shfl_down_sync(0xffffffffu, sq, o);
             }
             if (lane == 0) {
-                if (dysum != 0.f) red_add(g + MLP_B4, dysum);
-                if (!train || s >= a.tail_from) red_add(a.loss, sq);
+                yp[quad] = dysum;
+                yp[4 + quad] = sq;
             }
+        }
+        {
+            // Row r of G1: dW3 row r and db3 (r < 64), or dW2 row r - 64 and
+            // db2; this thread's 16 columns of it (every CTA has a tile).
+            // Through shared memory (the operand tiles are free), so that the
+            // slot is written 1 KB at a time: from the rows directly every
+            // store touched 32 lines.
+            const bool lo = r < 64;
+            float v[16];
+            tc::ld16(tl + TG1 + (lo ? 0u : 64u) + u0, v);
+            float4 *stage = reinterpret_cast<float4 *>(sm + SM_H2);          // [128 rows][16], columns swizzled
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                stage[r * 16 + ((cq * 4 + q) ^ (r & 15))] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            if (cq == 0) {
+                float b[8], v8[8];
+                tc::ld8(tl + TG1 + 128, b);
+                tc::ld8(tl + TG2, v8);
+                // the single values of rows r and r + 1, r even, as pairs of words
+                const float bn = __shfl_down_sync(0xffffffffu, b[0], 1), b1n = __shfl_down_sync(0xffffffffu, v8[4], 1);
+                const float w4 = v8[5] + v8[6], w4n = __shfl_down_sync(0xffffffffu, w4, 1);
+                if (lo) put_words(slot + MLP_W1 + 2 * r, word(tag, v8[0] + v8[1]), word(tag, v8[2] + v8[3]));
+                if (!(r & 1)) {
+                    put_words(slot + (lo ? MLP_B3 + r : MLP_B2 + (r - 64)), word(tag, b[0]), word(tag, bn));
+                    if (lo) put_words(slot + MLP_B1 + r, word(tag, v8[4]), word(tag, b1n));
+                    else put_words(slot + MLP_W4 + (r - 64), word(tag, w4), word(tag, w4n));
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = tid + k * TT, row = i >> 4, c = i & 15;
+                const float4 f = stage[row * 16 + (c ^ (row & 15))];
+                put_words(slot + (row < 64 ? MLP_W3 + row * 64 : MLP_W2 + (row - 64) * 64) + 4 * c, word(tag, f.x),
+                          word(tag, f.y), word(tag, f.z), word(tag, f.w));
+            }
+        }
+        if (tid == 0) {
+            put_words(slot + MLP_B4, word(tag, ((yp[0] + yp[1]) + yp[2]) + yp[3]), word(tag, 0u), word(tag, 0u), word(tag, 0u));
+            if (!train || s >= a.tail_from) loss += (double)(((yp[4] + yp[5]) + yp[6]) + yp[7]);
         }
         if (!train) break;
         // the next step's first samples do not depend on the update: drawn
@@ -441,43 +483,90 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train(TrainArgs a) {
             draw(s + 1, blockIdx.x);
             drawn = true;
         }
-        // every CTA's sums are in: the same Adam update in every CTA
-        if (!grid_sync(a.bar, (unsigned)(gridDim.x * (s + 1)), a.bar_polls, a.status, s_flag)) {
-            ok = false;
-            break;
-        }
         const float lr_c = a.sched[2 * s], ibc2 = a.sched[2 * s + 1];
         const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-        // four consecutive parameters per thread and group (every region of
-        // the layout starts at a multiple of four, so a group never straddles
-        // two), all gradient loads in flight before the first use
-        constexpr int NG = GSTRIDE / 4, AG = (NG + TT - 1) / TT;
-        float4 gv[AG];
-#pragma unroll
-        for (int k = 0; k < AG; ++k) {
-            const int gi = tid + k * TT;
-            gv[k] = gi < NG ? __ldcg(reinterpret_cast<const float4 *>(g) + gi) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
         auto adam = [&](float gr, float &m, float &v, float &pp) {
             m = b1 * m + (1.f - b1) * gr;
             v = b2 * v + (1.f - b2) * gr * gr;
             pp = pp - __fdividef(lr_c * m, sqrt_approx(v * ibc2) + eps);
         };
-#pragma unroll
-        for (int k = 0; k < AG; ++k) {
-            const int gi = tid + k * TT, p = 4 * gi;
-            if (gi >= NG) break;
+        // This CTA's groups: the slots' sum (share k adds slots k, k + shares,
+        // ..., then the shares are added: the same order in every run), Adam,
+        // the new weights.  With few CTAs a thread has several groups (and
+        // all their slots), one after another.
+        bool got = true;
+        auto update = [&](int gi, const float4 &t) {
             float4 m4 = reinterpret_cast<float4 *>(sM)[gi], v4 = reinterpret_cast<float4 *>(sV)[gi];
             float4 p4 = reinterpret_cast<float4 *>(sP)[gi];
-            adam(gv[k].x, m4.x, v4.x, p4.x);
-            adam(gv[k].y, m4.y, v4.y, p4.y);
-            adam(gv[k].z, m4.z, v4.z, p4.z);
-            adam(gv[k].w, m4.w, v4.w, p4.w);
+            adam(t.x, m4.x, v4.x, p4.x);
+            adam(t.y, m4.y, v4.y, p4.y);
+            adam(t.z, m4.z, v4.z, p4.z);
+            adam(t.w, m4.w, v4.w, p4.w);
+            put_words(a.weights + 2 * gi, word(tag, pack2(p4.x, p4.y)), word(tag, pack2(p4.z, p4.w)));
             reinterpret_cast<float4 *>(sM)[gi] = m4;
             reinterpret_cast<float4 *>(sV)[gi] = v4;
             reinterpret_cast<float4 *>(sP)[gi] = p4;
-            // the BF16 values where the passes read them
-            const uint2 b = make_uint2(pack2(p4.x, p4.y), pack2(p4.z, p4.w));
+        };
+        {
+            constexpr int BATCH = 5;                 // slots in flight: all of a thread's at 64 CTAs
+            const int G = (int)gridDim.x;
+            float4 gr = make_float4(0.f, 0.f, 0.f, 0.f);
+            int ql = tid % width, kl = share, q = ql, k = share;     // group and slot: next to load, next to add
+            while (share < shares && q < g_n && got) {
+                Words4 w[BATCH];
+#pragma unroll
+                for (int i = 0; i < BATCH; ++i) {
+                    if (ql >= g_n) continue;
+                    w[i].get(a.slots + (size_t)kl * GSTRIDE + 4 * (g_lo + ql));
+                    if ((kl += shares) >= G) { kl = share; ql += width; }
+                }
+#pragma unroll
+                for (int i = 0; i < BATCH; ++i) {
+                    if (q >= g_n || !got) continue;
+                    got = await_words(a.slots + (size_t)k * GSTRIDE + 4 * (g_lo + q), tag, w[i], a.polls, a.status);
+                    gr.x += __uint_as_float((uint32_t)w[i].v[0]);
+                    gr.y += __uint_as_float((uint32_t)w[i].v[1]);
+                    gr.z += __uint_as_float((uint32_t)w[i].v[2]);
+                    gr.w += __uint_as_float((uint32_t)w[i].v[3]);
+                    if ((k += shares) >= G) {
+                        if (shares == 1 && got) {
+                            update(g_lo + q, gr);
+                            gr = make_float4(0.f, 0.f, 0.f, 0.f);
+                        }
+                        k = share;
+                        q += width;
+                    }
+                }
+            }
+            if (shares > 1) {
+                float4 *part = reinterpret_cast<float4 *>(sm + SM_D3);       // [shares][width]
+                if (share < shares) part[tid] = gr;
+                got = __syncthreads_and(got);
+                if (share == 0 && tid < g_n && got) {
+                    float4 t = part[tid];
+                    for (int i = 1; i < shares; ++i) {
+                        const float4 f = part[i * width + tid];
+                        t.x += f.x; t.y += f.y; t.z += f.z; t.w += f.w;
+                    }
+                    update(g_lo + tid, t);
+                }
+            }
+            __syncwarp();
+        }
+        // the new BF16 weights of every group, written where the passes read
+        // them (every region of the layout starts at a multiple of four, so a
+        // group never straddles two); all loads in flight before the first use
+        constexpr int AG = (NG + TT - 1) / TT;
+        Words2 nw[AG];
+#pragma unroll
+        for (int k = 0; k < AG; ++k)
+            if (tid + k * TT < NG) nw[k].get(a.weights + 2 * (tid + k * TT));
+#pragma unroll
+        for (int k = 0; k < AG; ++k) {
+            const int gi = tid + k * TT, p = 4 * gi;
+            if (gi >= NG || !got) break;
+            got = await_words(a.weights + 2 * gi, tag, nw[k], a.polls, a.status);
+            const uint2 b = make_uint2((uint32_t)nw[k].v[0], (uint32_t)nw[k].v[1]);
             if (p >= MLP_W2 && p < MLP_B2) {
                 const int q = p - MLP_W2;
                 *reinterpret_cast<uint2 *>(sm + SM_W2 + wtile_off(q >> 6, q & 63)) = b;
@@ -491,22 +580,39 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train(TrainArgs a) {
                 *reinterpret_cast<float4 *>(wq + d) = make_float4(bf16_lo(b.x), bf16_hi(b.x), bf16_lo(b.y), bf16_hi(b.y));
             }
         }
-        // the sum two steps ahead was last read before this step's barrier
-        float *gz = a.gbuf + ((s + 2) % 3) * GSTRIDE;
-        for (int p = blockIdx.x * TT + tid; p < GSTRIDE; p += gridDim.x * TT) __stcg(gz + p, 0.f);
-        __syncthreads();
+        ok = __syncthreads_and(got);
     }
-    if (train && ok && blockIdx.x == 0) {
-        for (int p = tid; p < MLP_NP; p += TT) {
-            a.P[p] = sP[p];
-            a.M[p] = sM[p];
-            a.V[p] = sV[p];
-            a.W16[p] = __float2bfloat16_rn(sP[p]);
+    if (tid == 0) a.loss[blockIdx.x] = loss;
+    if (train && ok) {                               // each CTA hands its own parameters back
+        for (int p = 4 * g_lo + tid; p < 4 * (g_lo + g_n); p += TT) {
+            a.out[p] = sP[p];
+            a.out[GSTRIDE + p] = sM[p];
+            a.out[2 * GSTRIDE + p] = sV[p];
         }
     }
     tc::fence_before_sync();
     __syncthreads();
     if (warp == 0) tc::dealloc(tmem, TM_COLS);
+}
+
+// a training's parameters and moments to their places, unless a wait ran out
+// (one CTA's may have run out after another had finished)
+__global__ void k_mlp_commit(const float *out, const int *status, float *P, float *M, float *V, __nv_bfloat16 *W16) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= MLP_NP || *status) return;
+    P[i] = out[i];
+    M[i] = out[GSTRIDE + i];
+    V[i] = out[2 * GSTRIDE + i];
+    W16[i] = __float2bfloat16_rn(out[i]);
+}
+
+// the gradient call's sum over the CTAs' slots, in the order of the CTAs
+__global__ void k_mlp_sum_slots(const uint64_t *slots, int n, float *G) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= MLP_NP) return;
+    float s = 0.f;
+    for (int k = 0; k < n; ++k) s += __uint_as_float((uint32_t)slots[(size_t)k * GSTRIDE + i]);
+    G[i] = s;
 }
 
 __global__ void k_mlp_adam(float *P, float *M, float *V, float *G, __nv_bfloat16 *W16, float lr, float bc1, float bc2) {
@@ -571,8 +677,7 @@ using namespace sfq;
 static qed_status mlp_alloc(qed_ctx *ctx) {
     if (ctx->mlp_p) return QED_OK;
     if (cudaMalloc(&ctx->mlp_p, sizeof(float) * MLP_NP * 4) != cudaSuccess ||
-        cudaMalloc(&ctx->mlp_w16, sizeof(__nv_bfloat16) * (MLP_NP + 1)) != cudaSuccess ||
-        cudaMalloc(&ctx->mlp_loss, sizeof(float) * 2) != cudaSuccess)
+        cudaMalloc(&ctx->mlp_w16, sizeof(__nv_bfloat16) * (MLP_NP + 1)) != cudaSuccess)
         return QED_ERR_NOMEM;
     if (cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, TR_SMEM) != cudaSuccess)
         return QED_ERR_CUDA;
@@ -613,29 +718,50 @@ qed_status sfq_mlp_eval(qed_ctx *ctx, const float *feat, int64_t n, float *y) {
     return QED_OK;
 }
 
-// scratch of one training or gradient call: three gradient sums (the
-// gradient call uses the context's gradient buffer instead), the step
-// schedule, the barrier counter and the status word
+// Scratch of the training and gradient calls, kept in the context and grown
+// to the largest grid and step count asked for: the CTAs' slots, the new
+// weights, the CTAs' losses, the status word (all zeroed per call), the
+// parameters and moments at the end and the step schedule.
 struct TrainScratch {
-    void *mem = nullptr;
-    float *gbuf = nullptr, *sched = nullptr;
-    unsigned *bar = nullptr;
-    int *status = nullptr;
-    ~TrainScratch() {
-        if (mem) cudaFree(mem);
-    }
+    uint64_t *slots, *weights;
+    double *loss;
+    int *status;
+    float *out, *sched;
 };
 
-static qed_status train_scratch(TrainScratch &t, int64_t steps, cudaStream_t st) {
-    const size_t g = sizeof(float) * 3 * GSTRIDE, sc = sizeof(float) * 2 * (size_t)(steps > 0 ? steps : 1);
-    const size_t bytes = g + ((sc + 255) / 256) * 256 + 256;
-    if (cudaMalloc(&t.mem, bytes) != cudaSuccess) return QED_ERR_NOMEM;
-    t.gbuf = static_cast<float *>(t.mem);
-    t.sched = reinterpret_cast<float *>(static_cast<char *>(t.mem) + g);
-    t.bar = reinterpret_cast<unsigned *>(static_cast<char *>(t.mem) + g + ((sc + 255) / 256) * 256);
-    t.status = reinterpret_cast<int *>(t.bar + 1);
-    SFQ_CUDA(cudaMemsetAsync(t.gbuf, 0, g, st));
-    SFQ_CUDA(cudaMemsetAsync(t.bar, 0, 256, st));
+static qed_status train_scratch(qed_ctx *ctx, TrainScratch &t, int grid, int64_t steps) {
+    const size_t slots = sizeof(uint64_t) * GSTRIDE * (size_t)grid, weights = sizeof(uint64_t) * (GSTRIDE / 2 + 6);
+    const size_t loss = sizeof(double) * (size_t)grid, zeroed = slots + weights + loss + 16;
+    const size_t end = (zeroed + 255) / 256 * 256, bytes = end + sizeof(float) * (3 * GSTRIDE + 2 * (size_t)steps);
+    if (ctx->mlp_scratch_bytes < bytes) {
+        SFQ_CUDA(cudaStreamSynchronize(ctx->stream));
+        cudaFree(ctx->mlp_scratch);
+        ctx->mlp_scratch = nullptr;
+        ctx->mlp_scratch_bytes = 0;
+        if (cudaMalloc(&ctx->mlp_scratch, bytes) != cudaSuccess) return QED_ERR_NOMEM;
+        ctx->mlp_scratch_bytes = bytes;
+    }
+    char *m = static_cast<char *>(ctx->mlp_scratch);
+    t.slots = reinterpret_cast<uint64_t *>(m);
+    t.weights = reinterpret_cast<uint64_t *>(m + slots);
+    t.loss = reinterpret_cast<double *>(m + slots + weights);
+    t.status = reinterpret_cast<int *>(m + slots + weights + loss);
+    t.out = reinterpret_cast<float *>(m + end);
+    t.sched = t.out + 3 * GSTRIDE;
+    SFQ_CUDA(cudaMemsetAsync(m, 0, zeroed, ctx->stream));
+    return QED_OK;
+}
+
+// the CTAs' losses added in their order, and the status word
+static qed_status train_result(const TrainScratch &t, int grid, cudaStream_t st, double *loss) {
+    std::vector<double> h((size_t)grid + 1);         // the status word lies behind the losses
+    SFQ_CUDA(cudaMemcpyAsync(h.data(), t.loss, sizeof(double) * (size_t)grid + sizeof(int), cudaMemcpyDeviceToHost, st));
+    SFQ_CUDA(cudaStreamSynchronize(st));
+    int status;
+    memcpy(&status, &h[(size_t)grid], sizeof status);
+    if (status) return QED_ERR_TIMEOUT;
+    *loss = 0.0;
+    for (int k = 0; k < grid; ++k) *loss += h[(size_t)k];
     return QED_OK;
 }
 
@@ -660,23 +786,20 @@ qed_status sfq_mlp_grad(qed_ctx *ctx, const float *feat, const float *target, in
     cudaStream_t st = ctx->stream;
     float *P = ctx->mlp_p;
     TrainScratch t;
-    qed_status e = train_scratch(t, 0, st);
-    if (e != QED_OK) return e;
-    SFQ_CUDA(cudaMemsetAsync(ctx->mlp_loss, 0, sizeof(float), st));
     int grid = 0;
-    if ((e = train_grid((n + TS - 1) / TS, &grid)) != QED_OK) return e;
-    TrainArgs a{P, P + MLP_NP, P + 2 * MLP_NP, t.gbuf, ctx->mlp_w16, ctx->mlp_loss, ctx->icdf_em32, feat, target,
-                t.sched, 0ull, (long long)n, 0ll, 0ll, 1.0f / (float)n, t.bar, BAR_POLLS, t.status};
+    qed_status e = train_grid((n + TS - 1) / TS, &grid);
+    if (e == QED_OK) e = train_scratch(ctx, t, grid, 0);
+    if (e != QED_OK) return e;
+    TrainArgs a{P, P + MLP_NP, P + 2 * MLP_NP, t.out, t.slots, t.weights, t.loss, ctx->icdf_em32, feat, target,
+                t.sched, 0ull, (long long)n, 0ll, 0ll, 1.0f / (float)n, WORD_POLLS, t.status};
     k_mlp_train<<<grid, TT, TR_SMEM, st>>>(a);
+    k_mlp_sum_slots<<<(MLP_NP + 255) / 256, 256, 0, st>>>(t.slots, grid, P + 3 * MLP_NP);
     SFQ_CUDA(cudaGetLastError());
-    SFQ_LAUNCHED(ctx, 1);
-    float l = 0.f;
-    int status = 0;
-    SFQ_CUDA(cudaMemcpyAsync(grad_host, t.gbuf, sizeof(float) * MLP_NP, cudaMemcpyDeviceToHost, st));
-    SFQ_CUDA(cudaMemcpyAsync(&l, ctx->mlp_loss, sizeof(float), cudaMemcpyDeviceToHost, st));
-    SFQ_CUDA(cudaMemcpyAsync(&status, t.status, sizeof(int), cudaMemcpyDeviceToHost, st));
-    SFQ_CUDA(cudaStreamSynchronize(st));
-    if (status) return QED_ERR_TIMEOUT;
+    SFQ_LAUNCHED(ctx, 2);
+    SFQ_CUDA(cudaMemcpyAsync(grad_host, P + 3 * MLP_NP, sizeof(float) * MLP_NP, cudaMemcpyDeviceToHost, st));
+    SFQ_CUDA(cudaMemsetAsync(P + 3 * MLP_NP, 0, sizeof(float) * MLP_NP, st));    // zero between calls, as k_mlp_adam leaves it
+    double l = 0.0;
+    if ((e = train_result(t, grid, st, &l)) != QED_OK) return e;
     if (loss) *loss = l / (double)n;
     return QED_OK;
 }
@@ -703,26 +826,23 @@ qed_status sfq_mlp_train(qed_ctx *ctx, int64_t n_samples, int batch, double lr, 
         sched[2 * s + 1] = (float)(1.0 / bc2);
     }
     TrainScratch t;
-    if ((e = train_scratch(t, steps, st)) != QED_OK) return e;
-    SFQ_CUDA(cudaMemcpyAsync(t.sched, sched.data(), sizeof(float) * sched.size(), cudaMemcpyHostToDevice, st));
-    SFQ_CUDA(cudaMemsetAsync(ctx->mlp_loss, 0, sizeof(float), st));
     int grid = 0;
     if ((e = train_grid(batch / TS, &grid)) != QED_OK) return e;
+    if ((e = train_scratch(ctx, t, grid, steps)) != QED_OK) return e;
+    SFQ_CUDA(cudaMemcpyAsync(t.sched, sched.data(), sizeof(float) * sched.size(), cudaMemcpyHostToDevice, st));
     const int64_t tail = steps < 16 ? steps : 16;     // the loss is averaged over the last 16 steps
-    TrainArgs a{P, M, V, t.gbuf, ctx->mlp_w16, ctx->mlp_loss, ctx->icdf_em32, nullptr, nullptr, t.sched, seed,
-                (long long)batch, (long long)steps, (long long)(steps - tail), 1.0f / (float)batch, t.bar,
-                ctx->cfg.wait_polls > 0 ? (uint32_t)ctx->cfg.wait_polls : BAR_POLLS, t.status};
+    TrainArgs a{P, M, V, t.out, t.slots, t.weights, t.loss, ctx->icdf_em32, nullptr, nullptr, t.sched, seed,
+                (long long)batch, (long long)steps, (long long)(steps - tail), 1.0f / (float)batch,
+                ctx->cfg.wait_polls > 0 ? (uint32_t)ctx->cfg.wait_polls : WORD_POLLS, t.status};
     void *args[] = {&a};
     SFQ_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void *>(k_mlp_train), dim3(grid), dim3(TT), args,
                                          (size_t)TR_SMEM, st));
-    SFQ_LAUNCHED(ctx, 2);
-    float l = 0.f;
-    int status = 0;
-    SFQ_CUDA(cudaMemcpyAsync(&l, ctx->mlp_loss, sizeof(float), cudaMemcpyDeviceToHost, st));
-    SFQ_CUDA(cudaMemcpyAsync(&status, t.status, sizeof(int), cudaMemcpyDeviceToHost, st));
-    SFQ_CUDA(cudaStreamSynchronize(st));
-    if (status) return QED_ERR_TIMEOUT;
-    if (final_loss) *final_loss = (double)l / (double)(tail * batch);
+    k_mlp_commit<<<(MLP_NP + 255) / 256, 256, 0, st>>>(t.out, t.status, P, M, V, ctx->mlp_w16);
+    SFQ_CUDA(cudaGetLastError());
+    SFQ_LAUNCHED(ctx, 3);
+    double l = 0.0;
+    if ((e = train_result(t, grid, st, &l)) != QED_OK) return e;
+    if (final_loss) *final_loss = l / (double)(tail * batch);
     ctx->mlp_ready = 1;
     return QED_OK;
 }
