@@ -1046,6 +1046,10 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_photon_pass(P
         __syncwarp();
         flush_stats(ctl, ps);
     }
+    // No photon pushed, no pair born: the step-begin kernel's empty range stands.
+    // In particular a step opened after an overflow or a timeout has empty
+    // ranges while the counts are not zero, and must stay empty.
+    if (n == 0) return;
     if (last_block(ctl) && threadIdx.x < 2) ctl->born[threadIdx.x] = count_now(ctl, threadIdx.x);
 }
 
@@ -1224,6 +1228,7 @@ __global__ void __launch_bounds__(256, 2) k_photon_pass2(const __grid_constant__
         __syncwarp();
         flush_stats(ctl, ps);
     }
+    if (n == 0) return;                          // as in k_photon_pass
     if (last_block(ctl) && threadIdx.x < 2) ctl->born[threadIdx.x] = count_now(ctl, threadIdx.x);
 }
 #endif
