@@ -1111,7 +1111,10 @@ qed_status level_eval_impl(qed_ctx *ctx, qed_species *sp, double w, double *A, i
 
 using namespace sfq;
 
+// The captured step holds addresses inside these buffers: it goes when one of
+// them does, and the next batch of steps captures anew.
 qed_status sfq_ensure_work(qed_ctx *ctx, int64_t n_blocks, int64_t n_slots) {
+    if (ctx->blk_cap < n_blocks || ctx->slots_cap < n_slots) sfq_step_graph_free(ctx);
     if (ctx->blk_cap < n_blocks) {
         if (ctx->blk) SFQ_CUDA(cudaFreeAsync(ctx->blk, ctx->stream));
         ctx->blk = nullptr;
