@@ -99,7 +99,8 @@ typedef struct {
     int wait_polls;           /* polls of each wait of one block for another inside
                                  qed_train_surrogate before the launch gives up
                                  (QED_ERR_TIMEOUT); 0 = 2^24 */
-    int reserved[1];
+    int level_polls;          /* polls of each wait of one block for another inside the
+                                 leveling before it gives up (QED_ERR_TIMEOUT); 0 = 2^24 */
 } qed_config;
 
 /* Event methods of qed_push_and_generate.
@@ -225,7 +226,9 @@ qed_status qed_push_wait(qed_ctx *ctx, qed_particles *p, qed_stats *out);
  * apply global leveling at step index `step` (Sec. 4.2 merge step, Sec. 5.1).
  * Leveling: threshold w* with sum_i min(1, w_i/w*) = cap; particle i kept with
  * probability min(1, w_i/w*) (Philox counter word 3 = 0xFFFFFFFF); kept
- * particles below w* get weight w*.  Counts in *p are updated. */
+ * particles below w* get weight w*.  Counts in *p are updated.
+ * QED_ERR_TIMEOUT if a bounded wait inside the leveling ran out (the particles
+ * are then as they were). */
 qed_status qed_compact(qed_ctx *ctx, qed_particles *p, int64_t step);
 
 /* Push n_ens independent ensembles (ens[k] in the field fields[k]) through

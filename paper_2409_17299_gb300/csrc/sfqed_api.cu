@@ -144,6 +144,7 @@ extern "C" qed_status qed_compact(qed_ctx *ctx, qed_particles *p, int64_t step) 
     if (e != QED_OK) return e;
     SFQ_CUDA(cudaMemcpyAsync(ctx->ctl_host, ctx->ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, ctx->stream));
     SFQ_CUDA(cudaStreamSynchronize(ctx->stream));
+    if (ctx->ctl_host->timeout) return QED_ERR_TIMEOUT;         // the leveling gave up: nothing was changed
     if (ctx->ctl_host->bad_index) return QED_ERR_STATE;
     for (int s = 0; s < 3; ++s) p->s[s].count = (int64_t)ctx->ctl_host->count[s];
     ctx->acc.thinned += (int64_t)ctx->ctl_host->thinned;

@@ -479,6 +479,9 @@ struct LevWeights {
 // pass every block sums its share of each species' weights, the last block
 // to arrive reduces the partials and advances the iterations, and the others
 // wait for it (bounded; a wait that runs out marks the step as timed out).
+// Arrivals are counted in the control block, which every batch of steps and
+// every merge call opens anew: a wait that ran out leaves arrivals behind, and
+// no later leveling may count them.
 //
 // A pass over 1e7 weights takes 6 us from DRAM and less from L2, but as two
 // launches of a graph's while loop per pass and species it took 19 to 25 us,
@@ -489,10 +492,11 @@ struct LevWeights {
 // merged compaction launches: 40 steps of that cascade 88.2 -> 72.4 ms, 20
 // steps on the grid (1e6 per species) 20.8 -> 13.3 ms, 20 steps at the start
 // of a cascade 2.86 -> 2.00 ms, 40 steps at 5e7 photons 87.0 -> 83.9 ms.
-constexpr unsigned LEV_POLLS = 1u << 24;
+constexpr unsigned LEV_POLLS = 1u << 24;      // unless cfg.level_polls gives another limit
 
 template <class T>
-__global__ void __launch_bounds__(LEV_T, 4) k_level(LevWeights lwt, DevCtl *ctl, LevelWork *lw, long long cap) {
+__global__ void __launch_bounds__(LEV_T, 4) k_level(LevWeights lwt, DevCtl *ctl, LevelWork *lw, long long cap,
+                                                    unsigned max_polls) {
     __shared__ int s_last, s_out;
     __shared__ double s_w[3];
     __shared__ float s_wup[3];
@@ -527,7 +531,7 @@ __global__ void __launch_bounds__(LEV_T, 4) k_level(LevWeights lwt, DevCtl *ctl,
             if (!s_done[s]) lev_block_sums<T>(lwt.w[s], n[s], s_w[s], s_wup[s], lw, s);
         if (t == 0) {
             __threadfence();
-            s_last = atomicAdd(&lw->arrive, 1u) == gridDim.x - 1;
+            s_last = atomicAdd(&ctl->arrive, 1ull) == gridDim.x - 1;
             __threadfence();
         }
         __syncthreads();
@@ -552,7 +556,7 @@ __global__ void __launch_bounds__(LEV_T, 4) k_level(LevWeights lwt, DevCtl *ctl,
             }
             __syncthreads();
             if (t == 0) {
-                lw->arrive = 0;
+                ctl->arrive = 0;
                 __threadfence();
                 atomicExch(&lw->round, round0 + pass + 1);
             }
@@ -561,7 +565,7 @@ __global__ void __launch_bounds__(LEV_T, 4) k_level(LevWeights lwt, DevCtl *ctl,
             unsigned polls = 0;
             s_out = 0;
             while (!s_last && *reinterpret_cast<volatile unsigned long long *>(&lw->round) != round0 + pass + 1) {
-                if (++polls > LEV_POLLS) {
+                if (++polls > max_polls) {
                     atomicExch(&ctl->timeout, 1ull);
                     s_out = 1;
                     break;
@@ -1044,7 +1048,8 @@ template <class T> static qed_status level_launch(qed_ctx *ctx, const qed_partic
     int blocks = ctx->sm_count * (per_sm < 4 ? (per_sm > 0 ? per_sm : 1) : 4);
     blocks = blocks > LEVEL_MAX_BLOCKS ? LEVEL_MAX_BLOCKS : blocks;
     long long cap = (long long)ctx->cfg.thin_cap;
-    void *args[] = {&w, &ctx->ctl, &ctx->lev, &cap};
+    unsigned polls = ctx->cfg.level_polls > 0 ? (unsigned)ctx->cfg.level_polls : LEV_POLLS;
+    void *args[] = {&w, &ctx->ctl, &ctx->lev, &cap, &polls};
     SFQ_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void *>(k_level<T>), dim3((unsigned)blocks), dim3(LEV_T), args,
                                          0, ctx->stream));
     SFQ_LAUNCHED(ctx, 1);

@@ -64,7 +64,7 @@ struct DevCtl {
     unsigned long long moved;           // compaction: entries moved into holes
     unsigned long long pass_limit;      // generations of newborns a step may run (then timeout)
     unsigned long long born[2];         // leptons after the photon pass (its pairs lie behind the step-start range)
-    unsigned long long arrive;          // blocks of the running pass kernel that have finished
+    unsigned long long arrive;          // blocks of the running kernel that have arrived (passes, leveling, fill)
     unsigned long long spilled;         // newborn leptons left behind by the lepton pass
 };
 static_assert(sizeof(DevCtl) == 384, "control block layout");
@@ -95,7 +95,7 @@ struct LevelWork {
     unsigned long long on[3];                   // the current merge step leveled the species
     double prev[3];                             // last threshold found per species
     double ratio[3];                            // its growth over the one before (the next start: their product)
-    unsigned arrive;                            // blocks of the current pass that finished
+    unsigned arrive;                            // blocks of an evaluation for a shard that finished
     unsigned long long round;                   // passes finished
     double sumA;                                // sums of an evaluation for a shard
     unsigned long long sumC, sumN, sumM;

@@ -619,8 +619,6 @@ static qed_status wait_batch(qed_ctx *ctx, qed_particles *p, qed_stats *out) {
     qed_status rc = QED_OK;
     if (c.overflow) rc = QED_ERR_CAPACITY;
     if (c.timeout) rc = QED_ERR_TIMEOUT;
-    // a leveling wait that ran out may have left arrivals uncounted
-    if (c.timeout && ctx->lev) SFQ_CUDA(cudaMemsetAsync(&ctx->lev->arrive, 0, sizeof ctx->lev->arrive, ctx->stream));
     if (c.bad_index) rc = QED_ERR_STATE;
     qed_stats st{};
     st.particle_steps = (int64_t)c.particle_steps;
