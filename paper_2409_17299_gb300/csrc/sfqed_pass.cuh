@@ -850,6 +850,8 @@ __global__ void __launch_bounds__(LB<T>, (sizeof(T) == 4 && !MLP ? 3 : 2))
 // those without an event are pushed to the step end, the others go through
 // the stack as in the pass above and come back through the species arrays.
 // The arithmetic per particle and step is that of the pass, as are the draws.
+// Photons past the capacity are counted, not written, and every block takes
+// all steps: the demand and the statistics do not depend on their timing.
 //
 // A launch per step is bound by its latency where the ensemble is small: the
 // step-begin kernel, the tables' staging and the block's last, partly filled
@@ -863,8 +865,7 @@ __global__ void __launch_bounds__(LB<T>, 2) k_lepton_steps(const __grid_constant
     __shared__ LeptonStack<T> q;
     __shared__ StepTime s_tm;
     __shared__ Phase<T> s_ph;
-    __shared__ int s_stop;
-    const unsigned n0 = (unsigned)min(ctl->count[0], ctl->capacity[0]), n1 = (unsigned)min(ctl->count[1], ctl->capacity[1]);
+    const unsigned n0 = (unsigned)ctl->end[0], n1 = (unsigned)ctl->end[1];
     const unsigned n = n0 + n1;
     if (blockIdx.x * NT >= n) return;
     for (int i = threadIdx.x; i < RateWords<T>::N; i += NT) s_coef[i] = reinterpret_cast<const T *>(a.coef)[i];
@@ -903,10 +904,8 @@ __global__ void __launch_bounds__(LB<T>, 2) k_lepton_steps(const __grid_constant
                 s_tm.t_n_red_f = (float)fmod(t_n, 2.0 * 3.14159265358979323846);
                 s_tm.step = (unsigned)(step0 + it);
                 s_ph = time_phase<T, StepTime>(s_tm, 0.0);
-                s_stop = __ldcg(&ctl->overflow) != 0;
             }
             __syncthreads();
-            if (s_stop) break;                   // out of capacity: later steps do nothing
             const LeptonCtx<T> c{a, ctl, s_coef, a.coef32, reinterpret_cast<const T *>(a.icdf_em), ctl->capacity[2], 0u,
                                  (T)(ALPHA * RS), s_tm, s_ph};
             bool away = false;

@@ -58,11 +58,14 @@ __global__ void k_step_begin(DevCtl *ctl, double dt) {
     ctl->spilled = 0;
 }
 
-// the control block after nsteps steps taken by one launch
+// Opens nsteps steps taken by one launch: the leptons' ranges as in
+// k_step_begin, the control block as it is after the last step.
 __global__ void k_advance_step(DevCtl *ctl, double dt, unsigned long long nsteps) {
     ctl->step_next += nsteps;
     ctl->sv_step = (unsigned)(ctl->step_next - 1);
     ctl->sv_t_n = (double)(ctl->step_next - 1) * dt;
+    const bool stop = ctl_stopped(ctl);
+    for (int s = 0; s < 2; ++s) ctl->end[s] = stop ? 0 : min(ctl->count[s], ctl->capacity[s]);
 }
 
 __global__ void k_set_step(DevCtl *ctl, unsigned long long step) { ctl->step_next = step; }
@@ -580,8 +583,12 @@ static qed_status enqueue_steps(qed_ctx *ctx, const qed_field_desc *field, doubl
     a.fly_newborns = cascade && ctx->cfg.event_method == QED_METHOD_SUBSTEP ? 1 : 0;
 
     ctx->async_deferred = 1;
-    if (!cascade && ctx->cfg.thin_cap == 0 && ctx->cfg.event_method == QED_METHOD_SUBSTEP && !a.mlp_w16 && nsteps > 1) {
-        // an emission run of several steps: one launch for all of them
+    if (!cascade && ctx->cfg.thin_cap == 0 && ctx->cfg.event_method == QED_METHOD_SUBSTEP && !a.mlp_w16 && nsteps > 1 &&
+        ctx->cfg.restore_on_overflow) {
+        // An emission run of several steps: one launch for all of them.  Its
+        // blocks cannot stop at the step in which the photons run out of
+        // room, so it is taken where the state goes back to the batch's start
+        // then; the demand it counts is that of all its steps.
         a.pass = 0;
         k_advance_step<<<1, 1, 0, ctx->stream>>>(ctx->ctl, dt, (unsigned long long)nsteps);
         SFQ_LAUNCHED(ctx, 1);
