@@ -379,6 +379,8 @@ __device__ __forceinline__ bool surely_calm(const LeptonCtx<double> &c, const do
     if (a.field_zero) chi = sqrtf(e2 + ax * ax + ay * ay + az * az + bx * bx + by * by + bz * bz);     // E.(p x B) = 0
     else chi = sqrtf(e2 + ax * ax + ay * ay + az * az) + sqrtf(bx * bx + by * by + bz * bz);
     chi = (chi + sum * 0x1p-21f) * (float)(1.0 / RS) * 1.0001f;
+    // beyond FP32's range (an infinity, or a NaN from the difference of two) nothing is decided
+    if (!(chi < t_inf<float>() && gam < t_inf<float>())) return false;
     const float lam = (float)(ALPHA * RS) / gam * rate_em<float>(c.coef32, chi);
     const uint4 r = event_draw(a.keys, id, c.tm.step, 0u);
     float u, v;
@@ -406,6 +408,7 @@ __device__ __forceinline__ double own(double v) { asm volatile("" : "+d"(v)); re
 // chi_ub: an upper bound of chi; tab32: the FP32 rate pieces.
 __device__ __forceinline__ bool surely_flies(const PassArgs &a, const float *tab32, float chi_ub, float inv_k0, float h,
                                              unsigned long long id, unsigned step) {
+    if (!(chi_ub < t_inf<float>())) return false;      // beyond FP32's range, or a NaN: not decided
     const float lam = (float)(ALPHA * RS) * inv_k0 * rate_pair<float>(tab32, chi_ub * 1.0001f);
     const uint4 r = event_draw(a.keys, id, step, 0u);
     float u, v;
