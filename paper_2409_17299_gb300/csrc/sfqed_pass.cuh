@@ -1156,7 +1156,9 @@ __global__ void __launch_bounds__(256, 2) k_photon_pass2(const __grid_constant__
                     const float xq[3] = {x[0][q], x[1][q], x[2][q]}, kq[3] = {k[0][q], k[1][q], k[2][q]};
                     float E[3], B[3];
                     field_at<float>(a, xq, ph0, E, B);
-                    chi[q] = photon_chi<float, true>(k0[q], kq, E, B, ps.n64, a.field_zero);
+                    unsigned n64 = 0;                 // counted for photons that fly, not for dead places
+                    chi[q] = photon_chi<float, true>(k0[q], kq, E, B, n64, a.field_zero);
+                    if (fly[q]) ps.n64 += n64;
                 }
             }
             // rates (rate_pair<float>, its last piece's continuation apart)
