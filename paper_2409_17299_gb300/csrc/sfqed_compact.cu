@@ -992,9 +992,12 @@ static int64_t merge_blk_words(const int64_t bound[3]) {
     return n;
 }
 
+// words of species s: the dead list, then the movers
+static int64_t dead_words(int64_t bound) { return (bound + 3) / 4 + 1; }
+static int64_t mover_words(int64_t bound) { return bound / 2 + 1; }
 static int64_t merge_slot_words(const int64_t bound[3]) {
     int64_t n = 0;
-    for (int s = 0; s < 3; ++s) n += (bound[s] + 3) / 4 + bound[s] / 2 + 2;
+    for (int s = 0; s < 3; ++s) n += dead_words(bound[s]) + mover_words(bound[s]);
     return n;
 }
 
@@ -1011,9 +1014,9 @@ static qed_status merge_args(qed_ctx *ctx, const qed_particles *p, const int64_t
         m.blk[s] = blk;
         blk += m.nb[s] + 2;
         m.dl[s] = reinterpret_cast<unsigned short *>(slots);
-        slots += (bound[s] + 3) / 4 + 1;
+        slots += dead_words(bound[s]);
         m.movers[s] = slots;
-        slots += bound[s] / 2 + 1;
+        slots += mover_words(bound[s]);
     }
     m.ctl = ctx->ctl;
     m.lw = ctx->lev;
@@ -1141,6 +1144,12 @@ qed_status sfq_ensure_work(qed_ctx *ctx, int64_t n_blocks, int64_t n_slots) {
 
 qed_status sfq_ensure_merge(qed_ctx *ctx, const int64_t bound[3]) {
     return sfq_ensure_work(ctx, merge_blk_words(bound), merge_slot_words(bound));
+}
+
+unsigned *sfq_entry_words(const qed_ctx *ctx, const int64_t bound[3], int s) {
+    int64_t at = dead_words(bound[s]);                  // the movers of species s: half a 64-bit word per entry
+    for (int k = 0; k < s; ++k) at += dead_words(bound[k]) + mover_words(bound[k]);
+    return reinterpret_cast<unsigned *>(ctx->slots + at);
 }
 
 qed_status sfq_merge(qed_ctx *ctx, const qed_particles *p, const int64_t bound[3], int level_mask, int always,

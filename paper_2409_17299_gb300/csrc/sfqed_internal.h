@@ -158,6 +158,7 @@ struct PassArgs {
     unsigned long long seed;
     PhiloxKeys keys;        // round keys of seed (event draws)
     PhiloxKeys child_keys;  // round keys of the children's ids
+    unsigned *gen[2];       // generation of newborn leptons left for a further launch (by index, work buffer)
     int pass;               // 0: particles present at the step start (tau = 0)
     int soft_filter;
     int fly_newborns;       // newborns are pushed to the end of their birth step (cascades)
@@ -314,6 +315,8 @@ struct GraphBuild {
 // may_defer: the moves may be left for a later step (dead entries stay in
 // place while they are few; see k_scan_tiles).
 qed_status sfq_ensure_merge(qed_ctx *ctx, const int64_t bound[3]);
+// a word per entry of species s inside the merge's work buffers, free between merges
+unsigned *sfq_entry_words(const qed_ctx *ctx, const int64_t bound[3], int s);
 qed_status sfq_merge(qed_ctx *ctx, const qed_particles *p, const int64_t bound[3], int level_mask, int always,
                      int64_t step, bool step_from_ctl, bool may_defer);
 qed_status sfq_level_eval(qed_ctx *ctx, qed_species *sp, double w, double *A, int64_t *C, int64_t *N, double *M);

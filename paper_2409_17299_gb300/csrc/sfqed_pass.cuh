@@ -538,9 +538,11 @@ __device__ __forceinline__ void fly_newborn(const LeptonCtx<T> &c, LeptonStack<T
                     q.nb_idx[at] = i | ((unsigned)s << 31);
                     q.nb_gen[at] = gen + 1u;
                 } else {
-                    // left at its birth clock for a further launch; the sign
-                    // bit marks it (those taken up here stay unmarked)
+                    // left at its birth clock for a further launch, with its
+                    // generation; the sign bit marks it (those taken up here
+                    // stay unmarked)
                     a.sp[s].tau[i] = -tau;
+                    a.gen[s][i] = gen + 1u;
                     atomicAdd(&c.ctl->spilled, 1ull);
                 }
             });
@@ -683,7 +685,6 @@ __global__ void __launch_bounds__(LB<T>, (sizeof(T) == 4 && !MLP ? 3 : 2))
         if (threadIdx.x == 0) s_tm = load_step_time(a);
         __syncthreads();
         const unsigned gen_limit = (unsigned)ctl->pass_limit;
-        const unsigned gen0 = FRESH ? 1u : (unsigned)ctl->step_passes + 1u;   // generation of the newborns waiting
         const LeptonCtx<T> c{a, ctl, s_coef, a.coef32, reinterpret_cast<const T *>(a.icdf_em), ctl->capacity[2], gen_limit,
                              (T)(ALPHA * RS), s_tm, time_phase<T, StepTime>(s_tm, 0.0)};
         // FP32 step-start pass: each thread stages its particle of the block's
@@ -780,7 +781,7 @@ __global__ void __launch_bounds__(LB<T>, (sizeof(T) == 4 && !MLP ? 3 : 2))
                 // tile of those waiting in the species arrays
                 const bool own = pos.nb > 0;
                 const unsigned t = threadIdx.x;
-                unsigned idx = 0, gen = gen0;
+                unsigned idx = 0, gen = 1u;               // pairs of the photons present at the step start
                 bool have = false;
                 if (own) {
                     have = t < (unsigned)pos.nb;
@@ -801,6 +802,7 @@ __global__ void __launch_bounds__(LB<T>, (sizeof(T) == 4 && !MLP ? 3 : 2))
                         if (!own) {
                             have = __double_as_longlong(tau) < 0;
                             tau = -tau;
+                            if (have) gen = a.gen[idx >> 31][i];
                         }
                     }
                     if (have && gen > gen_limit) {

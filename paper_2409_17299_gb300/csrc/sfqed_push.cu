@@ -534,6 +534,8 @@ static qed_status enqueue_steps(qed_ctx *ctx, const qed_field_desc *field, doubl
                              reinterpret_cast<unsigned long long *>(S.id), S.nevents, s < 2 ? ctx->tau[s] : nullptr,
                              ctx->od[s]};
     }
+    const int64_t bound[3] = {p->s[0].capacity, p->s[1].capacity, p->s[2].capacity};
+    for (int s = 0; s < 2; ++s) a.gen[s] = sfq_entry_words(ctx, bound, s);
     a.ctl = ctx->ctl;
     const bool f32 = sizeof(T) == 4;
     a.coef = f32 ? (const void *)ctx->coef32 : (const void *)ctx->coef64;
