@@ -695,16 +695,15 @@ __global__ void __launch_bounds__(LT, 4) k_tile_dead(const __grid_constant__ Mer
         unsigned mask[LROUNDS];
         unsigned cnt = 0;
         // weights and (leveling) ids of G entries issued together, and those of
-        // the next G before this group's draws and stores.  Read-only loads:
-        // an entry's weight is read once, by the thread that may then store it,
-        // and the compiler need not keep the loads behind the stores.
+        // the next G before this group's draws and stores.  The weights are
+        // written by this kernel, so plain loads; the ids are not.
         T v[G], vn[G];
         unsigned long long idv[G], idn[G];
         auto load = [&](int c0, T (&vv)[G], unsigned long long (&ii)[G]) {
 #pragma unroll
             for (int r = 0; r < G; ++r) {
                 const unsigned long long i = wbase + (c0 + r) * 32 + lane;
-                vv[r] = i < n ? __ldg(reinterpret_cast<const T *>(S.w) + i) : (T)0;
+                vv[r] = i < n ? ld<T>(S.w, i) : (T)0;
                 ii[r] = (LEVEL && thin && i < n) ? __ldg(S.id + i) : 0ull;
             }
         };
