@@ -1059,14 +1059,21 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 ? 4 : 1)) k_photon_pass(P
 
 
 #if !SFQ_GRID
-// The FP32 photon pass in a field that does not depend on the position
-// (uniform, rotating E), two consecutive photons per thread.  A photon is a
+// The FP32 photon pass in a field that does not depend on the position and
+// where chi is a sum of squares (rotating E, uniform E or B), two consecutive
+// photons per thread.  A photon is a
 // chain of some 250 dependent instructions (a scheduler issued in 65% of the
 // cycles with one photon per thread and 32 warps per SM); the chains of two
 // photons interleave, and copies, shared-memory reads and stores move two
 // photons at a time.  Both photons' arithmetic is written out with explicit
 // rounding where the compiler could fuse either way.  5e7 photons, rotating E:
-// 40 steps of its cascade 82.2 -> 77.1 ms; two blocks per SM (106 registers) as fast as three (spills).
+// 40 steps of its cascade 82.2 -> 77.1 ms; two blocks per SM (105 registers) as fast as three (spills).
+// The pass, one photon per thread -> two, in us (rotating E, uniform E, uniform B):
+// 219 -> 173, 219 -> 183, 221 -> 184 at 2e7 photons, 22.1 -> 18.0, 22.7 -> 18.0,
+// 22.5 -> 19.8 at 1e6, 8.8 -> 7.8, 7.9 -> 7.6, 8.4 -> 7.6 at 2e4.  With E and B
+// both (field_zero 0) chi's FP64 fallback branches photon by photon and nothing
+// interleaves: 1734 -> 1723 at 2e7, 98 -> 102 at 1e6, 11.7 -> 15.8 at 2e4;
+// one photon per thread is the rule there.
 // In the standing wave the two sine and cosine evaluations do not interleave
 // (their argument reduction branches): 40 steps took 72.1 ms against 71.6 with
 // one photon per thread, which stays the rule there and on the grid.
@@ -1158,9 +1165,8 @@ __global__ void __launch_bounds__(256, 2) k_photon_pass2(const __grid_constant__
                     const float xq[3] = {x[0][q], x[1][q], x[2][q]}, kq[3] = {k[0][q], k[1][q], k[2][q]};
                     float E[3], B[3];
                     field_at<float>(a, xq, ph0, E, B);
-                    unsigned n64 = 0;                 // counted for photons that fly, not for dead places
-                    chi[q] = photon_chi<float, true>(k0[q], kq, E, B, n64, a.field_zero);
-                    if (fly[q]) ps.n64 += n64;
+                    unsigned n64 = 0;                 // a sum of squares: no evaluation in FP64
+                    chi[q] = photon_chi<float, true>(k0[q], kq, E, B, n64, a.field_zero == 1 ? 1 : 2);
                 }
             }
             // rates (rate_pair<float>, its last piece's continuation apart)
@@ -1534,7 +1540,7 @@ qed_status launch_pass(qed_ctx *ctx, PassArgs &a, bool photons, cudaGraphConditi
     qed_status e = QED_OK;
     if (a.pass == 0 && photons) {
 #if !SFQ_GRID
-        if (sizeof(T) == 4 && a.field_kind != QED_FIELD_STANDING_CP) {
+        if (sizeof(T) == 4 && a.field_kind != QED_FIELD_STANDING_CP && a.field_zero != 0) {
             const int bp = resident_blocks(ctx, k_photon_pass2, 256);
             e = timed_launch(ctx, 1, [&] { k_photon_pass2<<<bp, 256, 0, ctx->stream>>>(a); });
         } else
