@@ -213,8 +213,8 @@ qed_status qed_push_and_generate(qed_ctx *ctx, qed_particles *p, const qed_field
  * out->needed_capacity and, with restore_on_overflow, *p back at its state
  * when the batch opened (grow and replay the whole batch).  With
  * restore_on_overflow a call of several emission steps (photons recorded, no
- * leveling) runs all its steps as one: its demand and its statistics are then
- * those of all its steps.
+ * leveling) may run all its steps as one: its demand and its statistics are
+ * then those of all its steps.
  * While a batch is open, qed_compact, qed_level_eval, qed_level_apply,
  * qed_batch_push, qed_autotune_batch, qed_eval_chi and qed_set_optical_depth
  * return QED_ERR_STATE.

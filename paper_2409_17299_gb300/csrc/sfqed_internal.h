@@ -330,13 +330,15 @@ namespace pass_analytic {
 template <class T>
 qed_status launch_pass(qed_ctx *ctx, PassArgs &a, bool photons, cudaGraphConditionalHandle h, int loop);
 template <class T> qed_status launch_od(qed_ctx *ctx, PassArgs &a, bool photons);
-template <class T> qed_status launch_steps(qed_ctx *ctx, PassArgs &a, int64_t step0, int nsteps);
+template <class T> int steps_blocks(const qed_ctx *ctx, int64_t n, int nsteps);
+template <class T> qed_status launch_steps(qed_ctx *ctx, PassArgs &a, int64_t step0, int nsteps, int blocks);
 }
 namespace pass_grid {
 template <class T>
 qed_status launch_pass(qed_ctx *ctx, PassArgs &a, bool photons, cudaGraphConditionalHandle h, int loop);
 template <class T> qed_status launch_od(qed_ctx *ctx, PassArgs &a, bool photons);
-template <class T> qed_status launch_steps(qed_ctx *ctx, PassArgs &a, int64_t step0, int nsteps);
+template <class T> int steps_blocks(const qed_ctx *ctx, int64_t n, int nsteps);
+template <class T> qed_status launch_steps(qed_ctx *ctx, PassArgs &a, int64_t step0, int nsteps, int blocks);
 }
 }  // namespace sfq
 qed_status sfq_ensure_work(qed_ctx *ctx, int64_t n_blocks, int64_t n_slots);

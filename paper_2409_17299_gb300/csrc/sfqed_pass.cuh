@@ -1561,11 +1561,31 @@ qed_status launch_pass(qed_ctx *ctx, PassArgs &a, bool photons, cudaGraphConditi
     return QED_OK;
 }
 
+// Blocks of the one-launch emission run for n leptons; 0: the steps are taken
+// one by one.  A block keeps its 256 (FP64 128) leptons through all steps, so
+// with more leptons than resident threads it runs all steps for one tile after
+// another, drains its stack in every step of every tile, and has none of the
+// pass's staged loads; the pass's launches then cost less than that.  One
+// launch against a launch per step (graph), gain at 2 / 10 / 40 steps, uniform
+// B (a wave is 77824 leptons in both precisions):
+//   FP32  1 wave 1.20 / 1.84 / 2.71   2 waves 0.99 / 1.43 / 1.72   3 waves
+//         0.99 / 1.18 / 1.34   4 waves 1.00 / 1.07 / 1.14   6 waves 0.88 /
+//         0.87 / 0.89   13 waves 0.68 / 0.61 / 0.61 (2.4 times as slow at 4e6 leptons)
+//   FP64  1 wave 1.13 / 1.52 / 1.70   2 waves 0.86 / 1.00 / 1.07   3 waves
+//         0.72 / 0.82 / 0.85   13 waves 0.56 / 0.57 / 0.57
+// and much the same in the other analytic fields; on the grid FP32 3 waves
+// 0.98 / 1.00 / 1.00, 4 waves 0.84 / 0.89 / 0.92, FP64 2 waves 0.78 / 0.90 / 0.94.
 template <class T>
-qed_status launch_steps(qed_ctx *ctx, PassArgs &a, int64_t step0, int nsteps) {
+int steps_blocks(const qed_ctx *ctx, int64_t n, int nsteps) {
+    const int waves = (sizeof(T) == 4 ? 3 : 1) + (!SFQ_GRID && nsteps >= 16 ? 1 : 0);
     const int bl = resident_blocks(ctx, k_lepton_steps<T>, LB<T>);
+    return n <= (int64_t)waves * bl * LB<T> ? bl : 0;
+}
+
+template <class T>
+qed_status launch_steps(qed_ctx *ctx, PassArgs &a, int64_t step0, int nsteps, int blocks) {
     qed_status e = timed_launch(ctx, 0, [&] {
-        k_lepton_steps<T><<<bl, LB<T>, 0, ctx->stream>>>(a, (unsigned long long)step0, nsteps);
+        k_lepton_steps<T><<<blocks, LB<T>, 0, ctx->stream>>>(a, (unsigned long long)step0, nsteps);
     });
     if (e != QED_OK) return e;
     SFQ_LAUNCHED(ctx, 1);

@@ -587,15 +587,21 @@ static qed_status enqueue_steps(qed_ctx *ctx, const qed_field_desc *field, doubl
     ctx->async_deferred = 1;
     if (!cascade && ctx->cfg.thin_cap == 0 && ctx->cfg.event_method == QED_METHOD_SUBSTEP && !a.mlp_w16 && nsteps > 1 &&
         ctx->cfg.restore_on_overflow) {
-        // An emission run of several steps: one launch for all of them.  Its
-        // blocks cannot stop at the step in which the photons run out of
-        // room, so it is taken where the state goes back to the batch's start
-        // then; the demand it counts is that of all its steps.
-        a.pass = 0;
-        k_advance_step<<<1, 1, 0, ctx->stream>>>(ctx->ctl, dt, (unsigned long long)nsteps);
-        SFQ_LAUNCHED(ctx, 1);
-        if (field->kind == QED_FIELD_GRID) return pass_grid::launch_steps<T>(ctx, a, step0, nsteps);
-        return pass_analytic::launch_steps<T>(ctx, a, step0, nsteps);
+        // An emission run of several steps: one launch for all of them, where
+        // the leptons (their count does not change) are few enough for that to
+        // pay.  Its blocks cannot stop at the step in which the photons run
+        // out of room, so it is taken where the state goes back to the batch's
+        // start then; the demand it counts is that of all its steps.
+        const bool grid = field->kind == QED_FIELD_GRID;
+        const int64_t n = p->s[0].count + p->s[1].count;
+        const int blocks = grid ? pass_grid::steps_blocks<T>(ctx, n, nsteps) : pass_analytic::steps_blocks<T>(ctx, n, nsteps);
+        if (blocks > 0) {
+            a.pass = 0;
+            k_advance_step<<<1, 1, 0, ctx->stream>>>(ctx->ctl, dt, (unsigned long long)nsteps);
+            SFQ_LAUNCHED(ctx, 1);
+            return grid ? pass_grid::launch_steps<T>(ctx, a, step0, nsteps, blocks)
+                        : pass_analytic::launch_steps<T>(ctx, a, step0, nsteps, blocks);
+        }
     }
     StepGraph *G = ctx->cfg.profile ? nullptr : step_graph_for<T>(ctx, a, p, dt);
     if (!G) return host_steps<T>(ctx, p, a, dt, nsteps);
