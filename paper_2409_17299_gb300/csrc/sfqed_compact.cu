@@ -687,7 +687,9 @@ __global__ void __launch_bounds__(LT, 4) k_tile_dead(const __grid_constant__ Mer
     unsigned removed = 0;
     // FP32 leveling: groups of four entries whose draws are computed together
     constexpr bool SPEC = LEVEL && sizeof(T) == 4;
-    constexpr int G = SPEC ? 4 : 8;           // entries per group of loads
+    // entries per group of loads (with leveling four: eight FP64 weights and
+    // ids and the next eight spill 88 bytes; level_apply at 1e7 weights 346 us against 334)
+    constexpr int G = LEVEL ? 4 : 8;
     static_assert(LROUNDS % G == 0, "groups tile the rounds");
     for (long long tile = blockIdx.x; tile < nbe; tile += gridDim.x) {
         const unsigned long long base = (unsigned long long)tile * LTILE;
