@@ -54,10 +54,10 @@ namespace {
 // a step takes two one-way exchanges and no grid barrier.  A slot is free
 // again when the weights of its step have arrived, since an owner sends them
 // after it has read every slot.
-// What a step costs (GB300, its chain of dependent phases; atomics and a grid
-// barrier before -> now): 10.2 -> 10.3 us with 1 CTA, 10.4 -> 10.9 with 8,
-// 10.9 -> 11.2 with 64, 14.1 -> 12.4 with 152, 19.3 -> 18.1 with two tiles
-// each; FP64 atomics, whose order matters no more, took 13.8 with 64.
+// A call of 32 steps (GB300; a chain of dependent phases; atomics and a grid
+// barrier before -> now): 384 -> 364 us with 1 CTA, 374 -> 378 with 8, 387 ->
+// 399 with 16, 390 -> 379 with 32, 402 -> 386 with 64, 510 -> 424 with 152;
+// FP64 atomics, whose order matters no more, took 490 with 64.
 constexpr int TT = 512;                       // threads
 constexpr int TS = 128;                       // samples per tile = tensor-memory lanes
 constexpr int GSTRIDE = 8580;                 // MLP_NP rounded up to whole float4s
@@ -254,7 +254,8 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train(TrainArgs a) {
     bool ok = true;
 
     // shared-memory writes done: hand the tiles to the tensor cores, one
-    // thread issues `fn`, everyone waits for its completion
+    // thread issues `fn`, every thread waits for its completion by itself
+    // (whether all waits ended is asked once per tile)
     auto run_mma = [&](auto fn) -> bool {
         tc::fence_proxy_smem();
         tc::fence_before_sync();
@@ -264,11 +265,10 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train(TrainArgs a) {
             fn();
             tc::commit(mbar);
         }
-        bool done = tc::mbar_wait(mbar, phase, WAIT_POLLS);
+        const bool done = tc::mbar_wait(mbar, phase, WAIT_POLLS);
         phase ^= 1u;
         tc::fence_after_sync();
-        done = __syncthreads_and(done);
-        if (!done && tid == 0) atomicCAS(a.status, 0, 2);
+        if (!done) atomicCAS(a.status, 0, 2);
         return done;
     };
     auto k_steps = [&](uint32_t d, uint32_t aa, uint32_t alb, uint32_t asb, uint32_t ast, uint32_t bb,
@@ -352,8 +352,7 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train(TrainArgs a) {
                 tc::st16(tl + TD1 + u0, d);
             }
             // Z2 = H1 W2^T -> H2, SiLU'
-            ok = run_mma([&] { k_steps(tmem + TZ, base + SM_H1, 2048, 128, 4096, base + SM_W2, 128, 1024, 256, ID_FWD, 4, false); });
-            if (!ok) break;
+            ok &= run_mma([&] { k_steps(tmem + TZ, base + SM_H1, 2048, 128, 4096, base + SM_W2, 128, 1024, 256, ID_FWD, 4, false); });
             {
                 float z[16], d[16], h[16];
                 tc::ld16(tl + TZ + u0, z);
@@ -362,8 +361,7 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train(TrainArgs a) {
                 tc::st16(tl + TD2 + u0, d);
             }
             // Z3 = H2 W3^T -> H3, the output y (layer 4), D3 = dy W4 SiLU'(Z3)
-            ok = run_mma([&] { k_steps(tmem + TZ, base + SM_H2, 2048, 128, 4096, base + SM_W3, 128, 1024, 256, ID_FWD, 4, false); });
-            if (!ok) break;
+            ok &= run_mma([&] { k_steps(tmem + TZ, base + SM_H2, 2048, 128, 4096, base + SM_W3, 128, 1024, 256, ID_FWD, 4, false); });
             {
                 float z[16], d[16], h[16];
                 tc::ld16(tl + TZ + u0, z);
@@ -396,8 +394,7 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train(TrainArgs a) {
                 store_row(sm + SM_D3, u0, r, v);
             }
             // P3 = D3 W3; D2 = P3 SiLU'(Z2)
-            ok = run_mma([&] { k_steps(tmem + TZ, base + SM_D3, 2048, 128, 4096, base + SM_W3, 1024, 128, 2048, ID_BWD, 4, false); });
-            if (!ok) break;
+            ok &= run_mma([&] { k_steps(tmem + TZ, base + SM_D3, 2048, 128, 4096, base + SM_W3, 1024, 128, 2048, ID_BWD, 4, false); });
             {
                 float pv[16], d[16];
                 tc::ld16(tl + TZ + u0, pv);
@@ -407,8 +404,7 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train(TrainArgs a) {
                 store_row(sm + SM_D2, u0, r, pv);
             }
             // P2 = D2 W2; D1 = P2 SiLU'(Z1)
-            ok = run_mma([&] { k_steps(tmem + TZ, base + SM_D2, 2048, 128, 4096, base + SM_W2, 1024, 128, 2048, ID_BWD, 4, false); });
-            if (!ok) break;
+            ok &= run_mma([&] { k_steps(tmem + TZ, base + SM_D2, 2048, 128, 4096, base + SM_W2, 1024, 128, 2048, ID_BWD, 4, false); });
             {
                 float pv[16], d[16];
                 tc::ld16(tl + TZ + u0, pv);
@@ -419,11 +415,12 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train(TrainArgs a) {
             }
             // weight and bias gradients of the tile, accumulated over the CTA's tiles of the step
             const bool acc = !first;
-            ok = run_mma([&] {
+            ok &= run_mma([&] {
                 k_steps(tmem + TG1, base + SM_D3, 128, 2048, 256, base + SM_H2, 128, 2048, 256, ID_G1, 8, acc);
                 k_steps(tmem + TG2, base + SM_D1, 128, 2048, 256, base + SM_FB, 128, 2048, 256, ID_G2, 8, acc);
             });
             first = false;
+            ok = __syncthreads_and(ok);
         }
         if (!ok) break;
         if (cq == 0) {
@@ -606,12 +603,20 @@ __global__ void k_mlp_commit(const float *out, const int *status, float *P, floa
     W16[i] = __float2bfloat16_rn(out[i]);
 }
 
-// the gradient call's sum over the CTAs' slots, in the order of the CTAs
-__global__ void k_mlp_sum_slots(const uint64_t *slots, int n, float *G) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= MLP_NP) return;
+// The gradient call's sum over the CTAs' slots: 32 parameters per block, eight
+// threads to a parameter that take every eighth slot, then their sums in order.
+__global__ void __launch_bounds__(256) k_mlp_sum_slots(const uint64_t *slots, int n, float *G) {
+    __shared__ float part[8][32];
+    const int p = threadIdx.x & 31, share = threadIdx.x >> 5, i = blockIdx.x * 32 + p;
     float s = 0.f;
-    for (int k = 0; k < n; ++k) s += __uint_as_float((uint32_t)slots[(size_t)k * GSTRIDE + i]);
+    if (i < MLP_NP) {
+#pragma unroll 8
+        for (int k = share; k < n; k += 8) s += __uint_as_float((uint32_t)slots[(size_t)k * GSTRIDE + i]);
+    }
+    part[share][p] = s;
+    __syncthreads();
+    if (share || i >= MLP_NP) return;
+    for (int k = 1; k < 8; ++k) s += part[k][p];
     G[i] = s;
 }
 
@@ -748,7 +753,9 @@ static qed_status train_scratch(qed_ctx *ctx, TrainScratch &t, int grid, int64_t
     t.status = reinterpret_cast<int *>(m + slots + weights + loss);
     t.out = reinterpret_cast<float *>(m + end);
     t.sched = t.out + 3 * GSTRIDE;
-    SFQ_CUDA(cudaMemsetAsync(m, 0, zeroed, ctx->stream));
+    // the gradient call (no steps) reads no tag
+    const size_t from = steps > 0 ? 0 : slots + weights;
+    SFQ_CUDA(cudaMemsetAsync(m + from, 0, zeroed - from, ctx->stream));
     return QED_OK;
 }
 
@@ -793,7 +800,7 @@ qed_status sfq_mlp_grad(qed_ctx *ctx, const float *feat, const float *target, in
     TrainArgs a{P, P + MLP_NP, P + 2 * MLP_NP, t.out, t.slots, t.weights, t.loss, ctx->icdf_em32, feat, target,
                 t.sched, 0ull, (long long)n, 0ll, 0ll, 1.0f / (float)n, WORD_POLLS, t.status};
     k_mlp_train<<<grid, TT, TR_SMEM, st>>>(a);
-    k_mlp_sum_slots<<<(MLP_NP + 255) / 256, 256, 0, st>>>(t.slots, grid, P + 3 * MLP_NP);
+    k_mlp_sum_slots<<<(MLP_NP + 31) / 32, 256, 0, st>>>(t.slots, grid, P + 3 * MLP_NP);
     SFQ_CUDA(cudaGetLastError());
     SFQ_LAUNCHED(ctx, 2);
     SFQ_CUDA(cudaMemcpyAsync(grad_host, P + 3 * MLP_NP, sizeof(float) * MLP_NP, cudaMemcpyDeviceToHost, st));
