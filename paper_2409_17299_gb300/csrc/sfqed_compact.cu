@@ -7,13 +7,11 @@
 // above A (ranks from block scans), so no entry is read after it is written.
 //
 // Leveling: the threshold w* solves sum_i min(1, w_i / w*) = cap (solved on
-// the device, see k_lev_next).  Particle i is kept with probability
+// the device, see k_level).  Particle i is kept with probability
 // min(1, w_i / w*) from Philox(seed; id, step, 0xFFFFFFFF), and kept
 // particles below w* get weight w*.
 #include <math.h>
 #include <string.h>
-
-#include <chrono>
 
 #include "sfqed_device.cuh"
 #include "sfqed_internal.h"
@@ -980,13 +978,10 @@ template <class K> static unsigned tile_grid(const qed_ctx *ctx, K kernel, long 
     return (unsigned)(nb < g ? (nb > 0 ? nb : 1) : g);
 }
 
-// The four passes and the count update.  bound: an upper bound of the device
-// count (the host count, or the capacity when the count is only known on the
-// device); step_from_ctl: the leveling draws take the step index from the
-// control block (a captured step graph).  The work buffers must hold
-// bound / 1024 + 2 block words and bound hole words (sfq_ensure_work).
 // The work buffers of one merge over species of at most bound[s] entries:
-// per tile two words, per entry 16 bits of dead list and half a mover index.
+// a word per tile and two more, and per entry 16 bits of dead list and half a
+// mover index.  bound: an upper bound of the device's count (the host's count,
+// or the capacity where only the device knows the count).
 static int64_t merge_blk_words(const int64_t bound[3]) {
     int64_t n = 0;
     for (int s = 0; s < 3; ++s) n += (bound[s] + LTILE - 1) / LTILE + 2;

@@ -860,7 +860,7 @@ __global__ void __launch_bounds__(LB<T>, (sizeof(T) == 4 && !MLP ? 3 : 2))
 //
 // A launch per step is bound by its latency where the ensemble is small: the
 // step-begin kernel, the tables' staging and the block's last, partly filled
-// rounds took 80 us per step for 16384 electrons in FP64 (49 us here).
+// rounds took 80 us per step for 16384 electrons in FP64 (44 us here).
 template <class T>
 __global__ void __launch_bounds__(LB<T>, 2) k_lepton_steps(const __grid_constant__ PassArgs a, unsigned long long step0,
                                                            int nsteps) {
@@ -1491,20 +1491,6 @@ template <class K> inline int resident_blocks(const qed_ctx *ctx, K kernel, int 
             per_sm = 1;
     }
     return ctx->sm_count * per_sm;
-}
-
-// a group of launches timed as one (compaction, leveling)
-template <class F> inline qed_status timed_block(qed_ctx *ctx, int which, F body) {
-    if (!ctx->cfg.profile) return body();
-    if (ctx->ev_used[which] == qed_ctx::EVN) {
-        qed_status e = sfq_drain_events(ctx);
-        if (e != QED_OK) return e;
-    }
-    const int i = ctx->ev_used[which]++;
-    SFQ_CUDA(cudaEventRecord(ctx->ev[which][i][0], ctx->stream));
-    qed_status e = body();
-    SFQ_CUDA(cudaEventRecord(ctx->ev[which][i][1], ctx->stream));
-    return e;
 }
 
 template <class K> inline int resident_blocks_smem(const qed_ctx *ctx, K kernel, int threads, size_t smem) {
