@@ -51,11 +51,15 @@ EMIT_BYTES = {"fp32": 8 + 7 * 4 + 8 + 4, "fp64": 8 + 7 * 8 + 8 + 4}
 PHOTON_BYTES = {"fp32": 4 + 3 * 4 + 3 * 4 + 8 + 3 * 4, "fp64": 8 + 3 * 8 + 3 * 8 + 8 + 3 * 8}
 
 
+def start_photons(tot):
+    """Photon-steps of the photon pass: the photons present at the step starts
+    (each emission is one photon that flies in the lepton pass)."""
+    return max(0, tot["photon_steps"] - tot["emit_events"])
+
+
 def photon_pass_bytes(prec, tot):
-    """Algorithmic bytes of the photon pass: the photons present at the step
-    starts (each emission is one photon that flies in the lepton pass)."""
-    return (PHOTON_BYTES[prec] * max(0, tot["photon_steps"] - tot["emit_events"])
-            + PAIR_BYTES[prec] * tot["pair_events"])
+    """Algorithmic bytes of the photon pass."""
+    return PHOTON_BYTES[prec] * start_photons(tot) + PAIR_BYTES[prec] * tot["pair_events"]
 
 
 PAIR_BYTES = {"fp32": 4 + 2 * (7 * 4 + 8 + 4 + 8), "fp64": 8 + 2 * (7 * 8 + 8 + 4 + 8)}
@@ -71,15 +75,14 @@ OD_PHOTON_BYTES = {"fp32": PHOTON_BYTES["fp32"] + 8, "fp64": PHOTON_BYTES["fp64"
 # profiles/k_photon_pass_fp32_rotating_e_cascade.md and
 # profiles/k_lepton_pass_fp32_rotating_e_cascade.md.  None when the kernel
 # changed since its capture.
-NCU_PHOTON_BYTES_PER_STEP = {"fp32": None, "fp64": None}
-NCU_LEPTON_BYTES_PER_STEP = {"fp32": None, "fp64": None}
-# FP64 FLOPs (2 DFMA + DADD + DMUL thread instructions) per particle-step of
-# the FP64 step-start passes at the rotating-E cascade's cap (0.3 emissions
-# per lepton-step): the launch's count over the particles it pushed, from one
-# ncu capture.  None: the kernels changed since their capture
-# (profiles/fp64_passes_rotating_e_cascade.md: 481.7 and 206.0 before most
-# particles' steps were decided in FP32)
-NCU_FP64_FLOP_PER_STEP = {"k_lepton_pass": None, "k_photon_pass": None}
+NCU_PHOTON_BYTES_PER_STEP = {"fp32": 47.7, "fp64": None}
+NCU_LEPTON_BYTES_PER_STEP = {"fp32": 77.9, "fp64": None}
+# FP64 FLOPs (2 DFMA + DADD + DMUL thread instructions) of the FP64 passes at
+# the rotating-E cascade's cap, from one ncu capture
+# (profiles/fp64_passes_rotating_e_cascade.md): the lepton pass per lepton-step
+# (the flights of the photons it emits included), the photon pass per photon
+# present at the step start (most steps are decided in FP32)
+NCU_FP64_FLOP_PER_STEP = {"k_lepton_pass": 328.6, "k_photon_pass": 37.8}
 # algorithmic FLOPs per training sample of the 2-64-64-64-1 network: forward
 # 2 x (2*64 + 64*64 + 64*64 + 64) multiply-adds, backward the two 64x64 input
 # gradients, the two 64x64 weight gradients, W1's and W4's gradients
@@ -851,7 +854,7 @@ def main():
                           "bytes_per_photon_step": PHOTON_BYTES[prec], "bytes_per_pair": PAIR_BYTES[prec],
                           "units": "photon-steps %d, pairs %d" % (tot["photon_steps"], tot["pair_events"]),
                           "algorithmic_bytes_per_step": ph_bytes / steps,
-                          "traffic": (NCU_PHOTON_BYTES_PER_STEP[prec] * tot["photon_steps"] / steps
+                          "traffic": (NCU_PHOTON_BYTES_PER_STEP[prec] * start_photons(tot) / steps
                                       if NCU_PHOTON_BYTES_PER_STEP[prec] and w.push_photons else None)},
     }
     for k in kernels.values():
@@ -923,11 +926,11 @@ def main():
 # Instruction issue peak of one GB300: 152 SMs x 4 schedulers x 2.07 GHz,
 # one warp instruction per scheduler per clock.
 ISSUE_PEAK_WARP_INSTR = 152 * 4 * 2.07e9
-# Warp instructions per lepton-step of the step-fused batch kernel (128
-# threads) from one ncu capture of the current kernel: the 10-step call's
-# count over its 4.02e7 lepton-steps
+# Warp instructions per lepton-step of the step-fused batch kernel (256
+# threads, 32 warps per SM) from one ncu capture of the current kernel: the
+# 10-step call's count over its 4.02e7 lepton-steps
 # (profiles/k_emission_fused_batched_uniform_b.md); None when not captured
-NCU_FUSED_WARP_INSTR_PER_STEP = {"fp32": 40.8, "fp64": None}
+NCU_FUSED_WARP_INSTR_PER_STEP = {"fp32": 40.5, "fp64": None}
 
 
 # The paper's test problem (Sec. 5.1-5.2): growth rate of the cascade in its
@@ -1072,7 +1075,7 @@ def fp64_roofline(tot, hbm_peak):
                       "summed CUDA-event time of the launches", "kernels": {}}
     for k, ms, units, nbytes in (("k_lepton_pass", tot["kernel_ms"][0], tot["lepton_steps"],
                                   LEPTON_BYTES["fp64"] * tot["lepton_steps"] + EMIT_BYTES["fp64"] * tot["emit_events"]),
-                                 ("k_photon_pass", tot["kernel_ms"][1], tot["photon_steps"],
+                                 ("k_photon_pass", tot["kernel_ms"][1], start_photons(tot),
                                   photon_pass_bytes("fp64", tot))):
         if ms <= 0:
             continue

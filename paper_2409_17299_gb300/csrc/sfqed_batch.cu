@@ -297,7 +297,7 @@ __device__ __forceinline__ void fused_round(const FusedCtx &c, FusedStack<T, NT>
     __syncthreads();
 }
 
-// DENSE (FP32): 32 warps per SM at every block shape (64 registers, 32 bytes
+// DENSE (FP32, blocks of 256 and 512): 32 warps per SM (64 registers, 32 bytes
 // spilled), for calls whose tiles fill the chip.  The rounds' barriers and
 // dependent instructions leave the issue slots 40% idle at 16 warps (86
 // registers, what the compiler takes by itself).  64 bunches of 250 to 250000
@@ -305,9 +305,12 @@ __device__ __forceinline__ void fused_round(const FusedCtx &c, FusedStack<T, NT>
 // with 32, 6.65 with 40 (48 registers); 32 warps in blocks of 128: 6.10, of
 // 512: 6.43.  A call of which every block of the roomy kernel gets at most
 // one tile gains nothing from more warps and keeps that kernel (3 bunches of
-// 20 to 20000 leptons, 10 steps: 0.213 ms, dense 0.229).
+// 20 to 20000 leptons, 10 steps: 0.213 ms, dense 0.229).  Blocks of 128 hold 28
+// warps (68 registers) as they are; with 32 they were 1 to 4% faster at chi
+// 0.05 and 1 to 6% slower at chi 10 (16 x 16384 leptons, 30 steps: 0.887 and
+// 0.942 ms), so they stay.
 template <class T, int NT, bool DENSE> constexpr int fused_min_blocks() {
-    return sizeof(T) == 4 ? (DENSE ? 1024 / NT : NT == 128 ? 7 : 1) : 1;
+    return sizeof(T) == 4 ? (NT == 128 ? 7 : DENSE ? 1024 / NT : 1) : 1;
 }
 
 template <class T, int NT, bool DENSE>
@@ -401,7 +404,7 @@ template <class T, int NT, bool DENSE> static int fused_blocks(const qed_ctx *ct
 
 template <class T, int NT> static void launch_shape(const qed_ctx *ctx, const BatchArgs &b, cudaStream_t st) {
     const int blocks = fused_blocks<T, NT, false>(ctx);
-    if constexpr (sizeof(T) == 4) {
+    if constexpr (sizeof(T) == 4 && NT >= 256) {
         if (b.n_tiles > (unsigned long long)blocks) {
             k_emission_fused<T, NT, true><<<fused_blocks<T, NT, true>(ctx), NT, 0, st>>>(b);
             return;
